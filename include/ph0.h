@@ -96,7 +96,8 @@ typedef struct {
 typedef struct {
     int32_t status;          /* ph0_status of the device-side work            */
     int32_t sort_passes;     /* radix passes of the key range's plan (4 for
-                              * the packed sort of sort_form 1; else the     *
+                              * the packed sort of sort_form 1, 0 without a  *
+                              * sort, sort_form 3; else the                  *
                               * whole path runs those from slot 2 on)         */
     int32_t key_bits;        /* varying key bits sorted                       */
     int32_t windows;         /* reduction windows processed                   */
@@ -117,7 +118,10 @@ typedef struct {
     int32_t sort_form;       /* which sort gave the whole path's order: 0 the
                                 short sort of (key, value) records, 1 the packed
                                 sort of 64-bit words, 2 the complete sort run
-                                after a fix-up met a group it cannot order    */
+                                after a fix-up met a group it cannot order, 3
+                                none: positions and indices counted (clouds of
+                                up to 2896 points; tuning that asks for a form
+                                of the sort runs that form)                   */
     int32_t _pad;
 } ph0_stats;
 

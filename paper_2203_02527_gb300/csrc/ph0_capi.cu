@@ -72,6 +72,10 @@ cudaError_t launch_dedupe(const uint64_t *keys0, const uint64_t *keys1, const He
 cudaError_t launch_backward(const float *pts, int64_t n, int32_t d, int64_t ld, const ph0_bar *bars,
                             int64_t nb, const double *dl, float *grad, double *acc, cudaStream_t s);
 
+bool direct_applies(const Layout &L, int32_t d);
+cudaError_t launch_direct(void *ws, const Layout &L, const float *pts, int64_t n, int32_t d, int64_t ld,
+                          ph0_bar *bars, ph0_inf_bar *inf, cudaStream_t s, cudaEvent_t after_dist = nullptr,
+                          cudaEvent_t after_tree = nullptr);
 cudaError_t launch_reduce(const ReduceArgs &A, cudaStream_t s);
 cudaError_t launch_inf(Header *h, int64_t n, ph0_inf_bar *inf, cudaStream_t s);
 cudaError_t run_h1(void *ws, const H1Layout &H, int64_t n, const uint64_t *ek0, const uint64_t *ek1,
@@ -113,6 +117,7 @@ struct Tune {
     bool wide = false;  // edge-index records (always above kMaxN points)
     bool split = false;  // the whole path's sort as two merged halves (always above kSplitEdges edges)
     bool packed = false;  // the whole path's packed sort (k_sortp.cu)
+    bool sortless = true;  // the whole path may leave the sort out (k_direct.cu): no form asked for
     explicit Tune(const ph0_tuning *t, int64_t n = 0, int32_t d = 0) {
         const int64_t m = n_edges(n);
         wide = n > kMaxN;
@@ -121,6 +126,7 @@ struct Tune {
         if (!t) return;
         if (t->wide_ids == 1) wide = true;
         if (t->split_sort == 1) split = true;
+        sortless = t->wide_ids != 1 && t->split_sort != 1 && t->packed_sort != 0 && t->packed_sort != 1;
         if (t->packed_sort == 0) packed = false;
         if (t->packed_sort == 1) packed = m >= 1 && n <= kPackMaxN;
         if (split || wide) packed = false;  // its words take (u, v), not an edge index
@@ -411,6 +417,8 @@ int barcodes_whole(const float *pts_dev, int64_t n, int32_t d, int64_t ld, ph0_b
     uint64_t *k0 = at<uint64_t>(ws, L.key[0]), *k1 = at<uint64_t>(ws, L.key[1]);
     uint32_t *v0 = at<uint32_t>(ws, L.val[0]), *v1 = at<uint32_t>(ws, L.val[1]);
     uint32_t *cpref = at<uint32_t>(ws, L.cpref);
+    if (t.sortless && direct_applies(L, d))
+        return cuda_status(launch_direct(ws, L, pts_dev, n, d, ld, bars_dev, inf_dev, s));
     cudaError_t e = begin_call(ws, L, s, t.top_bits);
     if (e == cudaSuccess)
         e = launch_dist(pts_dev, n, d, ld, k0, v0, h, s, t.split16, t.tile, nullptr, t.wide, t.packed);
@@ -657,7 +665,23 @@ int ph0_barcodes_profiled(const float *pts_dev, int64_t n, int32_t d, int64_t ld
     // passes, then the fix-up, the short sort that runs only when the keys do
     // not pack, and the gated fallback)
     const Tune t(tuning, n, d);
+    const bool direct = t.sortless && direct_applies(L, d);
     e = cudaEventRecord(ev[0], s);
+    if (direct) {  // distances, tree, counts and bars: no sort, the pivots with the tree
+        if (e == cudaSuccess)
+            e = launch_direct(ws, L, pts_dev, n, d, ld, bars_dev, inf_dev, s, ev[1], ev[4 + kMaxPasses]);
+        if (e == cudaSuccess) e = cudaEventRecord(ev[5 + kMaxPasses], s);
+        if (e == cudaSuccess) e = cudaEventSynchronize(ev[5 + kMaxPasses]);
+        if (e == cudaSuccess) {
+            std::memset(prof, 0, sizeof(*prof));
+            cudaEventElapsedTime(&prof->total_ms, ev[0], ev[5 + kMaxPasses]);
+            cudaEventElapsedTime(&prof->dist_ms, ev[0], ev[1]);
+            cudaEventElapsedTime(&prof->reduce_ms, ev[1], ev[4 + kMaxPasses]);
+            cudaEventElapsedTime(&prof->emit_ms, ev[4 + kMaxPasses], ev[5 + kMaxPasses]);
+        }
+        for (int i = 0; i < kEv; ++i) cudaEventDestroy(ev[i]);
+        return cuda_status(e);
+    }
     if (e == cudaSuccess) e = begin_call(ws, L, s, t.top_bits);
     if (e == cudaSuccess)
         e = launch_dist(pts_dev, n, d, ld, k0, v0, h, s, t.split16, t.tile, nullptr, t.wide, t.packed);
@@ -727,7 +751,7 @@ int ph0_finish(const void *ws, void *stream, ph0_stats *stats) {
         stats->inf_vertex = hh.inf_vertex;
         stats->claim_rounds_max = int32_t(hh.claim_rounds_max);
         stats->claim_attempts = int64_t(hh.claim_attempts);
-        stats->sort_form = hh.fixup_fallback ? 2 : (hh.packed ? 1 : 0);
+        stats->sort_form = hh.direct ? 3 : hh.fixup_fallback ? 2 : (hh.packed ? 1 : 0);
         stats->_pad = 0;
     }
     return hh.status;
@@ -968,11 +992,16 @@ extern "C" int ph0_barcodes_noalloc(const float *pts_dev, int64_t n, int32_t d, 
     // header and the first look-back buffer, and every later stage clears or
     // overwrites what it reads before reading it
     const Tune t(nullptr);
-    cudaError_t e = begin_call(ws, L, s);
-    if (e == cudaSuccess) e = launch_dist(pts_dev, n, d, ld, k0, v0, h, s);
-    if (e == cudaSuccess) e = sort_whole(ws, L, pts_dev, n, d, ld, t, s);
-    if (e == cudaSuccess) e = launch_dedupe_scan(cpref, L.m, at<uint64_t>(ws, L.dlook), h, s);
-    if (e == cudaSuccess) e = reduce_and_emit(ws, L, n, v0, v1, k0, k1, h, nullptr, cpref, bars_dev, inf_dev, s);
+    cudaError_t e = cudaSuccess;
+    if (direct_applies(L, d)) {
+        e = launch_direct(ws, L, pts_dev, n, d, ld, bars_dev, inf_dev, s);
+    } else {
+        e = begin_call(ws, L, s);
+        if (e == cudaSuccess) e = launch_dist(pts_dev, n, d, ld, k0, v0, h, s);
+        if (e == cudaSuccess) e = sort_whole(ws, L, pts_dev, n, d, ld, t, s);
+        if (e == cudaSuccess) e = launch_dedupe_scan(cpref, L.m, at<uint64_t>(ws, L.dlook), h, s);
+        if (e == cudaSuccess) e = reduce_and_emit(ws, L, n, v0, v1, k0, k1, h, nullptr, cpref, bars_dev, inf_dev, s);
+    }
     // the status word is read on the caller's stream (a plain copy would go
     // through the legacy default stream and wait for other blocking streams)
     int32_t status = PH0_OK;

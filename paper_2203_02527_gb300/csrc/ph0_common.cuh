@@ -82,6 +82,12 @@ __host__ __device__ __forceinline__ uint32_t pack_edge(uint64_t w, uint32_t n) {
     return u * (2 * n - u - 1) / 2 + (v - u - 1);  // u(2n-u-1) < 2^31 at n <= 32768
 }
 
+// The whole path without a sort (k_direct.cu): up to kDirectMaxN points
+// (fewer than 2^22 edges); a row of the distance matrix has at most
+// kDirectChunks blocks of columns.
+constexpr int64_t kDirectMaxN = 2896;
+constexpr int kDirectChunks = 32;
+
 // Bounded device-side waits: about a second at most, then the kernel records
 // PH0_ETIMEOUT in the status word and returns cleanly.
 constexpr uint32_t kSpinLimit = 1u << 24;
@@ -152,6 +158,15 @@ struct Header {
     unsigned long long claim_attempts;  // atomic claims of the reduction (grid and tail rounds)
     uint32_t claim_rounds_max;   // most claim rounds in one window
     int32_t classic;             // a packed-sort call whose keys do not pack: the short sort runs
+    // the sortless form (k_direct.cu): set when it ran; edges whose distance
+    // an earlier one has, and the distances that occur more than once;
+    // finished CTAs of its count; complement of the smallest key (the header
+    // starts at zero)
+    int32_t direct;
+    uint32_t direct_dups;
+    uint32_t direct_repeats;
+    uint32_t direct_done;
+    uint64_t direct_nkmin;
     // class partition of the early path (radix slot kClassSlot): the key
     // bins of its histogram and the classes' bin ranges [bound[c], bound[c+1])
     uint64_t part_kmin;
