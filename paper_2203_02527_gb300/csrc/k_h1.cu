@@ -90,6 +90,7 @@ struct H1Counters {
     unsigned long long max_len;     // longest column met
     unsigned long long pool_used;   // keys held by the reduced columns
     unsigned long long nodes;       // pivots claimed by reduced columns
+    unsigned long long list_used;   // edges in the reduced columns' lists (bit-set form)
 };
 
 // -------------------------------------------------------------- step 1 ---
@@ -288,15 +289,17 @@ __global__ void k_h1_zlist(const uint64_t *scan_in, const uint64_t *zpref, int64
 // Kruskal over the listed edges in order (one thread; union-find with path
 // halving in shared memory): an edge that joins two trees is a spanning-
 // forest edge (tfirst = -2: its column is cleared), the others are positive
-// and go to rlist in order.  A full simplex's forest has n-1 edges.
+// and go to rlist in order.  A full simplex's forest has n-1 edges.  All
+// threads stage the listed edges in shared memory (the one thread alone would
+// wait for two dependent loads per edge).
+constexpr int kH1ForestChunk = 2048;
 __global__ void __launch_bounds__(256) k_h1_forest(const uint32_t *vals0, const uint32_t *vals1, const Header *esort,
                                                    const uint32_t *zlist, const uint64_t *zpref, int64_t m, int64_t n,
                                                    int32_t *tfirst, uint32_t *rlist, H1Counters *c, Header *h) {
     __shared__ uint16_t s_par[kH1MaxN];
+    __shared__ uint32_t s_p[kH1ForestChunk], s_uv[kH1ForestChunk];
     const uint32_t *vals = (make_plan(esort).passes & 1) ? vals1 : vals0;
     for (int i = threadIdx.x; i < n; i += blockDim.x) s_par[i] = uint16_t(i);
-    __syncthreads();
-    if (threadIdx.x != 0) return;
     auto find = [&](uint32_t x) {
         while (s_par[x] != x) {
             s_par[x] = s_par[s_par[x]];
@@ -306,19 +309,31 @@ __global__ void __launch_bounds__(256) k_h1_forest(const uint32_t *vals0, const 
     };
     const uint64_t Z = zpref[m];
     uint64_t forest = 0, k = 0;
-    for (uint64_t z = 0; z < Z; ++z) {
-        const uint32_t p = zlist[z];
-        uint32_t a, b;
-        if (!h1_uv(vals, p, n, a, b)) continue;
-        const uint32_t ra = find(a), rb = find(b);
-        if (ra != rb) {
-            s_par[ra] = uint16_t(rb);
-            tfirst[p] = -2;
-            ++forest;
-        } else {
-            rlist[k++] = p;
+    for (uint64_t z0 = 0; z0 < Z; z0 += kH1ForestChunk) {
+        const int len = Z - z0 < uint64_t(kH1ForestChunk) ? int(Z - z0) : kH1ForestChunk;
+        __syncthreads();
+        for (int i = threadIdx.x; i < len; i += blockDim.x) {
+            const uint32_t p = zlist[z0 + i];
+            uint32_t a, b;
+            s_p[i] = p;
+            s_uv[i] = h1_uv(vals, p, n, a, b) ? (a << 16) | b : kH1NoPos;
+        }
+        __syncthreads();
+        if (threadIdx.x != 0) continue;
+        for (int i = 0; i < len; ++i) {
+            const uint32_t uv = s_uv[i], p = s_p[i];
+            if (uv == kH1NoPos) continue;
+            const uint32_t ra = find(uv >> 16), rb = find(uv & 0xffffu);
+            if (ra != rb) {
+                s_par[ra] = uint16_t(rb);
+                tfirst[p] = -2;
+                ++forest;
+            } else {
+                rlist[k++] = p;
+            }
         }
     }
+    if (threadIdx.x != 0) return;
     c->zero = Z;
     c->forest = forest;
     c->reduced = k;
@@ -649,6 +664,332 @@ __global__ void __launch_bounds__(kH1Threads) k_h1_reduce(H1Reduce R) {
     }
 }
 
+// The listed columns as bit sets, several at a time (up to kH1BitsMaxN points).
+//
+// A triangle of diameter position dp and opposite vertex w is bit dp n + w: bit
+// order is triangle order.  A column under reduction is such a set in the
+// workspace, one per CTA, together with the set V of the edges whose
+// coboundaries add up to it (bits in shared memory).  Adding a column is
+// flipping the n-2 bits of each of its edges' coboundaries, nothing sorted or
+// merged; pivots only move up, so the next one is found by looking forward
+// over the blocks of kH1BlockBits bits that were touched (a bit per block in
+// shared memory; a block is zeroed when first touched, so a set is never
+// cleared as a whole).  A reduced column is kept as its list V.
+//
+// The gridDim.x columns of a batch run at the same time, each adding apparent
+// owners' and earlier batches' columns until neither owns its pivot; then, at
+// a grid barrier, of the columns with the same pivot the earliest in
+// processing order keeps it and the others add it and go on.  Only
+// columns from the left are ever added, so the pairs are those of the
+// left-to-right reduction (a matrix has one set of pairs).  A round ends every
+// chain that met another column, and a batch ends when all pivots differ.
+//
+// Bound by the latency of an addition's steps (pivot block, owner, rows of P,
+// flips), about 2 us each.  One CTA merging sorted runs of keys took 28.1 ms
+// of the 29.0 ms at 700 uniform points in the plane (173 columns, 1,024
+// additions).
+struct H1Bits {
+    int n;
+    int64_t m;
+    const uint32_t *vals0, *vals1;
+    const Header *esort;
+    const uint32_t *P;
+    const int32_t *tfirst;
+    const uint32_t *rlist;
+    int32_t *head;
+    uint32_t *claims;
+    uint64_t *node_key;
+    uint32_t *node_pos;
+    int32_t *node_next;
+    uint32_t *node_within;
+    uint32_t *own_node;
+    uint64_t *own_off;
+    uint32_t *own_len;
+    uint32_t *bits;            // [ctas][bit_words]
+    size_t bit_words;
+    uint32_t *pub;             // [ctas][m + 1] edges of the columns of this batch
+    uint32_t *pub_piv, *pub_len;  // [2][ctas] their pivots by the round's parity, [ctas] lengths
+    uint32_t *pool;            // edges of the reduced columns
+    int64_t pool_cap;
+    H1Counters *c;
+    Header *h;
+    uint32_t spin_limit;
+};
+
+constexpr int kH1Stage = 128;   // edges of an added column staged at a time
+constexpr uint32_t kH1NoPivot = 0xffffffffu;  // above every bit: m n < 2^30
+constexpr uint32_t kH1Busy = 0xfffffffeu;     // published by a column that is not done with a round
+constexpr uint32_t kH1RoundFlips = 1u << 24;  // flips before it goes on in the next: bounds the others' wait
+
+__global__ void __launch_bounds__(kH1Threads, 1) k_h1_columns(const H1Bits R) {
+    extern __shared__ uint32_t s_dyn[];
+    __shared__ uint64_t s_warp[kH1Threads / 32 + 1];
+    __shared__ uint32_t s_e[kH1Stage], s_ab[kH1Stage], s_pivs[kH1BitsCtas];
+    __shared__ int s_first[kH1BitsCtas];
+    __shared__ uint32_t s_piv, s_op, s_edge, s_uv, s_len;
+    __shared__ uint64_t s_off;
+    __shared__ int s_ok;
+    enum : uint32_t { kNone, kApparent, kReduced, kError };
+    const uint32_t n = uint32_t(R.n), vwords = uint32_t((R.m + 31) / 32);
+    const uint32_t blocks = uint32_t(R.bit_words * 32 / kH1BlockBits), twords = (blocks + 31) / 32;
+    uint32_t *s_v = s_dyn, *s_t = s_dyn + vwords;  // edges of V, touched blocks
+    const uint32_t *vals = (make_plan(R.esort).passes & 1) ? R.vals1 : R.vals0;
+    const int tid = threadIdx.x, T = blockDim.x, lane = tid & 31, warp = tid >> 5, G = gridDim.x, me = blockIdx.x;
+    const int64_t K = int64_t(R.c->reduced);
+    uint32_t *bits = R.bits + size_t(me) * R.bit_words, *mine = R.pub + size_t(me) * size_t(R.m + 1);
+    unsigned long long adds = 0;
+    int par = 0;
+
+    // the bit of {a, b, w}, edge {a, b} at position e; kH1NoPivot for w = a, b
+    auto bit_of = [&](uint32_t e, uint32_t a, uint32_t b, uint32_t w) {
+        if (w == a || w == b) return kH1NoPivot;
+        const uint32_t x = __ldg(R.P + size_t(a) * n + w), y = __ldg(R.P + size_t(b) * n + w);
+        if (e > x && e > y) return e * n + w;
+        return x > y ? x * n + b : y * n + a;
+    };
+    auto touch = [&](uint32_t bit) {  // zero the bit's block when it is the first of it
+        if (bit == kH1NoPivot) return;
+        const uint32_t blk = bit / kH1BlockBits, mask = 1u << (blk & 31);
+        if (s_t[blk >> 5] & mask) return;  // stale reads only repeat the atomic
+        if (atomicOr(s_t + (blk >> 5), mask) & mask) return;
+        uint4 *z = reinterpret_cast<uint4 *>(bits + size_t(blk) * (kH1BlockBits / 32));
+#pragma unroll
+        for (int q = 0; q < kH1BlockBits / 128; ++q) z[q] = make_uint4(0, 0, 0, 0);
+    };
+    auto flip = [&](uint32_t bit) {
+        if (bit != kH1NoPivot) atomicXor(bits + (bit >> 5), 1u << (bit & 31));
+    };
+    // add the coboundary of one edge (all threads; ends with a barrier)
+    auto add_edge = [&](uint32_t e, uint32_t uv) {
+        const uint32_t a = uv >> 16, b = uv & 0xffffu;
+        const uint32_t bit = uint32_t(tid) < n ? bit_of(e, a, b, uint32_t(tid)) : kH1NoPivot;
+        if (tid == 0) s_v[e >> 5] ^= 1u << (e & 31);
+        touch(bit);
+        __syncthreads();
+        flip(bit);
+        __syncthreads();
+    };
+    static_assert(kH1Threads >= kH1BitsMaxN, "a thread per third vertex");
+    // add the edges of a list written before a grid barrier
+    auto add_list = [&](const uint32_t *list, uint32_t len) {
+        for (uint32_t i0 = 0; i0 < len; i0 += kH1Stage) {
+            const uint32_t cnt = len - i0 < uint32_t(kH1Stage) ? len - i0 : uint32_t(kH1Stage);
+            if (uint32_t(tid) < cnt) {
+                const uint32_t e = __ldcg(list + i0 + tid);
+                s_e[tid] = e;
+                s_ab[tid] = __ldg(vals + e);
+                atomicXor(s_v + (e >> 5), 1u << (e & 31));
+            }
+            __syncthreads();
+            for (uint32_t i = warp; i < cnt; i += kH1Threads / 32) {
+                const uint32_t e = s_e[i], a = s_ab[i] >> 16, b = s_ab[i] & 0xffffu;
+                for (uint32_t w = lane; w < n; w += 32) touch(bit_of(e, a, b, w));
+            }
+            __syncthreads();
+            for (uint32_t i = warp; i < cnt; i += kH1Threads / 32) {
+                const uint32_t e = s_e[i], a = s_ab[i] >> 16, b = s_ab[i] & 0xffffu;
+                for (uint32_t w = lane; w < n; w += 32) flip(bit_of(e, a, b, w));
+            }
+            __syncthreads();
+        }
+    };
+    // the first bit at or after `from` (one warp): four touched blocks at a time
+    auto next_bit = [&](uint32_t from) -> uint32_t {
+        uint32_t word = (from / kH1BlockBits) >> 5, keep = ~0u << ((from / kH1BlockBits) & 31);
+        for (uint32_t w0 = word; w0 < twords; w0 += 32) {
+            uint32_t t = w0 + lane < twords ? s_t[w0 + lane] : 0u;
+            if (w0 == word && lane == 0) t &= keep;
+            for (;;) {
+                uint32_t blk = kH1NoPivot;  // of this lane's group of eight
+#pragma unroll
+                for (int g = 0; g < 4; ++g) {
+                    const unsigned some = __ballot_sync(0xffffffffu, t != 0);
+                    if (!some) break;
+                    const int src = __ffs(some) - 1;
+                    const uint32_t tw = __shfl_sync(0xffffffffu, t, src);
+                    if (lane == src) t &= t - 1;
+                    if (lane >> 3 == g) blk = (w0 + src) * 32 + __ffs(tw) - 1;
+                }
+                if (__shfl_sync(0xffffffffu, blk, 0) == kH1NoPivot) break;
+                uint32_t found = kH1NoPivot;
+                if (blk != kH1NoPivot) {
+                    const uint4 x = __ldcg(reinterpret_cast<const uint4 *>(
+                        bits + size_t(blk) * (kH1BlockBits / 32) + (lane & 7) * 4));
+                    const uint32_t base = blk * kH1BlockBits + (lane & 7) * 128;
+                    const uint32_t xs[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+                    for (int q = 3; q >= 0; --q) {
+                        uint32_t y = xs[q];
+                        const uint32_t b0 = base + q * 32;
+                        if (b0 + 31 < from) y = 0;
+                        else if (b0 < from) y &= ~0u << (from - b0);
+                        if (y) found = b0 + __ffs(y) - 1;
+                    }
+                }
+                found = __reduce_min_sync(0xffffffffu, found);
+                if (found != kH1NoPivot) return found;
+            }
+        }
+        return kH1NoPivot;
+    };
+    auto reset = [&]() {
+        for (uint32_t i = tid; i < vwords; i += T) s_v[i] = 0;
+        for (uint32_t i = tid; i < twords; i += T) s_t[i] = 0;
+        __syncthreads();
+    };
+
+    for (int64_t base = 0; base < K; base += G) {
+        const int64_t col = base + me;  // in processing order: from the latest edge down
+        bool active = col < K, running = active;
+        uint32_t p = 0, piv = kH1NoPivot, len = 0;
+        reset();
+        if (active) {
+            p = R.rlist[K - 1 - col];
+            uint32_t a = 0, b = 0;
+            h1_uv(vals, p, n, a, b);  // listed from checked records
+            add_edge(p, (a << 16) | b);
+            piv = 0;
+        }
+        for (;;) {
+            bool busy = false;
+            if (running) {
+                uint32_t work = 0;
+                // add apparent owners and earlier batches' columns
+                for (;;) {
+                    if (warp == 0) {
+                        const uint32_t x = next_bit(piv);
+                        uint32_t op = kNone, dp = 0, uv = 0, list_len = 0;
+                        uint64_t off = 0;
+                        if (x == kH1NoPivot) {
+                            op = kError;  // every positive column keeps a pivot: a bug if not
+                        } else {
+                            dp = x / n;
+                            const uint32_t w = x - dp * n;
+                            const int32_t f = __ldg(R.tfirst + dp);
+                            int32_t q = __ldcg(R.head + dp);
+                            uv = __ldg(vals + dp);
+                            if (f == int32_t(w)) {
+                                op = kApparent;
+                            } else if (q >= 0) {
+                                const uint64_t key = h1_key(dp, uv >> 16, uv & 0xffffu, w);
+                                for (; q >= 0; q = __ldcg(R.node_next + q))
+                                    if (__ldcg(R.node_key + q) == key) {
+                                        const uint32_t o = __ldcg(R.node_pos + q);
+                                        op = kReduced;
+                                        off = __ldcg(R.own_off + o);
+                                        list_len = __ldcg(R.own_len + o);
+                                        break;
+                                    }
+                            }
+                        }
+                        if (lane == 0) {
+                            s_piv = x;
+                            s_op = op;
+                            s_edge = dp;
+                            s_uv = uv;
+                            s_off = off;
+                            s_len = list_len;
+                        }
+                    }
+                    __syncthreads();
+                    piv = s_piv;
+                    const uint32_t op = s_op, e = s_edge, uv = s_uv, llen = s_len;
+                    const uint64_t off = s_off;
+                    __syncthreads();
+                    if (op == kNone) break;
+                    if (op == kError || adds >= kH1MaxAdditions) {
+                        if (tid == 0) set_status(R.h, op == kError ? PH0_EINTERNAL : PH0_ETOOBIG);
+                        active = false;
+                        piv = kH1NoPivot;
+                        break;
+                    }
+                    ++adds;
+                    if (op == kApparent) add_edge(e, uv);
+                    else add_list(R.pool + off, llen);
+                    work += (op == kApparent ? 1u : llen) * n;  // a list: below 2^30
+                    if ((busy = work >= kH1RoundFlips)) break;
+                }
+                // publish the pivot and the column's edges
+                uint64_t tot = 0;
+                if (active && !busy) {
+                    const uint32_t per = (vwords + T - 1) / T, w0 = tid * per;
+                    uint32_t cnt = 0;
+                    for (uint32_t w = w0; w < w0 + per && w < vwords; ++w) cnt += __popc(s_v[w]);
+                    uint32_t at = uint32_t(h1_block_scan(cnt, s_warp, tot));
+                    for (uint32_t w = w0; w < w0 + per && w < vwords; ++w)
+                        for (uint32_t x = s_v[w]; x; x &= x - 1) mine[at++] = w * 32 + __ffs(x) - 1;
+                }
+                len = uint32_t(tot);
+                if (tid == 0) R.pub_len[me] = len;
+            }
+            if (tid == 0) R.pub_piv[par * G + me] = busy ? kH1Busy : active ? piv : kH1NoPivot;
+            if (!grid_barrier(R.h, &s_ok, R.spin_limit)) return;
+            // of the columns with one pivot the first keeps it
+            if (tid < G) s_pivs[tid] = __ldcg(R.pub_piv + par * G + tid);
+            if (tid < G) s_first[tid] = tid;
+            __syncthreads();
+            bool again = false;
+            for (int t = tid >> 3; t < G; t += kH1Threads / 8) {
+                const uint32_t x = s_pivs[t];
+                if (x == kH1Busy) again = true;
+                if (x >= kH1Busy) continue;
+                for (int i = tid & 7; i < t; i += 8)
+                    if (s_pivs[i] == x) {
+                        atomicMin(s_first + t, i);
+                        again = true;
+                        break;
+                    }
+            }
+            again = __syncthreads_or(again);
+            par ^= 1;
+            if (!again) break;  // the same in every CTA
+            const int j = s_first[me];
+            running = busy;
+            if (j == me) continue;
+            running = true;
+            ++adds;
+            add_list(R.pub + size_t(j) * size_t(R.m + 1), __ldcg(R.pub_len + j));
+        }
+        if (active) {
+            // claim the pivot: a node in the list of its diameter position
+            const uint32_t dp = piv / n, w = piv - dp * n, uv = __ldg(vals + dp);
+            const uint32_t a2 = uv >> 16, b2 = uv & 0xffffu;
+            // its rank among the triangles of diameter dp: third vertices before w
+            const uint32_t *Pa = R.P + size_t(a2) * n, *Pb = R.P + size_t(b2) * n;
+            uint64_t within, keys;
+            h1_block_scan(uint32_t(tid) < w && Pa[tid] < dp && Pb[tid] < dp ? 1u : 0u, s_warp, within);
+            // the reduced column's length
+            uint64_t cnt = 0;
+            for (uint32_t b = warp; b < blocks; b += kH1Threads / 32)
+                if ((s_t[b >> 5] >> (b & 31)) & 1u) cnt += __popc(__ldcg(bits + size_t(b) * (kH1BlockBits / 32) + lane));
+            h1_block_scan(cnt, s_warp, keys);
+            if (tid == 0) {
+                const uint64_t off = atomicAdd(&R.c->list_used, (unsigned long long)len);
+                const bool fits = off + len <= uint64_t(R.pool_cap);
+                if (!fits) set_status(R.h, PH0_ETOOBIG);
+                s_len = fits ? len : 0u;
+                s_off = off;
+                const int32_t q = int32_t(col);
+                R.node_key[q] = h1_key(dp, a2, b2, w);
+                R.node_pos[q] = p;
+                R.node_within[q] = uint32_t(within);
+                R.own_node[p] = uint32_t(q);
+                R.own_off[p] = off;
+                R.own_len[p] = s_len;
+                R.node_next[q] = atomicExch(R.head + dp, q);
+                atomicAdd(R.claims + dp, 1u);
+                atomicAdd(&R.c->nodes, 1ull);
+                atomicAdd(&R.c->pool_used, (unsigned long long)keys);
+                atomicMax(&R.c->max_len, (unsigned long long)keys);
+            }
+            __syncthreads();
+            for (uint32_t i = tid; i < s_len; i += T) R.pool[s_off + i] = __ldcg(mine + i);
+        }
+        if (base + G < K && !grid_barrier(R.h, &s_ok, R.spin_limit)) return;
+    }
+    if (tid == 0 && adds) atomicAdd(&R.c->additions, adds);
+}
+
 // -------------------------------------------------------------- step 5 ---
 // scan_in[p] = (triangles of diameter p) << 24 | (claims at p), whose
 // exclusive prefix gives, at p, the rank of p's first triangle in triangle
@@ -754,38 +1095,82 @@ cudaError_t run_h1(void *ws, const H1Layout &H, int64_t n, const uint64_t *ek0, 
     // 3. the spanning forest; 4. the other columns
     k_h1_zlist<<<grid, 256, 0, s>>>(scan_in, zpref, m, zlist);
     k_h1_forest<<<1, 256, 0, s>>>(ev0, ev1, esort, zlist, zpref, m, n, tfirst, rlist, c, h);
-    H1Reduce R;
-    R.n = n;
-    R.vals0 = ev0;
-    R.vals1 = ev1;
-    R.esort = esort;
-    R.P = P;
-    R.tfirst = tfirst;
-    R.rlist = rlist;
-    R.head = head;
-    R.claims = claims;
-    R.node_key = at<uint64_t>(ws, H.node_key);
-    R.node_pos = at<uint32_t>(ws, H.node_pos);
-    R.node_next = at<int32_t>(ws, H.node_next);
-    R.node_within = at<uint32_t>(ws, H.node_within);
-    R.own_node = at<uint32_t>(ws, H.own_node);
-    R.own_off = at<uint64_t>(ws, H.own_off);
-    R.own_len = at<uint32_t>(ws, H.own_len);
-    R.col_x = at<uint64_t>(ws, H.col_x);
-    R.col_m = at<uint64_t>(ws, H.col_m);
-    R.col_cap = H.col_cap;
-    R.pool = at<uint64_t>(ws, H.pool);
-    R.pool_cap = H.pool_cap;
-    R.c = c;
-    R.h = h;
-    k_h1_reduce<<<1, kH1Threads, 0, s>>>(R);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    uint64_t *node_key = at<uint64_t>(ws, H.node_key), *own_off = at<uint64_t>(ws, H.own_off);
+    uint32_t *node_pos = at<uint32_t>(ws, H.node_pos), *node_within = at<uint32_t>(ws, H.node_within);
+    uint32_t *own_node = at<uint32_t>(ws, H.own_node), *own_len = at<uint32_t>(ws, H.own_len);
+    int32_t *node_next = at<int32_t>(ws, H.node_next);
+    if (H.ctas) {
+        const int ctas = H.ctas < sm_count() ? H.ctas : sm_count();
+        H1Bits R;
+        R.n = int(n);
+        R.m = m;
+        R.vals0 = ev0;
+        R.vals1 = ev1;
+        R.esort = esort;
+        R.P = P;
+        R.tfirst = tfirst;
+        R.rlist = rlist;
+        R.head = head;
+        R.claims = claims;
+        R.node_key = node_key;
+        R.node_pos = node_pos;
+        R.node_next = node_next;
+        R.node_within = node_within;
+        R.own_node = own_node;
+        R.own_off = own_off;
+        R.own_len = own_len;
+        R.bits = at<uint32_t>(ws, H.bits);
+        R.bit_words = H.bit_stride / 4;
+        R.pub = at<uint32_t>(ws, H.pub);
+        R.pub_piv = at<uint32_t>(ws, H.pub_piv);
+        R.pub_len = R.pub_piv + 2 * size_t(H.ctas);
+        R.pool = at<uint32_t>(ws, H.pool);
+        R.pool_cap = H.pool_cap;
+        R.c = c;
+        R.h = h;
+        R.spin_limit = kSpinLimit;
+        const size_t blocks = R.bit_words * 32 / kH1BlockBits;
+        const size_t smem = 4 * (size_t(m + 31) / 32 + (blocks + 31) / 32);
+        e = cudaFuncSetAttribute(k_h1_columns, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+        void *args[] = {&R};
+        if (e == cudaSuccess)
+            e = cudaLaunchCooperativeKernel((const void *)k_h1_columns, dim3(unsigned(ctas)), dim3(kH1Threads), args,
+                                            smem, s);
+        if (e != cudaSuccess) return e;
+    } else {
+        H1Reduce R;
+        R.n = n;
+        R.vals0 = ev0;
+        R.vals1 = ev1;
+        R.esort = esort;
+        R.P = P;
+        R.tfirst = tfirst;
+        R.rlist = rlist;
+        R.head = head;
+        R.claims = claims;
+        R.node_key = node_key;
+        R.node_pos = node_pos;
+        R.node_next = node_next;
+        R.node_within = node_within;
+        R.own_node = own_node;
+        R.own_off = own_off;
+        R.own_len = own_len;
+        R.col_x = at<uint64_t>(ws, H.col_x);
+        R.col_m = at<uint64_t>(ws, H.col_m);
+        R.col_cap = H.col_cap;
+        R.pool = at<uint64_t>(ws, H.pool);
+        R.pool_cap = H.pool_cap;
+        R.c = c;
+        R.h = h;
+        k_h1_reduce<<<1, kH1Threads, 0, s>>>(R);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    }
     if (after_reduce && (e = cudaEventRecord(after_reduce, s)) != cudaSuccess) return e;
     // 5. ranks in triangle order, the bars
     k_h1_pack<<<grid, 256, 0, s>>>(tcount, claims, m, scan_in);
     if ((e = h1_scan(scan_in, m, tpref, bsum, s)) != cudaSuccess) return e;
-    k_h1_emit<<<grid, 256, 0, s>>>(ek0, ek1, ev0, ev1, esort, a_of, tfirst, zpref, tpref, R.own_node, R.node_key,
-                                   R.node_within, head, R.node_next, m, n, m - (n - 1), bars, c);
+    k_h1_emit<<<grid, 256, 0, s>>>(ek0, ek1, ev0, ev1, esort, a_of, tfirst, zpref, tpref, own_node, node_key,
+                                   node_within, head, node_next, m, n, m - (n - 1), bars, c);
     return cudaGetLastError();
 }
 

@@ -282,13 +282,25 @@ constexpr int kH1VertexBits = 12;
 constexpr int kH1Threads = 1024;
 constexpr int64_t kH1ScanItems = 4 * kH1Threads;
 constexpr int kH1Runs = 32;
+// Columns as bit sets (k_h1_columns): up to kH1BitsMaxN points, where the bits
+// of the edges and of the touched blocks fit shared memory; at most
+// kH1BitsCtas columns at a time, in at most kH1BitsBytes of the workspace.
+constexpr int64_t kH1BitsMaxN = 1024;
+constexpr int kH1BitsCtas = 128;
+constexpr size_t kH1BitsBytes = size_t(1) << 31;
+constexpr int kH1BlockBits = 1024;  // bits per touched block
 
 // The first-homology regions of a workspace, after the dimension-0 layout.
-// col_cap bounds a column under reduction, pool_cap the reduced columns kept
-// (PH0_ETOOBIG beyond either): the runs of a column live in col_x, col_m
-// holds a merge.
+// Up to kH1BitsMaxN points a column under reduction is a bit set (bits, one
+// per CTA of k_h1_columns, with its list of edges in pub) and pool_cap bounds
+// the edges of the reduced columns' lists.  Above, col_cap bounds a column
+// under reduction, pool_cap the keys of the reduced columns kept (PH0_ETOOBIG
+// beyond either): the runs of a column live in col_x, col_m holds a merge.
 struct H1Layout {
     int64_t T, blocks, col_cap, pool_cap;
+    int ctas;              // columns reduced at a time (bit sets), 0: one CTA with runs
+    size_t bit_stride;     // bytes of a bit set
+    size_t bits, pub, pub_piv;
     size_t cnt, aof, posof, pmat, tcount, tfirst, scan_in, zpref, tpref, bsum, zlist, rlist, head, claims,
         node_key, node_pos, node_next, node_within, own_node, own_off, own_len, col_x, col_m, pool, total;
     H1Layout(int64_t n, size_t base) {
@@ -301,6 +313,15 @@ struct H1Layout {
         auto clamp = [](int64_t x, int64_t lo, int64_t hi) { return x < lo ? lo : (x > hi ? hi : x); };
         col_cap = clamp(2 * T, int64_t(1) << 18, int64_t(1) << 23) + 2 * n + 1;
         pool_cap = clamp(8 * T, int64_t(1) << 20, int64_t(1) << 26) + n + 1;
+        ctas = 0;
+        bit_stride = 0;
+        if (n <= kH1BitsMaxN) {
+            bit_stride = align_up((size_t(m) * size_t(n) + 7) / 8, kH1BlockBits / 8) + kH1BlockBits / 8;
+            const size_t fit = kH1BitsBytes / (bit_stride + 4 * size_t(m + 1));
+            ctas = fit < size_t(kH1BitsCtas) ? int(fit) : kH1BitsCtas;
+            col_cap = 0;
+            pool_cap *= 2;  // 4-byte entries
+        }
         size_t off = base;
         auto take = [&](size_t bytes) {
             size_t o = off;
@@ -331,7 +352,10 @@ struct H1Layout {
         own_len = take(4 * M1);
         col_x = take(8 * size_t(col_cap));
         col_m = take(8 * size_t(col_cap));
-        pool = take(8 * size_t(pool_cap));
+        pool = take(ctas ? 4 * size_t(pool_cap) : 8 * size_t(pool_cap));
+        bits = take(size_t(ctas) * bit_stride);
+        pub = take(size_t(ctas) * 4 * M1);
+        pub_piv = take(size_t(ctas) * 3 * 4);  // pivots (by the round's parity), lengths
         total = off;
     }
 };
