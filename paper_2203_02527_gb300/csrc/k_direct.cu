@@ -43,20 +43,15 @@ constexpr int kDirCountThreads = 512;
 constexpr int kDirMaxBuckets = 512;        // of kDirBucketLarge keys up to kDirectMaxN points
 constexpr int kDirBucketSmall = 4096, kDirBucketLarge = 8192;
 constexpr int kDirStrip = 32;              // rows of a tile staged at a time
+constexpr double kDirCrowd = 6.0;          // standard deviations over the mean that crowd a bucket
 constexpr int kDirMaxRounds = 13;          // 2^12 > kDirectMaxN components halve each round
 constexpr int kDirMstThreads = 1024;
 constexpr int kDirOwn = 3;                 // columns per thread of the claim rounds
 constexpr int kDirClaimRounds = 64;        // then one thread finishes in order
 static_assert(kDirOwn * kDirMstThreads >= kDirectMaxN, "every column has a thread");
 constexpr uint64_t kNoKey = kKeyBits;      // above every squared distance
-constexpr size_t kDirDistSmem = 200 * 1024;
+constexpr size_t kDirDistSmem = 220 * 1024;
 constexpr size_t kDirMstSmem = 224 * 1024;  // beside the static words, below the 227 KB of a CTA
-
-// A distance that occurs more than once: its key and the occurrences beyond the first.
-struct DirectRepeat {
-    uint64_t key;
-    uint32_t extra, pad;
-};
 
 struct DirectArgs {
     const float *pts;
@@ -65,7 +60,9 @@ struct DirectArgs {
     int buckets, bcap, table;  // hash buckets of keys, room of each, slots of its table
     uint64_t *bkeys;           // [buckets][bcap]
     uint32_t *bcount;          // [buckets] keys appended (beyond bcap: not stored)
-    DirectRepeat *rep;         // [m / 2] repeated distances
+    uint64_t *repk;            // [3 m / 4 + 1] repeated distances: key and how many occurrences
+    uint32_t *repx;            //     it stands for beyond the one left (a key may have several records)
+    uint32_t crowd;            // keys of a strip in one bucket that only repeated distances explain
     uint64_t *mat;             // [n][ldm] keys
     uint64_t *candk;           // [n][kDirectChunks] smallest key of each row and block of columns
     uint16_t *candv;           // ... and its column
@@ -113,7 +110,12 @@ __device__ __forceinline__ uint32_t hash_slot(uint64_t x, int table) {
 // latency of the steps.  The keys of the upper triangle are also appended to
 // the hash buckets, one counter addition per strip and bucket (a global hash
 // table with one compare-and-swap per key took 14 us of 28 at 256 points: an
-// SM gets about one such atomic back per ten clocks).
+// SM gets about one such atomic back per ten clocks).  A strip that crowds a
+// bucket (kDirCrowd standard deviations over the mean, which distinct keys
+// reach in one strip of hundreds) holds repeated distances: it appends one
+// key of each and records the others as repeats at once, so that lattices
+// and the like do not overflow the buckets (14^3 lattice points: 2744 points,
+// 299 distances; without this step 4.6 ms a call, the sorted path 0.63).
 template <int D, int BT>
 __global__ void __launch_bounds__(kDirThreads) k_direct_dist(const DirectArgs A) {
     const int n = A.n, d = D > 0 ? D : A.d, bt = BT > 0 ? BT : A.bt;
@@ -121,6 +123,7 @@ __global__ void __launch_bounds__(kDirThreads) k_direct_dist(const DirectArgs A)
     __shared__ uint64_t s_min[kDirThreads / 32], s_max[kDirThreads / 32];
     __shared__ int s_fixed;
     __shared__ uint32_t s_bcnt[kDirMaxBuckets], s_bbase[kDirMaxBuckets];
+    __shared__ uint32_t s_nrep, s_rbase, s_extra;
     double *su = s_coord, *sv = s_coord + size_t(d) * bt;
     int64_t *xu = reinterpret_cast<int64_t *>(su), *xv = reinterpret_cast<int64_t *>(sv);
     uint64_t *s_strip = reinterpret_cast<uint64_t *>(s_coord + size_t(2) * d * bt);  // [32][bt + 1]
@@ -129,6 +132,10 @@ __global__ void __launch_bounds__(kDirThreads) k_direct_dist(const DirectArgs A)
     int32_t *s_lo = s_g + d, *s_hi = s_lo + d;
     uint32_t *s_narrow30 = reinterpret_cast<uint32_t *>(s_hi + d);  // [(d+31)/32]
     uint16_t *s_colv = reinterpret_cast<uint16_t *>(s_narrow30 + (d + 31) / 32);  // [bt]
+    // a crowded strip's hash table of the places of its distinct keys, and
+    // their occurrences (two 16-bit counts per word; bt is even)
+    uint16_t *s_tab = s_colv + bt;                                                // [2 * 32 * bt]
+    uint32_t *s_occ = reinterpret_cast<uint32_t *>(s_tab + 2 * kDirStrip * bt);   // [32 * bt / 2]
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     constexpr int kWarps = kDirThreads / 32;
     static_assert(kWarps == 32, "one warp reduces the others' values");
@@ -238,13 +245,74 @@ __global__ void __launch_bounds__(kDirThreads) k_direct_dist(const DirectArgs A)
         __syncthreads();
         // the place of each key of the upper triangle among the strip's keys of its bucket
         uint32_t place[kPer];
+        bool crowded = false;
 #pragma unroll
         for (int w = 0; w < kPer; ++w) {
             const int i = tid / bt + w * rpp;
-            if (i < kDirStrip && u0 + s0 + i < v && v < n)
+            if (i < kDirStrip && u0 + s0 + i < v && v < n) {
                 place[w] = atomicAdd(s_bcnt + hash_bucket(key_hash(s_strip[i * (bt + 1) + j]), A.buckets), 1u);
+                crowded |= place[w] >= A.crowd;
+            }
         }
-        __syncthreads();
+        if (__syncthreads_or(crowded)) {
+            const uint32_t slots = uint32_t(2 * kDirStrip * bt);
+            uint32_t *tab32 = reinterpret_cast<uint32_t *>(s_tab);
+            for (uint32_t i = tid; i < slots / 2; i += kDirThreads) tab32[i] = 0xffffffffu;
+            for (int i = tid; i < kDirStrip * bt / 2; i += kDirThreads) s_occ[i] = 0;
+            for (int b = tid; b < A.buckets; b += kDirThreads) s_bcnt[b] = 0;
+            if (tid == 0) s_nrep = s_extra = 0;
+            __syncthreads();
+            // one key of each distance keeps its place, the others count for it
+            uint32_t mine = 0;
+#pragma unroll
+            for (int w = 0; w < kPer; ++w) {
+                const int i = tid / bt + w * rpp;
+                if (i >= kDirStrip || u0 + s0 + i >= v || v >= n) continue;
+                const uint64_t k = s_strip[i * (bt + 1) + j];
+                uint32_t slot = hash_slot(key_hash(k), int(slots));
+                for (uint32_t pr = 0; pr < slots; ++pr) {  // at most half the slots fill
+                    uint32_t old = *(volatile uint16_t *)(s_tab + slot);
+                    if (old == 0xffffu)
+                        old = atomicCAS(s_tab + slot, (unsigned short)0xffffu, (unsigned short)(i * bt + j));
+                    const uint32_t at = old == 0xffffu ? uint32_t(i * bt + j) : old;
+                    if (old == 0xffffu) mine |= 1u << w;
+                    if (old == 0xffffu || s_strip[(at / bt) * (bt + 1) + at % bt] == k) {
+                        atomicAdd(s_occ + at / 2, 1u << (16 * (at & 1)));
+                        break;
+                    }
+                    slot = (slot + 1) & (slots - 1);
+                }
+                place[w] = 0xffffffffu;
+            }
+            __syncthreads();
+            uint32_t at[kPer];
+#pragma unroll
+            for (int w = 0; w < kPer; ++w) {
+                if (!((mine >> w) & 1u)) continue;
+                const int i = tid / bt + w * rpp, x = i * bt + j;
+                const uint32_t extra = ((s_occ[x / 2] >> (16 * (x & 1))) & 0xffffu) - 1;
+                place[w] = atomicAdd(s_bcnt + hash_bucket(key_hash(s_strip[i * (bt + 1) + j]), A.buckets), 1u);
+                if (extra) {
+                    at[w] = atomicAdd(&s_nrep, 1u);
+                    atomicAdd(&s_extra, extra);
+                } else {
+                    mine &= ~(1u << w);
+                }
+            }
+            __syncthreads();
+            if (tid == 0 && s_nrep) {
+                s_rbase = atomicAdd(&A.h->direct_strips, s_nrep);
+                atomicAdd(&A.h->direct_dups, s_extra);
+            }
+            __syncthreads();
+#pragma unroll
+            for (int w = 0; w < kPer; ++w) {
+                if (!((mine >> w) & 1u)) continue;
+                const int i = tid / bt + w * rpp, x = i * bt + j;
+                A.repk[s_rbase + at[w]] = s_strip[i * (bt + 1) + j];
+                A.repx[s_rbase + at[w]] = ((s_occ[x / 2] >> (16 * (x & 1))) & 0xffffu) - 1;
+            }
+        }
         uint32_t base = 0;
         if (tid < A.buckets && s_bcnt[tid]) base = atomicAdd(A.bcount + tid, s_bcnt[tid]);
         // rows: the upper triangle (a diagonal tile: all of the tile)
@@ -288,7 +356,7 @@ __global__ void __launch_bounds__(kDirThreads) k_direct_dist(const DirectArgs A)
 #pragma unroll
         for (int w = 0; w < kPer; ++w) {
             const int i = tid / bt + w * rpp;
-            if (i < kDirStrip && u0 + s0 + i < v && v < n) {
+            if (i < kDirStrip && u0 + s0 + i < v && v < n && place[w] != 0xffffffffu) {
                 const uint64_t k = s_strip[i * (bt + 1) + j];
                 const uint32_t b = hash_bucket(key_hash(k), A.buckets), at = s_bbase[b] + place[w];
                 if (at < uint32_t(A.bcap)) A.bkeys[size_t(b) * A.bcap + at] = k;
@@ -368,9 +436,11 @@ struct DirMst {
 
 // The repeated distances of the buckets first, first + step, ...: a hash table
 // of (key + 1, occurrences) in shared memory per bucket.  A bucket whose keys
-// did not fit its room (a distance that occurs many times) takes them from
-// the matrix instead.  The hash spreads distinct keys evenly (the mean is at
-// most half the table), so a free slot ends every probe.
+// did not fit its room (distances that occur many times, but seldom within a
+// strip) takes the upper triangle's keys from the matrix instead, with the
+// repeats that crowded strips recorded taken off.  The hash spreads distinct
+// keys evenly (the mean is at most half the table), so a free slot ends every
+// probe.
 __device__ void direct_repeats(const DirectArgs &A, unsigned char *s_dyn, int first, int step) {
     unsigned long long *s_key = reinterpret_cast<unsigned long long *>(s_dyn);
     uint32_t *s_occ = reinterpret_cast<uint32_t *>(s_key + A.table);
@@ -403,19 +473,38 @@ __device__ void direct_repeats(const DirectArgs &A, unsigned char *s_dyn, int fi
                 insert(k, key_hash(k));
             }
         } else {
-            for (int u = 0; u < A.n - 1; ++u)
-                for (int v = u + 1 + tid; v < A.n; v += T) {
-                    const uint64_t k = A.mat[size_t(u) * A.ldm + v], x = key_hash(k);
-                    if (hash_bucket(x, A.buckets) == uint32_t(b)) insert(k, x);
+            const uint32_t n = uint32_t(A.n), items = n * n;
+            for (uint32_t i0 = tid; i0 < items; i0 += 8 * T) {
+                uint64_t key[8];
+#pragma unroll
+                for (int q = 0; q < 8; ++q) {
+                    const uint32_t i = i0 + q * T, u = i / n, v = i - u * n;
+                    key[q] = i < items && u < v ? __ldcg(A.mat + size_t(u) * A.ldm + v) : kNoKey;
                 }
+#pragma unroll
+                for (int q = 0; q < 8; ++q) {
+                    const uint64_t x = key_hash(key[q]);
+                    if (key[q] != kNoKey && hash_bucket(x, A.buckets) == uint32_t(b)) insert(key[q], x);
+                }
+            }
+            __syncthreads();
+            const uint32_t strips = A.h->direct_strips;
+            for (uint32_t r = tid; r < strips; r += T) {
+                const uint64_t k = A.repk[r], x = key_hash(k);
+                if (hash_bucket(x, A.buckets) != uint32_t(b)) continue;
+                uint32_t slot = hash_slot(x, A.table);
+                for (int pr = 0; pr < A.table && s_key[slot] != k + 1; ++pr) slot = (slot + 1) & uint32_t(A.table - 1);
+                if (s_key[slot] == k + 1) atomicSub(s_occ + slot, A.repx[r]);
+            }
         }
         __syncthreads();
         uint32_t extra = 0;
         for (int i = tid; i < A.table; i += T) {
             const uint32_t o = s_occ[i];
             if (o > 1) {
-                const uint32_t q = atomicAdd(&A.h->direct_repeats, 1u);
-                A.rep[q] = DirectRepeat{s_key[i] - 1, o - 1, 0u};
+                const uint32_t q = A.h->direct_strips + atomicAdd(&A.h->direct_repeats, 1u);
+                A.repk[q] = s_key[i] - 1;
+                A.repx[q] = o - 1;
                 extra += o - 1;
             }
         }
@@ -460,6 +549,8 @@ __global__ void __launch_bounds__(kDirMstThreads, 1) k_direct_mst(const DirectAr
     uint16_t *s_par = reinterpret_cast<uint16_t *>(s_dyn + S.par);
     uint16_t *s_sel = reinterpret_cast<uint16_t *>(s_dyn + S.sel);  // [n] component at the other end
     const int own = n > rank ? (n - rank + cl - 1) / cl : 0;  // rows of this CTA
+    // no CTA writes to another's shared memory before all have started
+    cluster.barrier_arrive();
 
     for (int u = tid; u < n; u += T) {
         s_comp[u] = uint16_t(u);
@@ -475,6 +566,7 @@ __global__ void __launch_bounds__(kDirMstThreads, 1) k_direct_mst(const DirectAr
     }
     int buf = 0;
     bool more = n > 1;
+    cluster.barrier_wait();
     for (int round = 0; round < kDirMaxRounds && more; ++round) {
         buf = round & 1;
         for (int c = tid; c < n; c += T) {
@@ -788,10 +880,10 @@ __global__ void __launch_bounds__(kDirCountThreads, 2) k_direct_count(const Dire
             if (s < np) atomicSub(s_corr + s, 1);
         }
     };
-    const uint32_t reps = A.h->direct_repeats;
+    const uint32_t reps = A.h->direct_strips + A.h->direct_repeats;
     for (uint32_t q = blockIdx.x * kDirCountThreads + tid; q < reps; q += gridDim.x * kDirCountThreads) {
-        const DirectRepeat r = A.rep[q];
-        if (r.key <= top) atomicAdd(s_dup + place(r.key), int32_t(r.extra));
+        const uint64_t k = A.repk[q];
+        if (k <= top) atomicAdd(s_dup + place(k), int32_t(A.repx[q]));
     }
     // rows a and n-2-a together hold n edges (n - 1 - a and a + 1; the middle
     // row of an even n stands alone): item i is edge i % n of pair i / n
@@ -915,7 +1007,7 @@ int direct_tile(int64_t n) { return n <= 32 * kDirectChunks ? 32 : n <= 64 * kDi
 
 size_t direct_dist_smem(int bt, int d) {
     return size_t(2) * bt * d * 8 + size_t(kDirStrip) * (bt + 1) * 8 + size_t(bt) * 8 + size_t(3) * d * 4 +
-           size_t((d + 31) / 32) * 4 + size_t(bt) * 2;
+           size_t((d + 31) / 32) * 4 + size_t(bt) * 2 + size_t(6) * kDirStrip * bt;
 }
 
 // The regions of this form within a workspace (from L.key[0] on, up to the
@@ -923,7 +1015,7 @@ size_t direct_dist_smem(int bt, int d) {
 struct DirectRegions {
     int64_t ldm;
     int buckets, bcap, table;
-    size_t bcount, cnt, corr, dup, zero_end, bkeys, rep, mat, candk, candv, pkey, puv, plow, total;
+    size_t bcount, cnt, corr, dup, zero_end, bkeys, repk, repx, mat, candk, candv, pkey, puv, plow, total;
     explicit DirectRegions(const Layout &L) {
         const size_t n = size_t(L.n);
         size_t off = L.key[0];
@@ -934,11 +1026,13 @@ struct DirectRegions {
         };
         ldm = (L.n + 3) & ~int64_t(3);
         // buckets of at most 4096 or 8192 keys on average: enough of them for
-        // the idle SMs, few counters per strip; a quarter more room is over
-        // ten standard deviations
+        // the idle SMs, few counters per strip.  Twice the room (small clouds:
+        // what the workspace has): distances
+        // repeated hundreds of times each, but seldom within a strip (random
+        // integers in one dimension), spread the buckets' counts that far
         const int per = L.m <= int64_t(1) << 19 ? kDirBucketSmall : kDirBucketLarge;
         buckets = int((L.m + per - 1) / per);
-        bcap = int((L.m + buckets - 1) / buckets) * 5 / 4 + 64;
+        bcap = int((L.m + buckets - 1) / buckets) * (per == kDirBucketSmall ? 7 : 8) / 4 + 64;
         table = 2 * per;
         bcount = take(4 * size_t(buckets));
         cnt = take(4 * n);
@@ -946,7 +1040,10 @@ struct DirectRegions {
         dup = take(4 * n);
         zero_end = off;
         bkeys = take(8 * size_t(buckets) * size_t(bcap));
-        rep = take(sizeof(DirectRepeat) * size_t(L.m / 2 + 1));
+        // a strip's record takes at least one key away, a bucket's at least
+        // one of those left, and there are no more of the first than keys left
+        repk = take(8 * size_t(L.m * 3 / 4 + 1));
+        repx = take(4 * size_t(L.m * 3 / 4 + 1));
         mat = take(8 * n * size_t(ldm));
         candk = take(8 * n * kDirectChunks);
         candv = take(2 * n * kDirectChunks);
@@ -987,9 +1084,12 @@ cudaError_t launch_direct(void *ws, const Layout &L, const float *pts, int64_t n
     A.buckets = G.buckets;
     A.bcap = G.bcap;
     A.table = G.table;
+    const double mean = double(kDirStrip * A.bt) / double(A.buckets);
+    A.crowd = uint32_t(mean + kDirCrowd * sqrt(mean)) + 1;
     A.bkeys = at<uint64_t>(ws, G.bkeys);
     A.bcount = at<uint32_t>(ws, G.bcount);
-    A.rep = at<DirectRepeat>(ws, G.rep);
+    A.repk = at<uint64_t>(ws, G.repk);
+    A.repx = at<uint32_t>(ws, G.repx);
     A.mat = at<uint64_t>(ws, G.mat);
     A.candk = at<uint64_t>(ws, G.candk);
     A.candv = at<uint16_t>(ws, G.candv);

@@ -164,7 +164,8 @@ struct Header {
     // starts at zero)
     int32_t direct;
     uint32_t direct_dups;
-    uint32_t direct_repeats;
+    uint32_t direct_strips;      // (records of the distance kernel's crowded strips,
+    uint32_t direct_repeats;     // and of the buckets after them)
     uint32_t direct_done;
     uint64_t direct_nkmin;
     // class partition of the early path (radix slot kClassSlot): the key
