@@ -176,8 +176,11 @@ typedef struct {
                                passes; clouds of at most 32768 points whose keys' top
                                part takes at most 256 values, else the short sort runs;
                                not with wide_ids = 1): 1 on any such cloud, 0 never,
-                               -1 built-in: from 2^22 edges (n >= 2897) up to n = 32768
-                               in dimension 4 and up                                   */
+                               2 and 3: as 0 and 1 where the whole path sorts at all (up
+                               to 2896 points it does not, nor above up to 65535 in
+                               dimensions 1 to 3 and from 2^24 edges); -1 built-in:
+                               there, and on other clouds from 2^22 edges (n >= 2897) up
+                               to n = 32768 in dimension 4 and up the packed sort      */
 } ph0_tuning;
 
 /* Early-terminating whole path (the paper has no counterpart; it exploits

@@ -267,5 +267,36 @@ __host__ __device__ __forceinline__ uint64_t sq_dist_mixed_ct(const int64_t *xu,
     return double_bits(s);
 }
 
+// sq_dist_mixed for any dimension and a stride S known at compile time:
+// dimensions in groups of eight, then of two, with the loads at fixed offsets
+// (a loop over single dimensions waits for each one's loads and branch).
+template <int S>
+__host__ __device__ __forceinline__ uint64_t sq_dist_mixed_st(const int64_t *xu, const int64_t *xv,
+                                                              const int32_t *g, int d, const uint32_t *narrow) {
+    double s = 0.0;
+    int k = 0;
+    for (; k + 8 <= d; k += 8) {
+        const uint32_t nw = narrow[k >> 5] >> (k & 31);
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            const double p = square_value(xu[(k + j) * S], xv[(k + j) * S], g[k + j], (nw >> j) & 1u);
+            s = k + j == 0 ? p : add_rn(s, p);
+        }
+    }
+    for (; k + 2 <= d; k += 2) {
+        const uint32_t nw = narrow[k >> 5] >> (k & 31);  // k is even: both bits in one word
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            const double p = square_value(xu[(k + j) * S], xv[(k + j) * S], g[k + j], (nw >> j) & 1u);
+            s = k + j == 0 ? p : add_rn(s, p);
+        }
+    }
+    if (k < d) {
+        const double p = square_value(xu[k * S], xv[k * S], g[k], (narrow[k >> 5] >> (k & 31)) & 1u);
+        s = k == 0 ? p : add_rn(s, p);
+    }
+    return double_bits(s);
+}
+
 }  // namespace emu
 }  // namespace ph0

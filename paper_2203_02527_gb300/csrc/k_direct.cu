@@ -87,13 +87,7 @@ __device__ __forceinline__ int warp_argmin(uint64_t k, uint64_t &mn) {
     return __ffs(who) - 1;
 }
 
-// Multiplicative (Fibonacci) hashing: the bucket from the high bits, the slot
-// in its table from the low ones.
-__device__ __forceinline__ uint64_t key_hash(uint64_t key) {
-    uint64_t x = key * 0x9E3779B97F4A7C15ull;
-    x ^= x >> 32;
-    return x * 0x9E3779B97F4A7C15ull;
-}
+// key_hash: the bucket from the high bits, the slot in its table from the low ones.
 __device__ __forceinline__ uint32_t hash_bucket(uint64_t x, int buckets) {
     return __umulhi(uint32_t(x >> 32), uint32_t(buckets));
 }
@@ -118,7 +112,8 @@ __device__ __forceinline__ uint32_t hash_slot(uint64_t x, int table) {
 // 299 distances; without this step 4.6 ms a call, the sorted path 0.63).
 template <int D, int BT>
 __global__ void __launch_bounds__(kDirThreads) k_direct_dist(const DirectArgs A) {
-    const int n = A.n, d = D > 0 ? D : A.d, bt = BT > 0 ? BT : A.bt;
+    const int n = A.n, d = D > 0 ? D : A.d;
+    constexpr int bt = BT;
     extern __shared__ double s_coord[];
     __shared__ uint64_t s_min[kDirThreads / 32], s_max[kDirThreads / 32];
     __shared__ int s_fixed;
@@ -225,7 +220,7 @@ __global__ void __launch_bounds__(kDirThreads) k_direct_dist(const DirectArgs A)
             if (u < n && v < n && u != v) {
                 if (fixed) {
                     if constexpr (D > 0) kb = emu::sq_dist_mixed_ct<D, BT>(xu + i, xv + j, s_g, nw);
-                    else kb = emu::sq_dist_mixed(xu + i, xv + j, s_g, d, bt, bt, s_narrow30);
+                    else kb = emu::sq_dist_mixed_st<BT>(xu + i, xv + j, s_g, d, s_narrow30);
                 } else {
                     double s = 0.0;
                     for (int k = 0; k < d; ++k) {
@@ -1126,7 +1121,10 @@ cudaError_t launch_direct(void *ws, const Layout &L, const float *pts, int64_t n
             PH0_DIRECT_CASE(8)
             PH0_DIRECT_CASE(16)
             PH0_DIRECT_CASE(32)
-            default: return go(k_direct_dist<0, 0>);
+            default:
+                if (A.bt == 32) return go(k_direct_dist<0, 32>);
+                if (A.bt == 64) return go(k_direct_dist<0, 64>);
+                return go(k_direct_dist<0, 128>);
         }
 #undef PH0_DIRECT_CASE
     };

@@ -68,17 +68,15 @@ __device__ __forceinline__ void tile_coords(int64_t lin, int64_t T, int64_t &bi,
 }
 
 // D, BT > 0: the instance for dimension D and tile edge BT (the d and bt
-// arguments equal them); 0: any.
+// arguments equal them); 0: any (the dimensions then in unrolled groups).
 template <int D, int BT>
 __global__ void __launch_bounds__(kDistThreads)
 k_dist(const float *__restrict__ pts, int n, int d, int64_t ld, int bt, int hw16,
        uint64_t *__restrict__ key, uint32_t *__restrict__ val, Header *__restrict__ h,
-       const int32_t *gate, int wide, int packed) {
+       const int32_t *gate, int wide, int form) {
     if (gate && ld_volatile(gate) == 0) return;  // a gated run (the sort's fallback) that is not needed
-    if constexpr (D > 0) {
-        d = D;
-        bt = BT;
-    }
+    if constexpr (D > 0) d = D;
+    if constexpr (BT > 0) bt = BT;
     // [d][bt] u block, then [d][bt] v block: binary64 values, or int64 fixed
     // point in units of 2^g[k] on the integer path; then g[d], lo[d], hi[d]
     extern __shared__ double s_coord[];
@@ -166,13 +164,18 @@ k_dist(const float *__restrict__ pts, int n, int d, int64_t ld, int bt, int hw16
     const int rows_per_pass = blockDim.x / bt;     // bt divides blockDim (bt <= 128)
     const int v = v0 + j;
     // the record of edge (u, v): key, value, histograms, key range
-    auto emit = [&](int u, uint64_t kb) {
-        const int64_t e = edge_index(n, u, v);
+    auto emit = [&](int u, uint64_t kb, int64_t e) {
         // wide: the value is the edge index, whose bit 32 (above 92,682
         // points) rides in the key's bit 63, never set by a squared distance
         key[e] = wide ? kb | (uint64_t(e >> 32) << 63) : kb;
+        kmax = kb > kmax ? kb : kmax;
+        if (form == kDistHashed) {  // the smallest key is the first tree edge's
+            atomicAdd(&s_flat[hash_part(part_hash(kb))], 1u);
+            return;
+        }
+        kmin = kb < kmin ? kb : kmin;
         val[e] = wide ? uint32_t(e) : (uint32_t(u) << 16) | uint32_t(v);
-        if (packed) {
+        if (form == kDistPacked) {
 #pragma unroll
             for (int q = 0; q < kPackPasses - 1; ++q) atomicAdd(&s_flat[q * kMaxRadix + pack_key_digit(kb, q)], 1u);
         } else {
@@ -180,17 +183,22 @@ k_dist(const float *__restrict__ pts, int n, int d, int64_t ld, int bt, int hw16
             for (int q = 0; q < kLowPasses; ++q) atomicAdd(&s_hist[q][(kb >> (8 * q)) & (kRadix - 1)], 1u);
         }
         atomicAdd(&s_top[(kb >> kTopShift) & (kMaxRadix - 1)], 1u);
-        kmin = kb < kmin ? kb : kmin;
-        kmax = kb > kmax ? kb : kmax;
     };
     bool unrolled = false;
-    if constexpr (D > 0) {
+    if constexpr (BT > 0) {
         if (fixed && hw16 >= 16) {  // every row on the mixed form
             unrolled = true;
             const uint32_t nw = s_narrow30[0];
-            for (int i = threadIdx.x / BT; i < BT; i += kDistThreads / BT) {
+            // the edge index from row to row: e(u + 1, v) = e(u, v) + n - u - 2
+            constexpr int R = kDistThreads / BT;
+            int64_t e = edge_index(n, u0 + int(threadIdx.x) / BT, v);
+            for (int i = threadIdx.x / BT; i < BT; i += R) {
                 const int u = u0 + i;
-                if (u < v && v < n) emit(u, emu::sq_dist_mixed_ct<D, BT>(xu + i, xv + j, s_g, nw));
+                if (u < v && v < n) {
+                    if constexpr (D > 0) emit(u, emu::sq_dist_mixed_ct<D, BT>(xu + i, xv + j, s_g, nw), e);
+                    else emit(u, emu::sq_dist_mixed_st<BT>(xu + i, xv + j, s_g, d, s_narrow30), e);
+                }
+                e += R * (n - u - 2) - R * (R - 1) / 2;
             }
         }
     }
@@ -202,7 +210,7 @@ k_dist(const float *__restrict__ pts, int n, int d, int64_t ld, int bt, int hw16
                 if (!fixed) kb = uint64_t(__double_as_longlong(sq_dist_f64(su, sv, d, bt, i, j)));
                 else if ((i & 15) < hw16) kb = emu::sq_dist_mixed(xu + i, xv + j, s_g, d, bt, bt, s_narrow30);
                 else kb = emu::sq_dist_fixed(xu + i, xv + j, s_g, d, bt, bt, s_narrow);
-                emit(u, kb);
+                emit(u, kb, edge_index(n, u, v));
             }
         }
     }
@@ -223,15 +231,13 @@ k_dist(const float *__restrict__ pts, int n, int d, int64_t ld, int bt, int hw16
             kmin = s_min[w] < kmin ? s_min[w] : kmin;
             kmax = s_max[w] > kmax ? s_max[w] : kmax;
         }
-        if (kmin != ~0ull) {
-            atomicMin((unsigned long long *)&h->kmin, (unsigned long long)kmin);
-            atomicMax((unsigned long long *)&h->kmax, (unsigned long long)kmax);
-        }
+        if (kmin != ~0ull) atomicMin((unsigned long long *)&h->kmin, (unsigned long long)kmin);
+        if (kmax != 0) atomicMax((unsigned long long *)&h->kmax, (unsigned long long)kmax);
     }
     for (int b = threadIdx.x; b < kLowPasses * kRadix; b += blockDim.x) {
         const uint32_t c = s_flat[b];
         if (!c) continue;
-        if (packed) atomicAdd(&h->phist[b / kMaxRadix][b % kMaxRadix], c);
+        if (form != kDistShort) atomicAdd(&h->phist[b / kMaxRadix][b % kMaxRadix], c);
         else atomicAdd(&h->hist[b / kRadix][b % kRadix], c);
     }
     for (int b = threadIdx.x; b < kMaxRadix; b += blockDim.x)
@@ -253,7 +259,7 @@ int dist_tile(int d, int want) {
 
 cudaError_t launch_dist(const float *pts, int64_t n, int32_t d, int64_t ld, uint64_t *key,
                         uint32_t *val, Header *h, cudaStream_t s, int split16, int tile,
-                        const int32_t *gate, bool wide, bool packed) {
+                        const int32_t *gate, bool wide, DistForm form) {
     if (n < 2) return cudaSuccess;
     const int bt = dist_tile(d, tile);
     const size_t smem = dist_smem(bt, d);
@@ -265,7 +271,7 @@ cudaError_t launch_dist(const float *pts, int64_t n, int32_t d, int64_t ld, uint
         cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024);
         if (e != cudaSuccess) return e;
         kernel<<<unsigned(tiles), kDistThreads, smem, s>>>(pts, int(n), int(d), ld, bt, hw16, key, val, h, gate,
-                                                           wide ? 1 : 0, packed ? 1 : 0);
+                                                           wide ? 1 : 0, int(form));
         return cudaGetLastError();
     };
 #define PH0_DIST_CASE(DD)                                       \
@@ -282,6 +288,8 @@ cudaError_t launch_dist(const float *pts, int64_t n, int32_t d, int64_t ld, uint
         default: break;
     }
 #undef PH0_DIST_CASE
+    if (bt == 128) return go(k_dist<0, 128>);
+    if (bt == 64) return go(k_dist<0, 64>);
     return go(k_dist<0, 0>);
 }
 

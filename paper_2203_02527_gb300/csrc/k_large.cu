@@ -1,0 +1,1335 @@
+// k_large.cu -- the whole barcode path without a sort for clouds above the
+// size of k_direct.cu (Rawson, Sec. 2; Sec. 4 steps 1-5).
+//
+// As there, the reduction keeps n-1 of the n(n-1)/2 columns, the minimum
+// spanning tree in the order (distance, u, v), and of the other edges a bar
+// only reads counts.  Sorting every edge to get them moved 77 to 130 bytes per
+// edge in four or five passes bound by integer work; here every edge's key is
+// written once, read a few times as a stream, and moved twice:
+//   k_dist              step 1: the key of edge e at e; a histogram of a hash
+//   k_large_sample,     places of the 512 hash partitions; from a sample of
+//   k_large_prep        the keys a threshold that about 64 n edges lie below
+//   k_large_move<0>     the keys by partition; the edges below the threshold
+//                       as a list; a tile of few distances keeps one key of
+//                       each and records how many more it stands for
+//   k_large_tree        the tree by Boruvka's rounds (cooperative): on the
+//                       list while it joins components, then on all keys
+//   k_large_runs, merge the tree's edges in order
+//   k_reduce            their columns' pivot rows (k_reduce.cu)
+//   k_large_count       every edge up to the last killing edge counted at its
+//                       place among the killing edges
+//   k_large_sub,        the partitions' keys by bucket of about ten thousand
+//   k_large_move<1>
+//   k_large_repeats     step 3: repeated distances, a bucket at a time in a
+//                       bit table in shared memory
+//   k_large_emit        running sums, the bars
+// Every step is exact for any input: partitions and buckets are counted before
+// they are filled, a list that overflows is not used, and ties are ordered by
+// (u, v) throughout, so the results equal the sorted path's bit for bit.
+//
+// Measured (device time, 1.25G edges of 50,021 points in the plane; the short
+// sort's path 67.4 ms): k_dist 7.7 ms, k_large_move<0> 7.7, the tree and its
+// pivots 1.3, the count 1.8, k_large_sub 1.4, k_large_move<1> 5.8,
+// k_large_repeats 5.2: 31.1 ms.  32,768 points of four circles in 16
+// dimensions (537M edges): 26.9 ms (packed sort 34.4), of which the distances,
+// bound by the binary64 adder, 15.6.  The count, k_large_sub and the tree's
+// passes run near the copy bandwidth; the moves are bound by shared-memory
+// wavefronts (60 to 66% of the peak) and their barriers.
+#include "ph0_common.cuh"
+
+namespace ph0 {
+
+int sm_count();
+
+namespace {
+
+#ifndef PH0_LG_TILE
+#define PH0_LG_TILE 8192
+#endif
+constexpr int kLgTile = PH0_LG_TILE;           // keys a CTA moves at a time
+constexpr int kLgThreads = kLgTile / 8;
+constexpr int kLgPer = kLgTile / kLgThreads;
+constexpr int kLgParts = 512;
+constexpr int kLgMaxSub = 512;                 // buckets per partition
+constexpr int kLgBucket = 10240;               // keys per bucket on average, at most
+constexpr int kLgPass = 14336;                 // keys of a bucket looked at at once (14 bits)
+constexpr int kLgWords = 20480;                // of a bucket's bit table, slots of its hash table
+constexpr int kLgSuspects = 512, kLgSusSlots = 2048, kLgSusKeys = 1024;
+constexpr int kLgPart = 5120;                  // keys of a larger bucket looked at together
+constexpr int kLgRepThreads = 512;
+constexpr int kLgListPerPoint = 64;            // edges per point the list aims at
+constexpr int kLgListRoom = 512;               // ... and has room for
+constexpr int kLgSample = 1 << 17;
+constexpr int kLgTreeThreads = 512;
+constexpr int kLgRun = 2048;                   // tree edges sorted by a CTA
+constexpr int kLgHot = 8192;                   // longest tree edges whose counts stay in shared memory
+constexpr int kLgCountThreads = 512;
+constexpr int kLgLutBits = 11, kLgLut = 1 << kLgLutBits;
+constexpr int kLgSubCtas = 4;                  // CTAs per partition
+// keys of a tile in one partition that only repeated distances explain: the
+// mean and seven standard deviations
+constexpr uint32_t kLgCrowd = kLgTile == 8192 ? 44 : 28;
+static_assert(kLgTile == 8192 || kLgTile == 4096, "kLgCrowd");
+constexpr uint64_t kNone = ~uint64_t(0);       // above every key
+
+struct LgRepeat {
+    uint64_t key;
+    uint32_t extra, pad;
+};
+
+struct LgArgs {
+    int64_t m;
+    int n, nsub;
+    const uint64_t *mat;       // [m] key of edge e
+    uint64_t *part, *bkt;      // [m] keys by partition, by bucket
+    LgRepeat *rep;             // [m / 2] records of crowded tiles (in bkt's place, read before it is filled)
+    uint64_t *lkey;            // [lcap] the edges below the threshold: key,
+    uint32_t *luv;             //     (u << 16) | v
+    uint32_t lcap;
+    uint32_t *cand;            // [ccap] edges that bettered a component's best
+    uint32_t ccap;
+    uint32_t *comp, *parent;   // [n]
+    unsigned long long *best;  // [n] per component: smallest key leaving it,
+    uint32_t *buv;             //     its edge
+    uint64_t *tkey, *skey;     // [n] the tree's edges as found, in order
+    uint32_t *tuv, *suv;
+    const unsigned long long *kill_key;  // [n] k_reduce's pivots: position,
+    const uint32_t *kill_val;            //     row
+    uint32_t *low;             // [n] pivot row by position
+    uint32_t *cnt, *corr, *dup;  // [n] counts per place among the tree's edges
+    uint32_t *poff, *pcur;     // [512 + 1], [512] places of the partitions, their ends
+    uint32_t *bcnt, *bcur;     // [512][nsub] keys per bucket, filled
+    uint32_t *boff;            // [512][nsub]
+    Header *h;
+    ph0_bar *bars;
+    ph0_inf_bar *inf;
+    uint32_t spin_limit;
+};
+
+__device__ __forceinline__ uint32_t hash_sub(uint32_t x, int nsub) { return __umulhi(x << 9, uint32_t(nsub)); }
+
+// Exclusive prefix sum over the CTA (T threads); s_w: T / 32 + 1 words.
+template <int T>
+__device__ __forceinline__ uint32_t block_scan(uint32_t x, uint32_t *s_w, uint32_t &total) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint32_t inc = x;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += y;
+    }
+    if (lane == 31) s_w[warp] = inc;
+    __syncthreads();
+    if (warp == 0) {
+        const uint32_t w = lane < T / 32 ? s_w[lane] : 0u;
+        uint32_t wi = w;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, wi, o);
+            if (lane >= o) wi += y;
+        }
+        if (lane < T / 32) s_w[lane] = wi - w;
+        if (lane == T / 32 - 1) s_w[T / 32] = wi;
+    }
+    __syncthreads();
+    const uint32_t r = inc - x + s_w[warp];
+    total = s_w[T / 32];
+    __syncthreads();
+    return r;
+}
+
+__device__ __forceinline__ bool lg_before(uint64_t ka, uint32_t ua, uint64_t kb, uint32_t ub) {
+    return ka < kb || (ka == kb && ua < ub);
+}
+
+// Tree edges of a smaller key (the last tree edge's is at least as large).
+__device__ __forceinline__ int lg_place(const uint64_t *skey, int lo, int hi, uint64_t key) {
+    while (lo < hi) {
+        const int mid = (lo + hi) >> 1;
+        if (skey[mid] < key) lo = mid + 1;
+        else hi = mid;
+    }
+    return lo;
+}
+
+// ------------------------------------------------------------------ prep ---
+// One CTA: the partitions' places from the distance kernel's histogram; the
+// list's threshold from a sample of the keys (evenly spread, jittered):
+// a bin of key >> 48 (sixteen to the octave) and within it one of the next 15
+// bits, so that about kLgListPerPoint n edges lie below; and the bin below
+// which at most a sixteenth of those do (for the rounds on the list).
+__host__ __device__ __forceinline__ int lg_samples(int n) {
+    // four keys per point, so that a few hundred lie below the threshold
+    const int S = 4 * n;
+    return S < kLgSample / 8 ? kLgSample / 8 : S > kLgSample ? kLgSample : S;
+}
+__global__ void __launch_bounds__(256) k_large_sample(const LgArgs A) {
+    const uint32_t S = uint32_t(lg_samples(A.n)), step = uint32_t(A.m / S);  // m > 2^22
+    for (uint32_t i = blockIdx.x * 256 + threadIdx.x; i < S; i += gridDim.x * 256)
+        A.lkey[i] = A.mat[size_t(i) * step + __umulhi(i * 2654435761u, step)];
+}
+__global__ void __launch_bounds__(1024) k_large_prep(const LgArgs A) {
+    extern __shared__ uint32_t s_bin[];  // [32768]
+    __shared__ uint32_t s_w[33];
+    __shared__ uint32_t s_at, s_below;
+    const int tid = threadIdx.x;
+    {
+        const uint32_t c = tid < kLgParts ? A.h->phist[0][tid] : 0u;
+        uint32_t total;
+        const uint32_t off = block_scan<1024>(c, s_w, total);
+        if (tid < kLgParts) {
+            A.poff[tid] = off;
+            A.pcur[tid] = off;
+        }
+        if (tid == 0) A.poff[kLgParts] = total;
+    }
+    const int S = lg_samples(A.n);
+    const double want = double(kLgListPerPoint) * double(A.n) * double(S) / double(A.m);
+    uint64_t limit = 0;
+    uint32_t target = uint32_t(want);
+    uint64_t prefix = 0;
+    for (int level = 0; level < 2; ++level) {
+        for (int i = tid; i < 32768; i += 1024) s_bin[i] = 0;
+        __syncthreads();
+#pragma unroll 16
+        for (uint32_t i = tid; i < uint32_t(S); i += 1024) {
+            const uint64_t k = A.lkey[i];
+            if (level == 0) atomicAdd(s_bin + ((k >> 48) & 32767), 1u);
+            else if ((k >> 48) == prefix) atomicAdd(s_bin + ((k >> 33) & 32767), 1u);
+        }
+        __syncthreads();
+        // the bin in which the running count passes the target
+        uint32_t sum = 0;
+        for (int i = 0; i < 32; ++i) sum += s_bin[tid * 32 + ((i + tid) & 31)];
+        uint32_t total;
+        uint32_t run = block_scan<1024>(sum, s_w, total);
+        if (tid == 0) s_at = 32768;
+        __syncthreads();
+        if (level == 0 && run <= target / 16 && run + sum > target / 16) {
+            uint32_t sixteenth = run;
+            for (int i = 0; i < 32; ++i) {
+                sixteenth += s_bin[tid * 32 + i];
+                if (sixteenth > target / 16) {
+                    A.h->lg_first = uint64_t(tid * 32 + i) << 48;
+                    break;
+                }
+            }
+        }
+        if (run <= target && run + sum > target) {
+            for (int i = 0; i < 32; ++i) {
+                const uint32_t c = s_bin[tid * 32 + i];
+                if (run + c > target) {
+                    s_at = uint32_t(tid * 32 + i);
+                    s_below = run;
+                    break;
+                }
+                run += c;
+            }
+        }
+        __syncthreads();
+        const uint32_t at = s_at;
+        if (level == 0) {
+            if (at == 32768) {
+                limit = kNone;  // fewer edges than wanted in all
+                break;
+            }
+            prefix = at;
+            target -= s_below;
+            limit = uint64_t(at) << 48;
+        } else if (at < 32768) {
+            limit |= uint64_t(at) << 33;
+        } else {
+            limit = (prefix + 1) << 48;
+        }
+        __syncthreads();
+    }
+    if (tid == 0) A.h->lg_limit = limit;
+}
+
+// ----------------------------------------------------- moving keys by hash ---
+// Tiles of eight keys per thread: a key's place among the tile's keys of
+// its partition by a shared-memory counter, the tile reordered there and
+// written out in runs.  The order within a partition is free.  LEVEL 0: all
+// keys to the partitions (with the list, and crowded tiles deduplicated); 1: a
+// partition's keys to its buckets.
+template <int LEVEL>
+__global__ void __launch_bounds__(kLgThreads, 2048 / kLgThreads) k_large_move(const LgArgs A) {
+    constexpr int kDig = LEVEL == 0 ? kLgParts : kLgMaxSub;
+    extern __shared__ __align__(16) unsigned char s_dyn[];
+    uint64_t *s_key = reinterpret_cast<uint64_t *>(s_dyn);          // [kLgTile]
+    uint32_t *s_cnt = reinterpret_cast<uint32_t *>(s_key + kLgTile);  // [kDig]
+    uint32_t *s_off = s_cnt + kDig, *s_to = s_off + kDig, *s_base = s_to + kDig;  // s_base: LEVEL 1
+    __shared__ uint32_t s_w[kLgThreads / 32 + 1], s_nrep, s_rbase, s_extra;
+    const int tid = threadIdx.x, lane = tid & 31;
+    int64_t begin = 0, end = A.m, first = blockIdx.x, step = gridDim.x;
+    const uint64_t *src = A.mat;
+    uint64_t *dst = A.part;
+    uint32_t *cursor = A.pcur;
+    int ndig = kLgParts;
+    const int p = blockIdx.x / kLgSubCtas;
+    if constexpr (LEVEL == 1) {
+        begin = A.poff[p];
+        end = A.pcur[p];
+        first = blockIdx.x % kLgSubCtas;
+        step = kLgSubCtas;
+        src = A.part;
+        dst = A.bkt;
+        ndig = A.nsub;
+        cursor = A.bcur + size_t(p) * ndig;
+        // the buckets' places
+        uint32_t total;
+        const uint32_t c = tid < ndig ? A.bcnt[size_t(p) * ndig + tid] : 0u;
+        const uint32_t run = uint32_t(begin) + block_scan<kLgThreads>(c, s_w, total);
+        if (tid < kDig) s_base[tid] = run;
+        if (tid < ndig && first == 0) A.boff[size_t(p) * ndig + tid] = run;
+    }
+    const uint64_t limit = LEVEL == 0 ? A.h->lg_limit : 0;
+    auto digit = [&](uint64_t k) { return LEVEL == 0 ? hash_part(part_hash(k)) : hash_sub(part_hash(k), ndig); };
+    for (int64_t t0 = begin + first * kLgTile; t0 < end; t0 += step * kLgTile) {
+        for (int i = tid; i < kDig; i += kLgThreads) s_cnt[i] = 0;
+        __syncthreads();
+        uint64_t key[kLgPer];
+        uint32_t place[kLgPer];  // (digit << 16) | place among the tile's keys of the digit
+#pragma unroll
+        for (int q = 0; q < kLgPer; ++q) {
+            const int64_t i = t0 + q * kLgThreads + tid;
+            key[q] = i < end ? __ldcs(src + i) : kNone;
+        }
+        bool crowded = false;
+#pragma unroll
+        for (int q = 0; q < kLgPer; ++q) {
+            place[q] = 0xffffffffu;
+            if (t0 + q * kLgThreads + tid >= end) continue;
+            const uint32_t dg = digit(key[q]), at = atomicAdd(s_cnt + dg, 1u);
+            place[q] = (dg << 16) | at;
+            crowded |= at >= kLgCrowd;
+        }
+        if constexpr (LEVEL == 0) {
+            // the list: one counter addition per warp
+            uint32_t mine = 0;
+#pragma unroll
+            for (int q = 0; q < kLgPer; ++q) mine += place[q] != 0xffffffffu && key[q] < limit;
+            if (__any_sync(0xffffffffu, mine != 0)) {
+                uint32_t at = mine;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const uint32_t y = __shfl_up_sync(0xffffffffu, at, o);
+                    if (lane >= o) at += y;
+                }
+                uint32_t base = 0;
+                if (lane == 31) base = atomicAdd(&A.h->lg_list, at);
+                at += __shfl_sync(0xffffffffu, base, 31) - mine;
+#pragma unroll
+                for (int q = 0; q < kLgPer; ++q) {
+                    if (place[q] == 0xffffffffu || key[q] >= limit) continue;
+                    if (at < A.lcap) {
+                        uint32_t u, v;
+                        edge_uv(t0 + q * kLgThreads + tid, A.n, u, v);
+                        A.lkey[at] = key[q];
+                        A.luv[at] = (u << 16) | v;
+                    }
+                    ++at;
+                }
+            }
+        }
+        const bool dedupe = __syncthreads_or(crowded);
+        if (LEVEL == 0 && dedupe) {
+            // one key of each distance stays; a table of half the tile's keys,
+            // at most eight probes (a key that finds no slot stays as it is)
+            constexpr int kSlots = kLgTile / 2;
+            unsigned long long *tab = reinterpret_cast<unsigned long long *>(s_key);
+            uint32_t *occ = reinterpret_cast<uint32_t *>(tab + kSlots);
+            for (int i = tid; i < kSlots; i += kLgThreads) {
+                tab[i] = 0;
+                occ[i] = 0;
+            }
+            for (int i = tid; i < kDig; i += kLgThreads) s_cnt[i] = 0;
+            if (tid == 0) s_nrep = s_extra = 0;
+            __syncthreads();
+            uint32_t stays = 0;
+            uint16_t at[kLgPer];
+#pragma unroll
+            for (int q = 0; q < kLgPer; ++q) {
+                at[q] = 0xffffu;
+                if (place[q] == 0xffffffffu) continue;
+                const unsigned long long tag = key[q] + 1;
+                uint32_t slot = uint32_t(key_hash(key[q])) & (kSlots - 1);
+                stays |= 1u << q;
+                for (int pr = 0; pr < 8; ++pr) {
+                    unsigned long long old = *(volatile unsigned long long *)(tab + slot);
+                    if (old == 0) old = atomicCAS(tab + slot, 0ull, tag);
+                    if (old == 0 || old == tag) {
+                        atomicAdd(occ + slot, 1u);
+                        if (old == 0) at[q] = uint16_t(slot);
+                        else stays &= ~(1u << q);
+                        break;
+                    }
+                    slot = (slot + 1) & (kSlots - 1);
+                }
+            }
+            __syncthreads();
+            uint32_t to[kLgPer], extra[kLgPer];
+#pragma unroll
+            for (int q = 0; q < kLgPer; ++q) {
+                extra[q] = 0;
+                if (!((stays >> q) & 1u)) {
+                    place[q] = 0xffffffffu;
+                    continue;
+                }
+                const uint32_t dg = digit(key[q]);
+                place[q] = (dg << 16) | atomicAdd(s_cnt + dg, 1u);
+                if (at[q] != 0xffffu) extra[q] = occ[at[q]] - 1;
+                if (extra[q]) {
+                    to[q] = atomicAdd(&s_nrep, 1u);
+                    atomicAdd(&s_extra, extra[q]);
+                }
+            }
+            __syncthreads();
+            if (tid == 0 && s_nrep) {
+                s_rbase = atomicAdd(&A.h->lg_reps, s_nrep);
+                atomicAdd(&A.h->direct_dups, s_extra);
+            }
+            __syncthreads();
+#pragma unroll
+            for (int q = 0; q < kLgPer; ++q)
+                if (extra[q]) A.rep[s_rbase + to[q]] = LgRepeat{key[q], extra[q], 0u};
+        }
+        // room for each digit's keys, their place within the tile
+        uint32_t total;
+        {
+            static_assert(kDig <= kLgThreads, "a thread per digit");
+            const uint32_t c = tid < kDig ? s_cnt[tid] : 0u;
+            uint32_t to = c ? atomicAdd(cursor + tid, c) : 0u;
+            if (LEVEL == 1 && tid < kDig) to += s_base[tid];
+            const uint32_t run = block_scan<kLgThreads>(c, s_w, total);
+            if (tid < kDig) {
+                s_off[tid] = run;
+                s_to[tid] = to - run;
+            }
+        }
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < kLgPer; ++q) {
+            if (place[q] == 0xffffffffu) continue;
+            s_key[s_off[place[q] >> 16] + (place[q] & 0xffffu)] = key[q];
+        }
+        __syncthreads();
+        for (uint32_t i = tid; i < total; i += kLgThreads) {
+            const uint64_t k = s_key[i];
+            dst[s_to[digit(k)] + i] = k;
+        }
+        __syncthreads();
+    }
+}
+
+size_t move_smem(int level) {
+    return size_t(kLgTile) * 8 + size_t(level == 0 ? kLgParts : kLgMaxSub) * 16;
+}
+
+// Keys per bucket of each partition.
+__global__ void __launch_bounds__(kLgThreads) k_large_sub(const LgArgs A) {
+    __shared__ uint32_t s_cnt[kLgMaxSub];
+    const int p = blockIdx.x / kLgSubCtas, tid = threadIdx.x;
+    for (int i = tid; i < A.nsub; i += kLgThreads) s_cnt[i] = 0;
+    __syncthreads();
+    const int64_t begin = A.poff[p], end = A.pcur[p];
+    constexpr int kU = 8;
+    for (int64_t i0 = begin + int64_t(blockIdx.x % kLgSubCtas) * kU * kLgThreads + tid; i0 < end;
+         i0 += int64_t(kLgSubCtas) * kU * kLgThreads) {
+        uint64_t key[kU];
+#pragma unroll
+        for (int q = 0; q < kU; ++q) key[q] = i0 + q * kLgThreads < end ? A.part[i0 + q * kLgThreads] : kNone;
+#pragma unroll
+        for (int q = 0; q < kU; ++q)
+            if (i0 + q * kLgThreads < end) atomicAdd(s_cnt + hash_sub(part_hash(key[q]), A.nsub), 1u);
+    }
+    __syncthreads();
+    for (int i = tid; i < A.nsub; i += kLgThreads)
+        if (s_cnt[i]) atomicAdd(A.bcnt + size_t(p) * A.nsub + i, s_cnt[i]);
+}
+
+// Repeated distances, a bucket at a time.  Few repeats: a bit table in shared
+// memory, one bit per key (10,240 keys set 1.6% of 655,360 bits); a key that
+// finds its bit set is a suspect, and a second look over the bucket's keys
+// picks out those that share a suspect's bit (about 160), which a small hash
+// table compares.  Where more than kLgSuspects are, a hash table of all keys
+// (32-bit slots: the key's place in the bucket and 18 bits of its hash, so an
+// occupied slot needs the key itself only when those agree); a bucket of more
+// than kLgPass keys in parts of kLgPart by another piece of the hash, with the
+// keys in the slots.  (The hash tables alone took 8.3 ps per key: a warp waits
+// for its lane with the most probes.)
+__global__ void __launch_bounds__(kLgRepThreads, 2) k_large_repeats(const LgArgs A) {
+    extern __shared__ __align__(16) unsigned char s_dyn[];
+    uint32_t *s_tab = reinterpret_cast<uint32_t *>(s_dyn);  // [kLgWords] bits, slots, or keys + 1 in half as many
+    __shared__ uint64_t s_key[kLgSusKeys];
+    __shared__ uint32_t s_sus[kLgSusSlots], s_ns, s_nk;
+    const int tid = threadIdx.x, np = A.n - 1;
+    const uint64_t top = A.skey[np - 1];
+    const bool two = A.nsub > 1;
+    const uint64_t *all = two ? A.bkt : A.part;
+    const int64_t buckets = int64_t(kLgParts) * A.nsub;
+    uint32_t dups = 0;
+    bool crowded = false;  // the last bucket was: likely the next one is too
+    constexpr int kU = 8;
+    auto again = [&](uint64_t key) {
+        ++dups;
+        if (key <= top) atomicAdd(A.dup + lg_place(A.skey, 0, np - 1, key), 1u);
+    };
+    auto clear = [&]() {
+        for (int i = tid; i < kLgWords / 4; i += kLgRepThreads) reinterpret_cast<uint4 *>(s_tab)[i] = make_uint4(0, 0, 0, 0);
+    };
+    auto bit_of = [](uint64_t x) { return __umulhi(uint32_t(x >> 24), uint32_t(kLgWords * 32)); };
+    for (int64_t b = blockIdx.x; b < buckets; b += gridDim.x) {
+        const uint32_t begin = two ? A.boff[b] : A.poff[b];
+        const uint32_t size = two ? A.bcur[b] : A.pcur[b] - begin;
+        const uint64_t *keys = all + begin;
+        if (size < 2) continue;
+        if (size <= uint32_t(kLgPass) && !crowded) {
+            clear();
+            for (int i = tid; i < kLgSusSlots; i += kLgRepThreads) s_sus[i] = 0;
+            if (tid == 0) s_ns = s_nk = 0;
+            __syncthreads();
+            for (uint32_t i0 = tid; i0 < size; i0 += kU * kLgRepThreads) {
+                uint64_t key[kU];
+#pragma unroll
+                for (int q = 0; q < kU; ++q) key[q] = i0 + q * kLgRepThreads < size ? keys[i0 + q * kLgRepThreads] : kNone;
+#pragma unroll
+                for (int q = 0; q < kU; ++q) {
+                    if (key[q] == kNone) continue;
+                    const uint32_t bit = bit_of(key_hash(key[q])), mask = 1u << (bit & 31);
+                    if (!(atomicOr(s_tab + (bit >> 5), mask) & mask)) continue;
+                    if (atomicAdd(&s_ns, 1u) >= kLgSuspects) continue;
+                    uint32_t slot = bit * 2654435761u >> 21;
+                    for (;;) {  // at most kLgSuspects of the slots fill
+                        const uint32_t old = atomicCAS(s_sus + slot, 0u, bit + 1);
+                        if (old == 0 || old == bit + 1) break;
+                        slot = (slot + 1) & (kLgSusSlots - 1);
+                    }
+                }
+            }
+            __syncthreads();
+            const uint32_t ns = s_ns;
+            __syncthreads();  // before s_ns is reset
+            if (ns == 0) continue;
+            crowded = ns > kLgSuspects;
+            if (!crowded) {
+                for (uint32_t i0 = tid; i0 < size; i0 += kU * kLgRepThreads) {
+                    uint64_t key[kU];
+#pragma unroll
+                    for (int q = 0; q < kU; ++q) key[q] = i0 + q * kLgRepThreads < size ? keys[i0 + q * kLgRepThreads] : kNone;
+#pragma unroll
+                    for (int q = 0; q < kU; ++q) {
+                        if (key[q] == kNone) continue;
+                        const uint32_t bit = bit_of(key_hash(key[q]));
+                        uint32_t slot = bit * 2654435761u >> 21, w;
+                        while ((w = s_sus[slot]) != 0 && w != bit + 1) slot = (slot + 1) & (kLgSusSlots - 1);
+                        if (w == 0) continue;
+                        const uint32_t at = atomicAdd(&s_nk, 1u);
+                        if (at < kLgSusKeys) s_key[at] = key[q];
+                    }
+                }
+                __syncthreads();
+                const uint32_t nk = s_nk;
+                crowded = nk > kLgSusKeys;
+                if (!crowded) {
+                    for (int i = tid; i < kLgSusSlots; i += kLgRepThreads) s_sus[i] = 0;
+                    __syncthreads();
+                    for (uint32_t i = tid; i < nk; i += kLgRepThreads) {
+                        const uint64_t key = s_key[i];
+                        uint32_t slot = uint32_t(key_hash(key)) & (kLgSusSlots - 1);
+                        for (;;) {  // at most kLgSusKeys of the slots fill
+                            const uint32_t old = atomicCAS(s_sus + slot, 0u, i + 1);
+                            if (old == 0) break;
+                            if (s_key[old - 1] == key) {
+                                again(key);
+                                break;
+                            }
+                            slot = (slot + 1) & (kLgSusSlots - 1);
+                        }
+                    }
+                    __syncthreads();
+                    continue;
+                }
+            }
+            __syncthreads();  // before the table is cleared again
+        }
+        if (size <= uint32_t(kLgPass)) {
+            clear();
+            __syncthreads();
+            uint32_t found = dups;
+            for (uint32_t i0 = tid; i0 < size; i0 += kU * kLgRepThreads) {
+                uint64_t key[kU];
+#pragma unroll
+                for (int q = 0; q < kU; ++q) key[q] = i0 + q * kLgRepThreads < size ? keys[i0 + q * kLgRepThreads] : kNone;
+#pragma unroll
+                for (int q = 0; q < kU; ++q) {
+                    if (key[q] == kNone) continue;
+                    const uint64_t x = key_hash(key[q]);
+                    const uint32_t print = uint32_t(x) << 14, word = print | (i0 + q * kLgRepThreads + 1);
+                    uint32_t slot = __umulhi(uint32_t(x) * 0x9E3779B9u, uint32_t(kLgWords));
+                    for (;;) {  // at most kLgPass of kLgWords fill: a free slot comes
+                        uint32_t old = *(volatile uint32_t *)(s_tab + slot);
+                        if (old == 0) old = atomicCAS(s_tab + slot, 0u, word);
+                        if (old == 0) break;
+                        if (((old ^ print) >> 14) == 0 && keys[(old & 16383u) - 1] == key[q]) {
+                            again(key[q]);
+                            break;
+                        }
+                        slot = slot + 1 == kLgWords ? 0 : slot + 1;
+                    }
+                }
+            }
+            // few after all: back to the bits
+            crowded = __syncthreads_count(dups != found) > kLgRepThreads / 4;
+            continue;
+        }
+        unsigned long long *tab = reinterpret_cast<unsigned long long *>(s_tab);
+        const uint32_t parts = (size + kLgPart - 1) / kLgPart;
+        for (uint32_t part = 0; part < parts; ++part) {
+            clear();
+            __syncthreads();
+            for (uint32_t i = tid; i < size; i += kLgRepThreads) {
+                const uint64_t key = keys[i], x = key_hash(key);
+                if (__umulhi(uint32_t(x) * 2654435761u, parts) != part) continue;
+                uint32_t slot = __umulhi(uint32_t(x) * 0x9E3779B9u, uint32_t(kLgWords / 2));
+                for (int pr = 0;; ++pr) {
+                    unsigned long long old = *(volatile unsigned long long *)(tab + slot);
+                    if (old == 0) old = atomicCAS(tab + slot, 0ull, (unsigned long long)(key + 1));
+                    if (old == 0) break;
+                    if (old == key + 1) {
+                        again(key);
+                        break;
+                    }
+                    slot = slot + 1 == kLgWords / 2 ? 0 : slot + 1;
+                    if (pr == kLgWords) {  // more distinct keys than slots: the hash does not spread them
+                        set_status(A.h, PH0_EINTERNAL);
+                        break;
+                    }
+                }
+            }
+            __syncthreads();
+        }
+    }
+    dups = __reduce_add_sync(0xffffffffu, dups);
+    if ((tid & 31) == 0 && dups) atomicAdd(&A.h->direct_dups, dups);
+}
+
+// ------------------------------------------------------------------ tree ---
+// The other component at component c's best edge.
+__device__ __forceinline__ uint32_t lg_other(const LgArgs &A, uint32_t c) {
+    const uint32_t uv = __ldcg(A.buv + c), a = __ldcg(A.comp + (uv >> 16)), b = __ldcg(A.comp + (uv & 0xffffu));
+    return a == c ? b : a;
+}
+
+__device__ __forceinline__ void lg_offer(const LgArgs &A, uint64_t key, uint32_t uv, uint32_t cu, uint32_t cv) {
+    if (key == __ldcg(A.best + cu)) atomicMin(A.buv + cu, uv);
+    if (key == __ldcg(A.best + cv)) atomicMin(A.buv + cv, uv);
+}
+
+// First row and column of 128 x 128 tile w of the upper triangle (T tiles a
+// side), row-major.
+__device__ __forceinline__ void lg_tile(int64_t w, int64_t T, int &u0, int &v0) {
+    const float b = float(2 * T + 1);
+    int64_t r = int64_t((b - sqrtf(b * b - 8.0f * float(w))) * 0.5f);
+    r = r < 0 ? 0 : r > T - 1 ? T - 1 : r;
+    while (r > 0 && r * T - r * (r - 1) / 2 > w) --r;
+    while (r < T - 1 && (r + 1) * T - (r + 1) * r / 2 <= w) ++r;
+    u0 = int(r) * 128;
+    v0 = int(r + w - (r * T - r * (r - 1) / 2)) * 128;
+}
+
+// Boruvka's rounds, a grid barrier between the steps of a round: every
+// component's smallest key leaving it; of the edges with that key the first
+// in (u, v); components hooked along them; components renamed.  Rounds on the
+// list come first: it holds every edge below the threshold, so the smallest
+// it has for a component is the smallest of all.  When it joins nothing more,
+// rounds on all keys: a warp reads 128 columns by 32 rows, four rows at a
+// time, against the best keys it knows of its rows' and columns' components;
+// only an edge that betters one is looked at further (a few in a thousand).
+__global__ void __launch_bounds__(kLgTreeThreads, 2) k_large_tree(const LgArgs A) {
+    __shared__ int s_ok;
+    const int n = A.n, tid = threadIdx.x, lane = tid & 31;
+    const int gthreads = gridDim.x * kLgTreeThreads, gtid = blockIdx.x * kLgTreeThreads + tid;
+    Header *h = A.h;
+    for (int v = gtid; v < n; v += gthreads) {
+        A.comp[v] = A.parent[v] = uint32_t(v);
+        A.best[v] = kNone;
+        A.buv[v] = 0xffffffffu;
+    }
+    if (!grid_barrier(h, &s_ok, A.spin_limit)) return;
+    const uint32_t listed = __ldcg(&h->lg_list), list = listed <= A.lcap ? listed : 0u;
+    uint32_t joined = 0, rounds = 0, passes = 0;
+    uint32_t live = uint32_t(gtid) < list ? (list - gtid - 1) / gthreads + 1 : 0u;  // entries of this thread
+    const uint64_t first = __ldcg(&h->lg_first);
+    bool on_list = list > 0;
+    const int64_t T = (n + 127) / 128, tiles = T * (T + 1) / 2;
+    const int warps = gthreads >> 5, gwarp = gtid >> 5;
+    while (joined < uint32_t(n - 1)) {
+        ++rounds;
+        if (on_list) {
+            // the shortest edges first: nearly every component has one among
+            // them, and what is left then betters few (all at once: the first
+            // round's two atomics per entry took most of the search)
+            for (uint32_t j = 0; j < live; j += 4) {
+                uint64_t k[4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) k[q] = j + q < live ? A.lkey[gtid + size_t(j + q) * gthreads] : kNone;
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    if (k[q] >= first) continue;
+                    const uint32_t uv = A.luv[gtid + size_t(j + q) * gthreads];
+                    const uint32_t cu = __ldcg(A.comp + (uv >> 16)), cv = __ldcg(A.comp + (uv & 0xffffu));
+                    if (cu == cv) continue;
+                    if (k[q] < __ldcg(A.best + cu)) atomicMin(A.best + cu, (unsigned long long)k[q]);
+                    if (k[q] < __ldcg(A.best + cv)) atomicMin(A.best + cv, (unsigned long long)k[q]);
+                }
+            }
+            if (!grid_barrier(h, &s_ok, A.spin_limit)) return;
+            // the others; a thread's entries, every gthreads-th, lose those
+            // within a component
+            const uint32_t had = live;
+            live = 0;
+            for (uint32_t j = 0; j < had; j += 4) {
+                uint64_t k[4], bu[4], bv[4];
+                uint32_t uv[4], cu[4], cv[4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const size_t i = gtid + size_t(j + q) * gthreads;
+                    uv[q] = j + q < had ? A.luv[i] : 0u;
+                    k[q] = j + q < had ? A.lkey[i] : kNone;
+                }
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    cu[q] = __ldcg(A.comp + (uv[q] >> 16));
+                    cv[q] = __ldcg(A.comp + (uv[q] & 0xffffu));
+                }
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    bu[q] = __ldcg(A.best + cu[q]);
+                    bv[q] = __ldcg(A.best + cv[q]);
+                }
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    if (cu[q] == cv[q]) continue;  // past the end too: an edge of vertex 0 with itself
+                    if (k[q] < bu[q]) atomicMin(A.best + cu[q], (unsigned long long)k[q]);
+                    if (k[q] < bv[q]) atomicMin(A.best + cv[q], (unsigned long long)k[q]);
+                    if (live < j + q) {
+                        const size_t i = gtid + size_t(live) * gthreads;
+                        A.luv[i] = uv[q];
+                        A.lkey[i] = k[q];
+                    }
+                    ++live;
+                }
+            }
+            if (!grid_barrier(h, &s_ok, A.spin_limit)) return;
+            for (uint32_t j = 0; j < live; j += 4) {
+                uint64_t k[4], bu[4], bv[4];
+                uint32_t uv[4], cu[4], cv[4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const size_t i = gtid + size_t(j + q) * gthreads;
+                    uv[q] = j + q < live ? A.luv[i] : 0u;
+                    k[q] = j + q < live ? A.lkey[i] : 0u;
+                }
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    cu[q] = __ldcg(A.comp + (uv[q] >> 16));
+                    cv[q] = __ldcg(A.comp + (uv[q] & 0xffffu));
+                }
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    bu[q] = __ldcg(A.best + cu[q]);
+                    bv[q] = __ldcg(A.best + cv[q]);
+                }
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    if (cu[q] == cv[q]) continue;
+                    if (k[q] == bu[q]) atomicMin(A.buv + cu[q], uv[q]);
+                    if (k[q] == bv[q]) atomicMin(A.buv + cv[q], uv[q]);
+                }
+            }
+        } else {
+            ++passes;
+            // first a sixteenth of the rows, for bounds that few edges better
+            // in the pass over all keys (without them nearly every row of the
+            // first tiles took the long way: 6.8 ms instead of 2.7 at 30,000
+            // points in eight clusters)
+            for (int64_t w = gwarp; w < tiles; w += warps) {
+                int u0, v0;
+                lg_tile(w, T, u0, v0);
+                uint32_t cv[4];
+                uint64_t mv[4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const int v = v0 + q * 32 + lane;
+                    cv[q] = v < n ? __ldcg(A.comp + v) : 0xffffffffu;
+                    mv[q] = kNone;
+                }
+                for (int i = 0; i < 8; i += 4) {
+                    uint64_t key[4][4];
+                    uint32_t cu[4];
+#pragma unroll
+                    for (int r = 0; r < 4; ++r) {
+                        const int u = u0 + (i + r) * 16 + int(w & 15);
+                        cu[r] = u < n ? __ldcg(A.comp + u) : 0xffffffffu;
+                    }
+#pragma unroll
+                    for (int r = 0; r < 4; ++r) {
+                        const int u = u0 + (i + r) * 16 + int(w & 15);
+                        const int64_t e0 = edge_index(n, u, 0);
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) {
+                            const int v = v0 + q * 32 + lane;
+                            key[r][q] = u < v && v < n && cu[r] != cv[q] ? __ldcg(A.mat + e0 + v) : kNone;
+                        }
+                    }
+#pragma unroll
+                    for (int r = 0; r < 4; ++r) {
+                        uint64_t mine = kNone;
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) {
+                            const uint64_t k = key[r][q];
+                            mv[q] = k < mv[q] ? k : mv[q];
+                            mine = k < mine ? k : mine;
+                        }
+                        const uint32_t mh = __reduce_min_sync(0xffffffffu, uint32_t(mine >> 32));
+                        const uint32_t ml =
+                            __reduce_min_sync(0xffffffffu, uint32_t(mine >> 32) == mh ? uint32_t(mine) : 0xffffffffu);
+                        const uint64_t mn = (uint64_t(mh) << 32) | ml;
+                        if (lane == r && mn != kNone && mn < __ldcg(A.best + cu[r]))
+                            atomicMin(A.best + cu[r], (unsigned long long)mn);
+                    }
+                }
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+                    if (mv[q] != kNone && mv[q] < __ldcg(A.best + cv[q])) atomicMin(A.best + cv[q], (unsigned long long)mv[q]);
+            }
+            if (!grid_barrier(h, &s_ok, A.spin_limit)) return;
+            for (int64_t w = gwarp; w < 4 * tiles; w += warps) {
+                int u0, v0;
+                lg_tile(w >> 2, T, u0, v0);
+                u0 += int(w & 3) * 32;
+                if (u0 >= n - 1 || u0 >= v0 + 127) continue;
+                // bounds: a key at or below what others found so far, then
+                // only keys below what this warp saw (its edges come in
+                // (u, v) order, so a later equal key is no better)
+                uint32_t cv[4];
+                uint64_t bv[4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const int v = v0 + q * 32 + lane;
+                    cv[q] = v < n ? __ldcg(A.comp + v) : 0xffffffffu;
+                    bv[q] = v < n ? __ldcg(A.best + cv[q]) : 0u;
+                    if (bv[q] != kNone && v < n) ++bv[q];
+                }
+                // rows and columns of one component have nothing to offer
+                const uint32_t c0 = __shfl_sync(0xffffffffu, cv[0], 0);
+                bool alike = true;
+#pragma unroll
+                for (int q = 0; q < 4; ++q) alike &= cv[q] == c0 || v0 + q * 32 + lane >= n;
+                alike = __all_sync(0xffffffffu, alike);
+                const int ul = u0 + lane;
+                const uint32_t cul = ul < n ? __ldcg(A.comp + ul) : 0xffffffffu;
+                uint64_t bul = ul < n ? __ldcg(A.best + cul) : 0u;
+                if (bul != kNone && ul < n) ++bul;
+                if (alike && __all_sync(0xffffffffu, cul == c0 || ul >= n)) continue;
+                // whole tiles off the diagonal need no look at u < v < n
+                const bool inner = u0 + 31 < v0 && v0 + 127 < n;
+                const uint64_t *line = A.mat + (edge_index(n, u0, 0) + v0 + lane);
+                for (int i0 = 0; i0 < 32; i0 += 4) {
+                    uint64_t key[4][4];
+#pragma unroll
+                    for (int r = 0; r < 4; ++r) {
+                        const int u = u0 + i0 + r;
+                        const uint32_t cu = __shfl_sync(0xffffffffu, cul, i0 + r);
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) {
+                            const int v = v0 + q * 32 + lane;
+                            key[r][q] = cu != cv[q] && (inner || (u < v && v < n)) ? __ldcs(line + q * 32) : kNone;
+                        }
+                        line += n - u - 2;
+                    }
+#pragma unroll
+                    for (int r = 0; r < 4; ++r) {
+                        // by the high words first: a pass over all keys is
+                        // bound by the instructions per key otherwise
+                        const uint32_t bh = __shfl_sync(0xffffffffu, uint32_t(bul >> 32), i0 + r);
+                        bool near = false;
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) {
+                            const uint32_t ch = uint32_t(bv[q] >> 32);
+                            near |= uint32_t(key[r][q] >> 32) <= (bh > ch ? bh : ch);
+                        }
+                        if (!__any_sync(0xffffffffu, near)) continue;
+                        const uint64_t bu = __shfl_sync(0xffffffffu, bul, i0 + r);
+                        bool hit = false;
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) hit |= key[r][q] < bu || key[r][q] < bv[q];
+                        if (!__any_sync(0xffffffffu, hit)) continue;
+                        const uint32_t cu = __shfl_sync(0xffffffffu, cul, i0 + r);
+                        const int64_t e0 = edge_index(n, u0 + i0 + r, 0) + v0 + lane;
+                        // the row's smallest key and the first edge that has it
+                        uint64_t mine = kNone;
+                        uint32_t at = 0xffffffffu;
+#pragma unroll
+                        for (int q = 0; q < 4; ++q)
+                            if (key[r][q] < mine) {
+                                mine = key[r][q];
+                                at = uint32_t(q * 32 + lane);
+                            }
+                        const uint32_t hi = uint32_t(mine >> 32), mh = __reduce_min_sync(0xffffffffu, hi);
+                        const uint32_t lo = hi == mh ? uint32_t(mine) : 0xffffffffu;
+                        const uint32_t ml = __reduce_min_sync(0xffffffffu, lo);
+                        const uint64_t mn = (uint64_t(mh) << 32) | ml;
+                        at = __reduce_min_sync(0xffffffffu, mine == mn ? at : 0xffffffffu);
+                        const bool row = mn < bu;
+                        if (row) {
+                            if (lane == 0) atomicMin(A.best + cu, (unsigned long long)mn);
+                            if (cul == cu && mn < bul) bul = mn;
+                        }
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) {
+                            const bool col = key[r][q] < bv[q];
+                            if (col) {
+                                bv[q] = key[r][q];
+                                atomicMin(A.best + cv[q], (unsigned long long)bv[q]);
+                            }
+                            const bool take = col || (row && at == uint32_t(q * 32 + lane));
+                            const unsigned who = __ballot_sync(0xffffffffu, take);
+                            if (!who) continue;
+                            uint32_t j = 0;
+                            if (lane == 0) j = atomicAdd(&h->lg_cand, uint32_t(__popc(who)));
+                            j = __shfl_sync(0xffffffffu, j, 0) + __popc(who & ((1u << lane) - 1u));
+                            if (take && j < A.ccap) A.cand[j] = uint32_t(e0 + q * 32);
+                        }
+                    }
+                }
+            }
+            if (!grid_barrier(h, &s_ok, A.spin_limit)) return;
+            const uint32_t cands = __ldcg(&h->lg_cand);
+            if (gtid == 0) h->lg_offers += cands;
+            const bool whole = cands > A.ccap;  // the list does not hold them all: every edge instead
+            const int64_t len = whole ? A.m : int64_t(cands);
+            for (int64_t i = gtid; i < len; i += gthreads) {
+                const int64_t e = whole ? i : int64_t(__ldcg(A.cand + i));
+                uint32_t u, v;
+                edge_uv(e, n, u, v);
+                const uint32_t cu = __ldcg(A.comp + u), cv = __ldcg(A.comp + v);
+                if (cu != cv) lg_offer(A, __ldcg(A.mat + e), (u << 16) | v, cu, cv);
+            }
+        }
+        if (!grid_barrier(h, &s_ok, A.spin_limit)) return;
+        // hook: of two components that chose the same edge the smaller stays
+        for (int c0 = gtid - lane; c0 < n; c0 += gthreads) {
+            const uint32_t c = uint32_t(c0 + lane);
+            bool take = false;
+            uint32_t o = 0;
+            if (c < uint32_t(n) && __ldcg(A.comp + c) == c && __ldcg(A.buv + c) != 0xffffffffu) {
+                o = lg_other(A, c);
+                take = !(__ldcg(A.buv + o) != 0xffffffffu && lg_other(A, o) == c && c < o);
+            }
+            const unsigned who = __ballot_sync(0xffffffffu, take);
+            if (!who) continue;
+            uint32_t j = 0;
+            if (lane == 0) j = atomicAdd(&h->lg_tree, uint32_t(__popc(who)));
+            j = __shfl_sync(0xffffffffu, j, 0) + __popc(who & ((1u << lane) - 1u));
+            if (take) {
+                A.parent[c] = o;
+                if (j < uint32_t(n)) {
+                    A.tkey[j] = __ldcg(A.best + c);
+                    A.tuv[j] = __ldcg(A.buv + c);
+                }
+            }
+        }
+        if (gtid == 0) h->lg_cand = 0;
+        if (!grid_barrier(h, &s_ok, A.spin_limit)) return;
+        for (int v = gtid; v < n; v += gthreads) {
+            uint32_t r = __ldcg(A.comp + v);
+            for (int i = 0;; ++i) {
+                const uint32_t p = __ldcg(A.parent + r);
+                if (p == r) break;
+                if (i > n) {  // a cycle: never, with one order of the edges
+                    set_status(h, PH0_EINTERNAL);
+                    break;
+                }
+                const uint32_t g = __ldcg(A.parent + p);
+                if (g != p) A.parent[r] = g;  // path halving (only moves toward the root)
+                r = g;
+            }
+            A.comp[v] = r;
+            A.best[v] = kNone;
+            A.buv[v] = 0xffffffffu;
+        }
+        const uint32_t now = __ldcg(&h->lg_tree);
+        if (!grid_barrier(h, &s_ok, A.spin_limit)) return;
+        if (now == joined) {
+            if (!on_list) {  // keys that are not numbers
+                if (gtid == 0) set_status(h, PH0_EINTERNAL);
+                break;
+            }
+            on_list = false;
+        }
+        joined = now;
+    }
+    if (gtid == 0) {
+        h->lg_rounds = rounds;
+        h->lg_passes = passes;
+    }
+}
+
+// The tree's edges in order: runs sorted by a CTA each (bitonic), then every
+// edge's place from binary searches in the other runs.
+__global__ void __launch_bounds__(1024) k_large_runs(const LgArgs A) {
+    __shared__ uint64_t s_k[kLgRun];
+    __shared__ uint32_t s_u[kLgRun];
+    const int base = blockIdx.x * kLgRun, tid = threadIdx.x;
+    const uint32_t have = A.h->lg_tree;
+    for (int i = tid; i < kLgRun; i += 1024) {
+        const uint32_t g = uint32_t(base + i);
+        const bool in = g < uint32_t(A.n - 1) && g < have;
+        s_k[i] = in ? A.tkey[g] : kNone;
+        s_u[i] = in ? A.tuv[g] : 0xffff0000u | (g & 0xffffu);  // missing after an error: no edge, all different
+    }
+    for (int kk = 2; kk <= kLgRun; kk <<= 1)
+        for (int j = kk >> 1; j > 0; j >>= 1) {
+            __syncthreads();
+            const int i = ((tid & ~(j - 1)) << 1) | (tid & (j - 1)), o = i | j;
+            const uint64_t a = s_k[i], b = s_k[o];
+            const uint32_t ua = s_u[i], ub = s_u[o];
+            if (lg_before(b, ub, a, ua) == ((i & kk) == 0)) {
+                s_k[i] = b;
+                s_k[o] = a;
+                s_u[i] = ub;
+                s_u[o] = ua;
+            }
+        }
+    __syncthreads();
+    for (int i = tid; i < kLgRun && base + i < A.n; i += 1024) {
+        A.tkey[base + i] = s_k[i];
+        A.tuv[base + i] = s_u[i];
+    }
+}
+
+// A warp per edge, a lane per run (at most 32 up to 65,535 points).
+__global__ void __launch_bounds__(256) k_large_merge(const LgArgs A) {
+    const int i = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31, np = A.n - 1;
+    if (i >= np) return;
+    const uint64_t k = A.tkey[i];
+    const uint32_t uv = A.tuv[i];
+    const int start = lane * kLgRun;
+    int lo = start, hi = start + kLgRun < np ? start + kLgRun : np;
+    if (lane == i / kLgRun) lo = hi = i;
+    while (lo < hi) {
+        const int mid = (lo + hi) >> 1;
+        if (lg_before(A.tkey[mid], A.tuv[mid], k, uv)) lo = mid + 1;
+        else hi = mid;
+    }
+    const int rank = __reduce_add_sync(0xffffffffu, start < np ? uint32_t(lo - start) : 0u);
+    if (lane == 0) {
+        A.skey[rank] = k;  // rank < np: places among np edges
+        A.suv[rank] = uv;
+    }
+}
+static_assert(32 * kLgRun >= kMaxN - 1, "a lane per run");
+
+// ---------------------------------------------------------- counts, bars ---
+// s(e), t(e), order and a as in k_direct.cu.  The counts of the kLgHot longest
+// tree edges, where nearly all edges up to the last one fall, are kept in
+// shared memory; the others go to the L2 cache.
+__global__ void __launch_bounds__(kLgCountThreads, 2) k_large_count(const LgArgs A) {
+    extern __shared__ __align__(16) unsigned char s_dyn[];
+    const int np = A.n - 1, hot = np < kLgHot ? np : kLgHot, base = np - hot, tid = threadIdx.x;
+    uint64_t *s_key = reinterpret_cast<uint64_t *>(s_dyn);      // [hot]
+    uint32_t *s_cnt = reinterpret_cast<uint32_t *>(s_key + hot);  // [hot]
+    // where to look: the first hot key at or beyond each of kLgLut steps of
+    // the way from the first to the last (a search over them all takes a warp
+    // with a few keys to place 13 steps: 3.0 ms instead of 1.15 at 30,000
+    // points in eight clusters, 450M keys)
+    __shared__ uint16_t s_lut[kLgLut + 2];
+    for (int i = tid; i < hot; i += kLgCountThreads) {
+        s_key[i] = A.skey[base + i];
+        s_cnt[i] = 0;
+    }
+    const int64_t gtid = int64_t(blockIdx.x) * kLgCountThreads + tid, gthreads = int64_t(gridDim.x) * kLgCountThreads;
+    for (int64_t j = gtid; j < np; j += gthreads) {
+        const unsigned long long p = A.kill_key[j];
+        if (p < (unsigned long long)np) A.low[p] = A.kill_val[j];
+    }
+    __syncthreads();
+    const uint64_t top = s_key[hot - 1], bottom = s_key[0];
+    int shift = bitlen64(top - bottom) - kLgLutBits;
+    if (shift < 0) shift = 0;
+    for (int i = tid; i < kLgLut + 2; i += kLgCountThreads) s_lut[i] = uint16_t(hot - 1);
+    __syncthreads();
+    for (int i = tid; i < hot; i += kLgCountThreads) {
+        const int b = int((s_key[i] - bottom) >> shift), a = i > 0 ? int((s_key[i - 1] - bottom) >> shift) : -1;
+        for (int j = a + 1; j <= b; ++j) s_lut[j] = uint16_t(i);
+    }
+    __syncthreads();
+    const uint32_t reps = A.h->lg_reps;
+    for (uint32_t q = uint32_t(gtid); q < reps; q += uint32_t(gthreads)) {
+        const LgRepeat r = A.rep[q];
+        if (r.key <= top) atomicAdd(A.dup + lg_place(A.skey, 0, np - 1, r.key), r.extra);
+    }
+    auto take = [&](uint64_t key, int64_t e) {
+        if (key > top) return;
+        int t;
+        bool tie;
+        if (key > bottom || base == 0) {
+            const int b = key > bottom ? int((key - bottom) >> shift) : 0;
+            const int i = lg_place(s_key, s_lut[b], s_lut[b + 1], key);
+            tie = s_key[i] == key;
+            t = base + i;
+            if (!tie) {
+                atomicAdd(s_cnt + i, 1u);
+                return;
+            }
+        } else {
+            t = lg_place(A.skey, 0, base, key);
+            tie = A.skey[t] == key;
+            if (!tie) {
+                atomicAdd(A.cnt + t, 1u);
+                return;
+            }
+        }
+        // as long as a tree edge: its place among them by (u, v)
+        uint32_t u, v;
+        edge_uv(e, A.n, u, v);
+        const uint32_t uv = (u << 16) | v;
+        int lo = t, hi = np;
+        while (lo < hi) {
+            const int mid = (lo + hi) >> 1;
+            if (lg_before(A.skey[mid], A.suv[mid], key, uv)) lo = mid + 1;
+            else hi = mid;
+        }
+        if (lo < np) atomicAdd(lo >= base ? s_cnt + (lo - base) : A.cnt + lo, 1u);
+        if (lo != t) {
+            atomicAdd(A.corr + t, 1u);
+            if (lo < np) atomicSub(A.corr + lo, 1u);
+        }
+    };
+    constexpr int kU = 8;
+    for (int64_t e0 = gtid; e0 < A.m; e0 += kU * gthreads) {
+        uint64_t key[kU];
+#pragma unroll
+        for (int q = 0; q < kU; ++q) key[q] = e0 + q * gthreads < A.m ? __ldcs(A.mat + e0 + q * gthreads) : kNone;
+#pragma unroll
+        for (int q = 0; q < kU; ++q) take(key[q], e0 + q * gthreads);
+    }
+    __syncthreads();
+    for (int i = tid; i < hot; i += kLgCountThreads)
+        if (s_cnt[i]) atomicAdd(A.cnt + base + i, s_cnt[i]);
+}
+
+// Each CTA adds up the counts before its 1024 tree edges, then writes their
+// bars; the last one to finish writes the bar that never dies.
+__global__ void __launch_bounds__(1024) k_large_emit(const LgArgs A) {
+    __shared__ uint32_t s_w[33], s_pre[2];
+    __shared__ int s_last;
+    const int tid = threadIdx.x, np = A.n - 1, base = blockIdx.x * 1024, p = base + tid;
+    if (tid < 2) s_pre[tid] = 0;
+    __syncthreads();
+    uint32_t so = 0, sa = 0;
+    for (int i = tid; i < base; i += 1024) {
+        const uint32_t c = A.cnt[i];
+        so += c;
+        sa += c + A.corr[i] - A.dup[i];
+    }
+    so = __reduce_add_sync(0xffffffffu, so);
+    sa = __reduce_add_sync(0xffffffffu, sa);
+    if ((tid & 31) == 0) {
+        atomicAdd(s_pre, so);
+        atomicAdd(s_pre + 1, sa);
+    }
+    __syncthreads();
+    const uint32_t c = p < np ? A.cnt[p] : 0u, a = p < np ? c + A.corr[p] - A.dup[p] : 0u;
+    uint32_t total;
+    const uint32_t order = s_pre[0] + block_scan<1024>(c, s_w, total) + c;
+    const uint32_t aval = s_pre[1] + block_scan<1024>(a, s_w, total) + a;
+    uint32_t low = 0;
+    if (p < np) {
+        const uint32_t uv = A.suv[p];
+        low = A.low[p];
+        ph0_bar b;
+        b.u = int32_t(uv >> 16);
+        b.v = int32_t(uv & 0xffffu);
+        b.a = aval;
+        b.low = int32_t(low);
+        b.order = int64_t(order) - 1;
+        b.death_sq = __longlong_as_double((long long)A.skey[p]);
+        b.death = __dsqrt_rn(b.death_sq);
+        A.bars[p] = b;
+    }
+    low = __reduce_xor_sync(0xffffffffu, low);
+    if ((tid & 31) == 0) atomicXor(&A.h->inf_xor, low);  // starts as the XOR of 0..n-1 (k_reduce_init)
+    __threadfence();
+    __syncthreads();
+    if (tid == 0) s_last = atomicAdd(&A.h->direct_done, 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!s_last || tid != 0) return;
+    __threadfence();
+    Header *h = A.h;
+    uint32_t v = ld_volatile(&h->inf_xor);
+    if (v >= uint32_t(A.n)) {  // only after a reported error
+        set_status(h, PH0_EINTERNAL);
+        v = 0;
+    }
+    h->inf_vertex = int32_t(v);
+    h->kmin = A.skey[0];
+    h->n_distinct = A.m - int64_t(h->direct_dups);
+    h->sort_passes = 0;
+    h->key_bits = make_plan(h->kmin, h->kmax).bits;
+    h->windows = int32_t(h->lg_rounds);
+    h->edges_scanned = A.m;
+    h->sorted_edges = A.m;
+    h->direct = 1;
+    if (A.inf) {
+        ph0_inf_bar b;
+        b.vertex = int32_t(v);
+        b._pad = 0;
+        b.birth = 0.0;
+        b.death = __longlong_as_double(0x7ff0000000000000ll);  // +inf
+        *A.inf = b;
+    }
+}
+
+int large_nsub(int64_t m) {
+    const int64_t per = (m + kLgParts - 1) / kLgParts;
+    if (per <= kLgBucket + kLgBucket / 4) return 1;
+    return int((per + kLgBucket - 1) / kLgBucket);
+}
+
+// The regions of this form within the sorts' (key, value and look-back
+// buffers, candidate lists) and the reduction's.
+LgArgs large_args(void *ws, const Layout &L, ph0_bar *bars, ph0_inf_bar *inf, uint32_t spin_limit, size_t &zero,
+                  size_t &zero_end) {
+    LgArgs A;
+    const size_t n = size_t(L.n);
+    A.m = L.m;
+    A.n = int(L.n);
+    A.nsub = large_nsub(L.m);
+    A.mat = at<uint64_t>(ws, L.key[0]);
+    A.part = at<uint64_t>(ws, L.key[1]);
+    A.bkt = at<uint64_t>(ws, L.val[0]);
+    A.rep = at<LgRepeat>(ws, L.val[0]);
+    const int64_t wcap = L.m < kMaxWindow ? L.m : kMaxWindow;
+    A.lkey = at<uint64_t>(ws, L.candr);
+    A.luv = at<uint32_t>(ws, L.cand[0]);
+    A.lcap = uint32_t(wcap < kLgListRoom * L.n ? wcap : kLgListRoom * L.n);  // above lg_samples
+    A.cand = at<uint32_t>(ws, L.cand[1]);
+    A.ccap = uint32_t(wcap);
+    A.comp = at<uint32_t>(ws, L.comp);
+    A.parent = at<uint32_t>(ws, L.parent);
+    A.best = at<unsigned long long>(ws, L.res);
+    A.tkey = at<uint64_t>(ws, L.kill_key[1]);
+    A.tuv = at<uint32_t>(ws, L.kill_val[1]);
+    A.kill_key = at<unsigned long long>(ws, L.kill_key[0]);
+    A.kill_val = at<uint32_t>(ws, L.kill_val[0]);
+    size_t off = L.look[0];
+    auto take = [&](size_t bytes) {
+        const size_t o = off;
+        off = align_up(off + bytes, 256);
+        return o;
+    };
+    const size_t nb = size_t(kLgParts) * size_t(A.nsub);
+    zero = off;
+    A.cnt = at<uint32_t>(ws, take(4 * n));
+    A.corr = at<uint32_t>(ws, take(4 * n));
+    A.dup = at<uint32_t>(ws, take(4 * n));
+    A.bcnt = at<uint32_t>(ws, take(4 * nb));
+    A.bcur = at<uint32_t>(ws, take(4 * nb));
+    zero_end = off;
+    A.boff = at<uint32_t>(ws, take(4 * nb));
+    A.poff = at<uint32_t>(ws, take(4 * (kLgParts + 1)));
+    A.pcur = at<uint32_t>(ws, take(4 * kLgParts));
+    A.buv = at<uint32_t>(ws, take(4 * n));
+    A.skey = at<uint64_t>(ws, take(8 * n));
+    A.suv = at<uint32_t>(ws, take(4 * n));
+    A.low = at<uint32_t>(ws, take(4 * n));
+    A.h = at<Header>(ws, L.hdr);
+    A.bars = bars;
+    A.inf = inf;
+    A.spin_limit = spin_limit;
+    // at least 8 * kMaxRadix bytes per 4096 edges, a byte per edge: the
+    // regions take 36 n bytes and 12 per 5632 edges
+    if (off > L.look[0] + 8 * size_t(L.tiles) * kMaxRadix) A.n = 0;
+    return A;
+}
+
+template <typename K>
+cudaError_t room(K kernel, size_t smem) {
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+}
+
+}  // namespace
+
+cudaError_t launch_dist(const float *pts, int64_t n, int32_t d, int64_t ld, uint64_t *key, uint32_t *val, Header *h,
+                        cudaStream_t s, int split16, int tile, const int32_t *gate, bool wide, DistForm form);
+
+// Up to the tree's edges in order: *records, n-1 of them ((u << 16) | v), for
+// the reduction.
+cudaError_t launch_large_tree(void *ws, const Layout &L, const float *pts, int64_t n, int32_t d, int64_t ld,
+                              int split16, int tile, uint32_t spin_limit, const uint32_t **records, cudaStream_t s,
+                              cudaEvent_t after_dist, cudaEvent_t after_part) {
+    size_t zero, zero_end;
+    const LgArgs A = large_args(ws, L, nullptr, nullptr, spin_limit, zero, zero_end);
+    if (A.n == 0) return cudaErrorInvalidValue;
+    *records = A.suv;
+    cudaError_t e = cudaMemsetAsync(at<char>(ws, L.hdr), 0, sizeof(Header), s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(at<char>(ws, zero), 0, zero_end - zero, s);
+    if (e == cudaSuccess)
+        e = launch_dist(pts, n, d, ld, at<uint64_t>(ws, L.key[0]), nullptr, A.h, s, split16, tile, nullptr, false,
+                        kDistHashed);
+    if (e == cudaSuccess && after_dist) e = cudaEventRecord(after_dist, s);
+    if (e == cudaSuccess) e = room(k_large_prep, 32768 * 4);
+    if (e != cudaSuccess) return e;
+    k_large_sample<<<unsigned((lg_samples(A.n) + 255) / 256), 256, 0, s>>>(A);  // into the list's place
+    k_large_prep<<<1, 1024, 32768 * 4, s>>>(A);
+    e = room(k_large_move<0>, move_smem(0));
+    if (e != cudaSuccess) return e;
+    const int64_t moves = (L.m + kLgTile - 1) / kLgTile;
+    const int ctas = 2 * sm_count(), mctas = 2048 / kLgThreads * sm_count();
+    k_large_move<0><<<unsigned(moves < mctas ? moves : mctas), kLgThreads, move_smem(0), s>>>(A);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    if (after_part && (e = cudaEventRecord(after_part, s)) != cudaSuccess) return e;
+
+    // fewer CTAs for small clouds (cheaper grid barriers): a warp per 128 columns by 32 rows
+    const int64_t T = (n + 127) / 128, want = (T * (T + 1) * 2 * 32 + kLgTreeThreads - 1) / kLgTreeThreads;
+    LgArgs args = A;
+    void *params[] = {&args};
+    e = cudaLaunchCooperativeKernel((const void *)k_large_tree, dim3(unsigned(want < ctas ? want : ctas)),
+                                    dim3(kLgTreeThreads), params, 0, s);
+    if (e != cudaSuccess) return e;
+    k_large_runs<<<unsigned((n - 1 + kLgRun - 1) / kLgRun), 1024, 0, s>>>(A);
+    k_large_merge<<<unsigned((n - 1 + 7) / 8), 256, 0, s>>>(A);
+    return cudaGetLastError();
+}
+
+// The rest, after the reduction of the tree's edges (its pivots in kill_key,
+// kill_val).
+cudaError_t launch_large_bars(void *ws, const Layout &L, int64_t n, ph0_bar *bars, ph0_inf_bar *inf, cudaStream_t s,
+                              cudaEvent_t after_counts) {
+    size_t zero, zero_end;
+    const LgArgs A = large_args(ws, L, bars, inf, 0, zero, zero_end);
+    const int ctas = 2 * sm_count();
+    const int hot = n - 1 < kLgHot ? int(n - 1) : kLgHot;
+    cudaError_t e = room(k_large_count, size_t(kLgHot) * 12);
+    if (e != cudaSuccess) return e;
+    const int64_t counts = (L.m + kLgCountThreads * 16 - 1) / (kLgCountThreads * 16);
+    k_large_count<<<unsigned(counts < ctas ? counts : ctas), kLgCountThreads, size_t(hot) * 12, s>>>(A);
+    if (A.nsub > 1) {
+        e = room(k_large_move<1>, move_smem(1));
+        if (e != cudaSuccess) return e;
+        k_large_sub<<<kLgParts * kLgSubCtas, kLgThreads, 0, s>>>(A);
+        k_large_move<1><<<kLgParts * kLgSubCtas, kLgThreads, move_smem(1), s>>>(A);
+    }
+    e = room(k_large_repeats, size_t(kLgWords) * 4);
+    if (e != cudaSuccess) return e;
+    k_large_repeats<<<unsigned(ctas), kLgRepThreads, size_t(kLgWords) * 4, s>>>(A);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    if (after_counts && (e = cudaEventRecord(after_counts, s)) != cudaSuccess) return e;
+    k_large_emit<<<unsigned((n - 1 + 1023) / 1024), 1024, 0, s>>>(A);
+    return cudaGetLastError();
+}
+
+}  // namespace ph0

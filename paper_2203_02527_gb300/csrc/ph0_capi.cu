@@ -18,7 +18,7 @@ namespace ph0 {
 
 cudaError_t launch_dist(const float *pts, int64_t n, int32_t d, int64_t ld, uint64_t *key,
                         uint32_t *val, Header *h, cudaStream_t s, int split16 = -1, int tile = -1,
-                        const int32_t *gate = nullptr, bool wide = false, bool packed = false);
+                        const int32_t *gate = nullptr, bool wide = false, DistForm form = kDistShort);
 cudaError_t launch_sort_init(Header *h, uint64_t *look0, int64_t tiles, cudaStream_t s,
                              int top_bits = kDefaultTopBits, int64_t sorted_edges = -1,
                              const int32_t *gate = nullptr);
@@ -73,6 +73,11 @@ cudaError_t launch_backward(const float *pts, int64_t n, int32_t d, int64_t ld, 
                             int64_t nb, const double *dl, float *grad, double *acc, cudaStream_t s);
 
 bool direct_applies(const Layout &L, int32_t d);
+cudaError_t launch_large_tree(void *ws, const Layout &L, const float *pts, int64_t n, int32_t d, int64_t ld,
+                              int split16, int tile, uint32_t spin_limit, const uint32_t **records, cudaStream_t s,
+                              cudaEvent_t after_dist = nullptr, cudaEvent_t after_part = nullptr);
+cudaError_t launch_large_bars(void *ws, const Layout &L, int64_t n, ph0_bar *bars, ph0_inf_bar *inf, cudaStream_t s,
+                              cudaEvent_t after_counts = nullptr);
 cudaError_t launch_direct(void *ws, const Layout &L, const float *pts, int64_t n, int32_t d, int64_t ld,
                           ph0_bar *bars, ph0_inf_bar *inf, cudaStream_t s, cudaEvent_t after_dist = nullptr,
                           cudaEvent_t after_tree = nullptr);
@@ -118,18 +123,21 @@ struct Tune {
     bool split = false;  // the whole path's sort as two merged halves (always above kSplitEdges edges)
     bool packed = false;  // the whole path's packed sort (k_sortp.cu)
     bool sortless = true;  // the whole path may leave the sort out (k_direct.cu): no form asked for
+    bool large = false;   // ... and does so by k_large.cu
     explicit Tune(const ph0_tuning *t, int64_t n = 0, int32_t d = 0) {
         const int64_t m = n_edges(n);
         wide = n > kMaxN;
         split = m > kSplitEdges;
         packed = m >= kPackMinEdges && n <= kPackMaxN && d >= kPackMinD;
+        large = n > kDirectMaxN && n <= kMaxN && (d < kPackMinD || m >= kLargeMinEdges);
         if (!t) return;
         if (t->wide_ids == 1) wide = true;
         if (t->split_sort == 1) split = true;
         sortless = t->wide_ids != 1 && t->split_sort != 1 && t->packed_sort != 0 && t->packed_sort != 1;
-        if (t->packed_sort == 0) packed = false;
-        if (t->packed_sort == 1) packed = m >= 1 && n <= kPackMaxN;
+        if (t->packed_sort == 0 || t->packed_sort == 2) packed = false;
+        if (t->packed_sort == 1 || t->packed_sort == 3) packed = m >= 1 && n <= kPackMaxN;
         if (split || wide) packed = false;  // its words take (u, v), not an edge index
+        large = large && sortless;
         if (t->dist_split16 >= 0 && t->dist_split16 <= 16) split16 = t->dist_split16;
         if (t->dist_tile == 32 || t->dist_tile == 64 || t->dist_tile == 128) tile = t->dist_tile;
         if (t->sort_top_bits == 8 || t->sort_top_bits == 9) top_bits = t->sort_top_bits;
@@ -305,6 +313,20 @@ cudaError_t run_reduce(void *ws, const Layout &L, int64_t n, int64_t m, const ui
     return launch_reduce(A, s);
 }
 
+// The whole path above kDirectMaxN points without a sort (k_large.cu): the
+// tree's edges in order, their columns' pivots, the counts and the bars.
+// ev: after the distances, the partition, the pivots, the counts; or null.
+cudaError_t run_large(void *ws, const Layout &L, const float *pts, int64_t n, int32_t d, int64_t ld, const Tune &t,
+                      ph0_bar *bars, ph0_inf_bar *inf, cudaStream_t s, const cudaEvent_t *ev = nullptr) {
+    const uint32_t *rec = nullptr;
+    cudaError_t e = launch_large_tree(ws, L, pts, n, d, ld, t.split16, t.tile, t.spin_limit, &rec, s,
+                                      ev ? ev[0] : nullptr, ev ? ev[1] : nullptr);
+    if (e == cudaSuccess) e = run_reduce(ws, L, n, n - 1, rec, rec, nullptr, s, t.spin_limit);
+    if (e == cudaSuccess && ev) e = cudaEventRecord(ev[2], s);
+    if (e == cudaSuccess) e = launch_large_bars(ws, L, n, bars, inf, s, ev ? ev[3] : nullptr);
+    return e;
+}
+
 // The read-out after run_reduce: order the n-1 pivot columns by position
 // (their discovery order within a window is not the filtration order) and
 // emit the bars, then the bar that never dies (inf may be null).  key as val;
@@ -419,9 +441,11 @@ int barcodes_whole(const float *pts_dev, int64_t n, int32_t d, int64_t ld, ph0_b
     uint32_t *cpref = at<uint32_t>(ws, L.cpref);
     if (t.sortless && direct_applies(L, d))
         return cuda_status(launch_direct(ws, L, pts_dev, n, d, ld, bars_dev, inf_dev, s));
+    if (t.large) return cuda_status(run_large(ws, L, pts_dev, n, d, ld, t, bars_dev, inf_dev, s));
     cudaError_t e = begin_call(ws, L, s, t.top_bits);
     if (e == cudaSuccess)
-        e = launch_dist(pts_dev, n, d, ld, k0, v0, h, s, t.split16, t.tile, nullptr, t.wide, t.packed);
+        e = launch_dist(pts_dev, n, d, ld, k0, v0, h, s, t.split16, t.tile, nullptr, t.wide,
+                        t.packed ? kDistPacked : kDistShort);
     if (t.packed) {
         if (e == cudaSuccess) e = sort_packed(ws, L, pts_dev, n, d, ld, t, s, fallback);
         if (e == cudaSuccess) e = launch_dedupe_scan(cpref, L.m, at<uint64_t>(ws, L.dlook), h, s);
@@ -682,9 +706,27 @@ int ph0_barcodes_profiled(const float *pts_dev, int64_t n, int32_t d, int64_t ld
         for (int i = 0; i < kEv; ++i) cudaEventDestroy(ev[i]);
         return cuda_status(e);
     }
+    if (t.large) {  // distances, partition, tree and pivots, counts, bars
+        const cudaEvent_t at[4] = {ev[1], ev[2], ev[3], ev[4]};
+        if (e == cudaSuccess) e = run_large(ws, L, pts_dev, n, d, ld, t, bars_dev, inf_dev, s, at);
+        if (e == cudaSuccess) e = cudaEventRecord(ev[5], s);
+        if (e == cudaSuccess) e = cudaEventSynchronize(ev[5]);
+        if (e == cudaSuccess) {
+            std::memset(prof, 0, sizeof(*prof));
+            cudaEventElapsedTime(&prof->total_ms, ev[0], ev[5]);
+            cudaEventElapsedTime(&prof->dist_ms, ev[0], ev[1]);
+            cudaEventElapsedTime(&prof->sort_ms, ev[1], ev[2]);
+            cudaEventElapsedTime(&prof->reduce_ms, ev[2], ev[3]);
+            cudaEventElapsedTime(&prof->dedupe_ms, ev[3], ev[4]);
+            cudaEventElapsedTime(&prof->emit_ms, ev[4], ev[5]);
+        }
+        for (int i = 0; i < kEv; ++i) cudaEventDestroy(ev[i]);
+        return cuda_status(e);
+    }
     if (e == cudaSuccess) e = begin_call(ws, L, s, t.top_bits);
     if (e == cudaSuccess)
-        e = launch_dist(pts_dev, n, d, ld, k0, v0, h, s, t.split16, t.tile, nullptr, t.wide, t.packed);
+        e = launch_dist(pts_dev, n, d, ld, k0, v0, h, s, t.split16, t.tile, nullptr, t.wide,
+                        t.packed ? kDistPacked : kDistShort);
     if (e == cudaSuccess) e = cudaEventRecord(ev[1], s);
     if (e == cudaSuccess && L.m > 0) e = prepare_sort_kernels();
     if (t.packed) {

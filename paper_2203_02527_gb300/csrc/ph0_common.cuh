@@ -88,6 +88,30 @@ __host__ __device__ __forceinline__ uint32_t pack_edge(uint64_t w, uint32_t n) {
 constexpr int64_t kDirectMaxN = 2896;
 constexpr int kDirectChunks = 32;
 
+// Above (k_large.cu): records (u << 16) | v, positions below 2^32.  Between
+// 2^22 and 2^24 edges in dimension 4 and up the packed sort stays.
+constexpr int64_t kLargeMinEdges = int64_t(1) << 24;
+
+// What the distance kernel writes and counts beside the keys: records and
+// the short sort's digit histograms, records and the packed sort's, or the
+// histogram of the keys' hash partitions alone (no records).
+enum DistForm { kDistShort = 0, kDistPacked = 1, kDistHashed = 2 };
+
+// Multiplicative (Fibonacci) hashing of a key.
+__device__ __forceinline__ uint64_t key_hash(uint64_t key) {
+    uint64_t x = key * 0x9E3779B97F4A7C15ull;
+    x ^= x >> 32;
+    return x * 0x9E3779B97F4A7C15ull;
+}
+// The high word of one such product, for the partitions and buckets of
+// k_large.cu: three multiplications, in kernels that are bound by such work.
+__device__ __forceinline__ uint32_t part_hash(uint64_t key) {
+    constexpr uint32_t kLo = 0x7F4A7C15u, kHi = 0x9E3779B9u;
+    const uint32_t lo = uint32_t(key), hi = uint32_t(key >> 32);
+    return __umulhi(lo, kLo) + lo * kHi + hi * kLo;
+}
+__device__ __forceinline__ uint32_t hash_part(uint32_t x) { return x >> 23; }
+
 // Bounded device-side waits: about a second at most, then the kernel records
 // PH0_ETIMEOUT in the status word and returns cleanly.
 constexpr uint32_t kSpinLimit = 1u << 24;
@@ -168,6 +192,19 @@ struct Header {
     uint32_t direct_repeats;     // and of the buckets after them)
     uint32_t direct_done;
     uint64_t direct_nkmin;
+    // ... above its sizes (k_large.cu): the list's threshold and length, edges
+    // that bettered a component's best, tree edges found, records of crowded
+    // tiles, rounds of the tree search
+    uint64_t lg_limit;
+    uint64_t lg_first;           // (about a sixteenth of the list lies below)
+    uint32_t lg_list;
+    uint32_t lg_cand;
+    uint32_t lg_tree;
+    uint32_t lg_reps;
+    uint32_t lg_rounds;
+    uint32_t lg_passes;          // (of them over all keys)
+    uint32_t lg_offers;          // (edges that bettered a component's best in these)
+    uint32_t lg_pad;
     // class partition of the early path (radix slot kClassSlot): the key
     // bins of its histogram and the classes' bin ranges [bound[c], bound[c+1])
     uint64_t part_kmin;

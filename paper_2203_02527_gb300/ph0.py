@@ -112,7 +112,11 @@ def _tuning(n: int, d: int, tuning):
         return tuning if isinstance(tuning, _lib.Tuning) else _lib.Tuning.make(**tuning)
     from . import autotune
     t = autotune.cached(d, n)
-    return _lib.Tuning.make(**t) if t else None
+    if not t:
+        return None
+    if "packed_sort" in t:  # the choice between the sorts, where the call sorts
+        t = {**t, "packed_sort": t["packed_sort"] + 2}
+    return _lib.Tuning.make(**t)
 
 
 def barcodes(pts: torch.Tensor, ws: Workspace | None = None, stats: bool = False,
