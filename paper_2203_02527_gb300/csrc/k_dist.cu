@@ -274,19 +274,24 @@ cudaError_t launch_dist(const float *pts, int64_t n, int32_t d, int64_t ld, uint
                                                            wide ? 1 : 0, int(form));
         return cudaGetLastError();
     };
-#define PH0_DIST_CASE(DD)                                       \
-    case DD:                                                    \
-        if (bt == 128) return go(k_dist<DD, 128>);              \
-        if (bt == 64) return go(k_dist<DD, 64>);                \
-        break;
-    switch (d) {
-        PH0_DIST_CASE(2)
-        PH0_DIST_CASE(3)
-        PH0_DIST_CASE(8)
-        PH0_DIST_CASE(16)
-        PH0_DIST_CASE(32)
-        default: break;
-    }
+    // every dimension to 32 has its instance for the default tile (unrolled
+    // groups at a run-time d took 4.94 ms instead of 3.86 for 450M edges at
+    // d = 5, 15.7 instead of 14.3 at d = 13)
+#define PH0_DIST_CASE(DD) \
+    case DD: return go(k_dist<DD, 128>);
+#define PH0_DIST_CASES(DD) PH0_DIST_CASE(DD) PH0_DIST_CASE(DD + 1) PH0_DIST_CASE(DD + 2) PH0_DIST_CASE(DD + 3)
+    if (bt == 128) switch (d) {
+            PH0_DIST_CASES(1)
+            PH0_DIST_CASES(5)
+            PH0_DIST_CASES(9)
+            PH0_DIST_CASES(13)
+            PH0_DIST_CASES(17)
+            PH0_DIST_CASES(21)
+            PH0_DIST_CASES(25)
+            PH0_DIST_CASES(29)
+            default: break;
+        }
+#undef PH0_DIST_CASES
 #undef PH0_DIST_CASE
     if (bt == 128) return go(k_dist<0, 128>);
     if (bt == 64) return go(k_dist<0, 64>);
