@@ -186,7 +186,7 @@ def h1(pts: torch.Tensor):
     bars = torch.empty((max(nb, 1), _lib.H1_BAR_BYTES), dtype=torch.uint8, device=pts.device)
     st = _lib.H1Stats()
     check(lib.ph0_h1(_ptr(pts), n, d, ld, _ptr(bars), _ptr(ws), nbytes, _stream(), ctypes.byref(st)), "ph0_h1")
-    out = bars[:nb].cpu().numpy().reshape(-1).view(_lib.H1_DTYPE).copy()
+    out = bars[:nb].cpu().numpy().reshape(-1).view(_lib.H1_DTYPE)  # host memory of its own
     return out, st.as_dict()
 
 
