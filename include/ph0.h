@@ -166,8 +166,10 @@ typedef struct {
                                points (test aid: runs the large-cloud form on any n);
                                -1 or 0: only above 65535 points                          */
     int32_t early_rounds;   /* ph0_barcodes_early_tuned: 1 always sorts the prefix in
-                               rounds, 0 never (the whole path); -1 built-in: rounds
-                               only for clouds of at least 2^27 edges (n >= 16385)     */
+                               rounds, 0 never (the whole path); -1 built-in: from 2^27
+                               edges on (n >= 16385) the form without a sort up to
+                               65535 points (step 3 only up to the last killing edge),
+                               rounds above                                            */
     int32_t split_sort;     /* 1: the whole path sorts the edges as two halves merged, as
                                it always does above 2^32 - 4096 edges (test aid: runs that
                                form on any n); -1 or 0: only above                       */

@@ -169,8 +169,8 @@ k_dist(const float *__restrict__ pts, int n, int d, int64_t ld, int bt, int hw16
         // points) rides in the key's bit 63, never set by a squared distance
         key[e] = wide ? kb | (uint64_t(e >> 32) << 63) : kb;
         kmax = kb > kmax ? kb : kmax;
-        if (form == kDistHashed) {  // the smallest key is the first tree edge's
-            atomicAdd(&s_flat[hash_part(part_hash(kb))], 1u);
+        if (form >= kDistHashed) {  // the smallest key is the first tree edge's
+            if (form == kDistHashed) atomicAdd(&s_flat[hash_part(part_hash(kb))], 1u);
             return;
         }
         kmin = kb < kmin ? kb : kmin;

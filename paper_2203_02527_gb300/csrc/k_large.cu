@@ -28,10 +28,10 @@
 // (u, v) throughout, so the results equal the sorted path's bit for bit.
 //
 // Measured (device time, 1.25G edges of 50,021 points in the plane; the short
-// sort's path 67.4 ms): k_dist 7.7 ms, k_large_move<0> 7.7, the tree and its
-// pivots 1.3, the count 1.8, k_large_sub 1.4, k_large_move<1> 5.8,
-// k_large_repeats 5.2: 31.1 ms.  32,768 points of four circles in 16
-// dimensions (537M edges): 26.9 ms (packed sort 34.4), of which the distances,
+// sort's path 67.4 ms): k_dist 5.9 ms, k_large_move<0> 7.0, the tree and its
+// pivots 1.2, the count 1.8, k_large_sub 1.4, k_large_move<1> 5.8,
+// k_large_repeats 5.2: 28.5 ms.  32,768 points of four circles in 16
+// dimensions (537M edges): 26.4 ms (packed sort 34.4), of which the distances,
 // bound by the binary64 adder, 15.6.  The count, k_large_sub and the tree's
 // passes run near the copy bandwidth; the moves are bound by shared-memory
 // wavefronts (60 to 66% of the peak) and their barriers.
@@ -100,6 +100,8 @@ struct LgArgs {
     uint32_t *poff, *pcur;     // [512 + 1], [512] places of the partitions, their ends
     uint32_t *bcnt, *bcur;     // [512][nsub] keys per bucket, filled
     uint32_t *boff;            // [512][nsub]
+    bool prefix;               // the early path: step 3 on the keys up to the last killing edge only,
+    uint64_t *keep;            //     [m] which the count puts here
     Header *h;
     ph0_bar *bars;
     ph0_inf_bar *inf;
@@ -168,21 +170,28 @@ __global__ void __launch_bounds__(256) k_large_sample(const LgArgs A) {
     for (uint32_t i = blockIdx.x * 256 + threadIdx.x; i < S; i += gridDim.x * 256)
         A.lkey[i] = A.mat[size_t(i) * step + __umulhi(i * 2654435761u, step)];
 }
+// The partitions' places from their histogram (1024 threads; s_w: 33 words).
+__device__ __forceinline__ void lg_places(const LgArgs &A, uint32_t *s_w) {
+    const int tid = threadIdx.x;
+    const uint32_t c = tid < kLgParts ? A.h->phist[0][tid] : 0u;
+    uint32_t total;
+    const uint32_t off = block_scan<1024>(c, s_w, total);
+    if (tid < kLgParts) {
+        A.poff[tid] = off;
+        A.pcur[tid] = off;
+    }
+    if (tid == 0) A.poff[kLgParts] = total;
+}
+__global__ void __launch_bounds__(1024) k_large_places(const LgArgs A) {
+    __shared__ uint32_t s_w[33];
+    lg_places(A, s_w);
+}
 __global__ void __launch_bounds__(1024) k_large_prep(const LgArgs A) {
     extern __shared__ uint32_t s_bin[];  // [32768]
     __shared__ uint32_t s_w[33];
     __shared__ uint32_t s_at, s_below;
     const int tid = threadIdx.x;
-    {
-        const uint32_t c = tid < kLgParts ? A.h->phist[0][tid] : 0u;
-        uint32_t total;
-        const uint32_t off = block_scan<1024>(c, s_w, total);
-        if (tid < kLgParts) {
-            A.poff[tid] = off;
-            A.pcur[tid] = off;
-        }
-        if (tid == 0) A.poff[kLgParts] = total;
-    }
+    lg_places(A, s_w);
     const int S = lg_samples(A.n);
     const double want = double(kLgListPerPoint) * double(A.n) * double(S) / double(A.m);
     uint64_t limit = 0;
@@ -246,6 +255,73 @@ __global__ void __launch_bounds__(1024) k_large_prep(const LgArgs A) {
     if (tid == 0) A.h->lg_limit = limit;
 }
 
+// A thread's place for the `mine` entries it appends, by one addition per
+// warp to the counter.  For the list the counter is the CTA's, in shared
+// memory; after a barrier one thread takes the CTA's room in the list with one
+// addition to the global counter (an addition per warp there: all the GPU's
+// warps on one word, about one a nanosecond, 0.93 ms to list 1.3M of 200M keys
+// instead of 0.52, and 0.7 of the 7.7 ms of k_large_move<0> on 1.25G).
+__device__ __forceinline__ uint32_t lg_rank(uint32_t mine, uint32_t *s_n) {
+    const int lane = threadIdx.x & 31;
+    if (!__any_sync(0xffffffffu, mine != 0)) return 0;
+    uint32_t at = mine;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, at, o);
+        if (lane >= o) at += y;
+    }
+    uint32_t base = 0;
+    if (lane == 31) base = atomicAdd(s_n, at);
+    return __shfl_sync(0xffffffffu, base, 31) + at - mine;
+}
+__device__ __forceinline__ void lg_room(uint32_t *counter, uint32_t *s_n, uint32_t *s_base) {
+    if (threadIdx.x == 0) {
+        if (*s_n) *s_base = atomicAdd(counter, *s_n);
+        *s_n = 0;
+    }
+}
+// The keys of a thread below the limit, with their edges, to the list from
+// place `at` on.  (kNone, past the end, is below no limit.)
+template <int N>
+__device__ __forceinline__ void lg_list_put(const LgArgs &A, const uint64_t (&key)[N], int64_t e0, int64_t step,
+                                            uint64_t limit, uint32_t at) {
+#pragma unroll
+    for (int q = 0; q < N; ++q) {
+        if (key[q] >= limit) continue;
+        if (at < A.lcap) {
+            uint32_t u, v;
+            edge_uv(e0 + q * step, A.n, u, v);
+            A.lkey[at] = key[q];
+            A.luv[at] = (u << 16) | v;
+        }
+        ++at;
+    }
+}
+
+// The list alone (the early path, whose keys are not all moved).
+__global__ void __launch_bounds__(1024, 2) k_large_list(const LgArgs A) {
+    __shared__ uint32_t s_n, s_base;
+    constexpr int kU = 8;
+    const uint64_t limit = A.h->lg_limit;
+    const int64_t stride = int64_t(gridDim.x) * 1024;
+    if (threadIdx.x == 0) s_n = 0;
+    __syncthreads();
+    for (int64_t b = int64_t(blockIdx.x) * 1024; b < A.m; b += kU * stride) {  // the same for a whole CTA
+        const int64_t e0 = b + threadIdx.x;
+        uint64_t key[kU];
+        uint32_t mine = 0;
+#pragma unroll
+        for (int q = 0; q < kU; ++q) key[q] = e0 + q * stride < A.m ? A.mat[e0 + q * stride] : kNone;
+#pragma unroll
+        for (int q = 0; q < kU; ++q) mine += key[q] < limit;
+        const uint32_t at = lg_rank(mine, &s_n);
+        __syncthreads();
+        lg_room(&A.h->lg_list, &s_n, &s_base);
+        __syncthreads();
+        if (mine) lg_list_put<kU>(A, key, e0, stride, limit, s_base + at);
+    }
+}
+
 // ----------------------------------------------------- moving keys by hash ---
 // Tiles of eight keys per thread: a key's place among the tile's keys of
 // its partition by a shared-memory counter, the tile reordered there and
@@ -259,10 +335,10 @@ __global__ void __launch_bounds__(kLgThreads, 2048 / kLgThreads) k_large_move(co
     uint64_t *s_key = reinterpret_cast<uint64_t *>(s_dyn);          // [kLgTile]
     uint32_t *s_cnt = reinterpret_cast<uint32_t *>(s_key + kLgTile);  // [kDig]
     uint32_t *s_off = s_cnt + kDig, *s_to = s_off + kDig, *s_base = s_to + kDig;  // s_base: LEVEL 1
-    __shared__ uint32_t s_w[kLgThreads / 32 + 1], s_nrep, s_rbase, s_extra;
-    const int tid = threadIdx.x, lane = tid & 31;
-    int64_t begin = 0, end = A.m, first = blockIdx.x, step = gridDim.x;
-    const uint64_t *src = A.mat;
+    __shared__ uint32_t s_w[kLgThreads / 32 + 1], s_nrep, s_rbase, s_extra, s_nlist, s_list;
+    const int tid = threadIdx.x;
+    int64_t begin = 0, end = A.prefix ? int64_t(A.h->lg_keep) : A.m, first = blockIdx.x, step = gridDim.x;
+    const uint64_t *src = A.prefix ? A.keep : A.mat;
     uint64_t *dst = A.part;
     uint32_t *cursor = A.pcur;
     int ndig = kLgParts;
@@ -283,7 +359,8 @@ __global__ void __launch_bounds__(kLgThreads, 2048 / kLgThreads) k_large_move(co
         if (tid < kDig) s_base[tid] = run;
         if (tid < ndig && first == 0) A.boff[size_t(p) * ndig + tid] = run;
     }
-    const uint64_t limit = LEVEL == 0 ? A.h->lg_limit : 0;
+    const uint64_t limit = LEVEL == 0 && !A.prefix ? A.h->lg_limit : 0;
+    if (tid == 0) s_nlist = 0;
     auto digit = [&](uint64_t k) { return LEVEL == 0 ? hash_part(part_hash(k)) : hash_sub(part_hash(k), ndig); };
     for (int64_t t0 = begin + first * kLgTile; t0 < end; t0 += step * kLgTile) {
         for (int i = tid; i < kDig; i += kLgThreads) s_cnt[i] = 0;
@@ -304,35 +381,14 @@ __global__ void __launch_bounds__(kLgThreads, 2048 / kLgThreads) k_large_move(co
             place[q] = (dg << 16) | at;
             crowded |= at >= kLgCrowd;
         }
+        uint32_t mine = 0, at = 0;  // for the list
         if constexpr (LEVEL == 0) {
-            // the list: one counter addition per warp
-            uint32_t mine = 0;
 #pragma unroll
-            for (int q = 0; q < kLgPer; ++q) mine += place[q] != 0xffffffffu && key[q] < limit;
-            if (__any_sync(0xffffffffu, mine != 0)) {
-                uint32_t at = mine;
-#pragma unroll
-                for (int o = 1; o < 32; o <<= 1) {
-                    const uint32_t y = __shfl_up_sync(0xffffffffu, at, o);
-                    if (lane >= o) at += y;
-                }
-                uint32_t base = 0;
-                if (lane == 31) base = atomicAdd(&A.h->lg_list, at);
-                at += __shfl_sync(0xffffffffu, base, 31) - mine;
-#pragma unroll
-                for (int q = 0; q < kLgPer; ++q) {
-                    if (place[q] == 0xffffffffu || key[q] >= limit) continue;
-                    if (at < A.lcap) {
-                        uint32_t u, v;
-                        edge_uv(t0 + q * kLgThreads + tid, A.n, u, v);
-                        A.lkey[at] = key[q];
-                        A.luv[at] = (u << 16) | v;
-                    }
-                    ++at;
-                }
-            }
+            for (int q = 0; q < kLgPer; ++q) mine += key[q] < limit;
+            at = lg_rank(mine, &s_nlist);
         }
         const bool dedupe = __syncthreads_or(crowded);
+        if (LEVEL == 0) lg_room(&A.h->lg_list, &s_nlist, &s_list);
         if (LEVEL == 0 && dedupe) {
             // one key of each distance stays; a table of half the tile's keys,
             // at most eight probes (a key that finds no slot stays as it is)
@@ -347,10 +403,10 @@ __global__ void __launch_bounds__(kLgThreads, 2048 / kLgThreads) k_large_move(co
             if (tid == 0) s_nrep = s_extra = 0;
             __syncthreads();
             uint32_t stays = 0;
-            uint16_t at[kLgPer];
+            uint16_t slot_of[kLgPer];
 #pragma unroll
             for (int q = 0; q < kLgPer; ++q) {
-                at[q] = 0xffffu;
+                slot_of[q] = 0xffffu;
                 if (place[q] == 0xffffffffu) continue;
                 const unsigned long long tag = key[q] + 1;
                 uint32_t slot = uint32_t(key_hash(key[q])) & (kSlots - 1);
@@ -360,7 +416,7 @@ __global__ void __launch_bounds__(kLgThreads, 2048 / kLgThreads) k_large_move(co
                     if (old == 0) old = atomicCAS(tab + slot, 0ull, tag);
                     if (old == 0 || old == tag) {
                         atomicAdd(occ + slot, 1u);
-                        if (old == 0) at[q] = uint16_t(slot);
+                        if (old == 0) slot_of[q] = uint16_t(slot);
                         else stays &= ~(1u << q);
                         break;
                     }
@@ -378,7 +434,7 @@ __global__ void __launch_bounds__(kLgThreads, 2048 / kLgThreads) k_large_move(co
                 }
                 const uint32_t dg = digit(key[q]);
                 place[q] = (dg << 16) | atomicAdd(s_cnt + dg, 1u);
-                if (at[q] != 0xffffu) extra[q] = occ[at[q]] - 1;
+                if (slot_of[q] != 0xffffu) extra[q] = occ[slot_of[q]] - 1;
                 if (extra[q]) {
                     to[q] = atomicAdd(&s_nrep, 1u);
                     atomicAdd(&s_extra, extra[q]);
@@ -408,6 +464,7 @@ __global__ void __launch_bounds__(kLgThreads, 2048 / kLgThreads) k_large_move(co
             }
         }
         __syncthreads();
+        if (LEVEL == 0 && mine) lg_list_put<kLgPer>(A, key, t0 + tid, kLgThreads, limit, s_list + at);
 #pragma unroll
         for (int q = 0; q < kLgPer; ++q) {
             if (place[q] == 0xffffffffu) continue;
@@ -448,6 +505,17 @@ __global__ void __launch_bounds__(kLgThreads) k_large_sub(const LgArgs A) {
         if (s_cnt[i]) atomicAdd(A.bcnt + size_t(p) * A.nsub + i, s_cnt[i]);
 }
 
+// The records of crowded tiles, at their places among the tree's edges.
+__device__ __forceinline__ void lg_reps(const LgArgs &A, uint32_t first, uint32_t step) {
+    const int np = A.n - 1;
+    const uint64_t top = A.skey[np - 1];
+    const uint32_t reps = A.h->lg_reps;
+    for (uint32_t q = first; q < reps; q += step) {
+        const LgRepeat r = A.rep[q];
+        if (r.key <= top) atomicAdd(A.dup + lg_place(A.skey, 0, np - 1, r.key), r.extra);
+    }
+}
+
 // Repeated distances, a bucket at a time.  Few repeats: a bit table in shared
 // memory, one bit per key (10,240 keys set 1.6% of 655,360 bits); a key that
 // finds its bit set is a suspect, and a second look over the bucket's keys
@@ -478,12 +546,37 @@ __global__ void __launch_bounds__(kLgRepThreads, 2) k_large_repeats(const LgArgs
     auto clear = [&]() {
         for (int i = tid; i < kLgWords / 4; i += kLgRepThreads) reinterpret_cast<uint4 *>(s_tab)[i] = make_uint4(0, 0, 0, 0);
     };
+    if (A.prefix) lg_reps(A, blockIdx.x * kLgRepThreads + tid, gridDim.x * kLgRepThreads);
+    // the repeats among the first nk of s_key (ends with a barrier)
+    auto compare = [&](uint32_t nk) {
+        for (int i = tid; i < kLgSusSlots; i += kLgRepThreads) s_sus[i] = 0;
+        __syncthreads();
+        for (uint32_t i = tid; i < nk; i += kLgRepThreads) {
+            const uint64_t key = s_key[i];
+            uint32_t slot = uint32_t(key_hash(key)) & (kLgSusSlots - 1);
+            for (;;) {  // at most kLgSusKeys of the slots fill
+                const uint32_t old = atomicCAS(s_sus + slot, 0u, i + 1);
+                if (old == 0) break;
+                if (s_key[old - 1] == key) {
+                    again(key);
+                    break;
+                }
+                slot = (slot + 1) & (kLgSusSlots - 1);
+            }
+        }
+        __syncthreads();
+    };
     auto bit_of = [](uint64_t x) { return __umulhi(uint32_t(x >> 24), uint32_t(kLgWords * 32)); };
     for (int64_t b = blockIdx.x; b < buckets; b += gridDim.x) {
         const uint32_t begin = two ? A.boff[b] : A.poff[b];
         const uint32_t size = two ? A.bcur[b] : A.pcur[b] - begin;
         const uint64_t *keys = all + begin;
         if (size < 2) continue;
+        if (size <= uint32_t(kLgSusKeys)) {  // few keys: compared at once
+            for (uint32_t i = tid; i < size; i += kLgRepThreads) s_key[i] = keys[i];
+            compare(size);
+            continue;
+        }
         if (size <= uint32_t(kLgPass) && !crowded) {
             clear();
             for (int i = tid; i < kLgSusSlots; i += kLgRepThreads) s_sus[i] = 0;
@@ -532,22 +625,7 @@ __global__ void __launch_bounds__(kLgRepThreads, 2) k_large_repeats(const LgArgs
                 const uint32_t nk = s_nk;
                 crowded = nk > kLgSusKeys;
                 if (!crowded) {
-                    for (int i = tid; i < kLgSusSlots; i += kLgRepThreads) s_sus[i] = 0;
-                    __syncthreads();
-                    for (uint32_t i = tid; i < nk; i += kLgRepThreads) {
-                        const uint64_t key = s_key[i];
-                        uint32_t slot = uint32_t(key_hash(key)) & (kLgSusSlots - 1);
-                        for (;;) {  // at most kLgSusKeys of the slots fill
-                            const uint32_t old = atomicCAS(s_sus + slot, 0u, i + 1);
-                            if (old == 0) break;
-                            if (s_key[old - 1] == key) {
-                                again(key);
-                                break;
-                            }
-                            slot = (slot + 1) & (kLgSusSlots - 1);
-                        }
-                    }
-                    __syncthreads();
+                    compare(nk);
                     continue;
                 }
             }
@@ -1036,8 +1114,14 @@ static_assert(32 * kLgRun >= kMaxN - 1, "a lane per run");
 // s(e), t(e), order and a as in k_direct.cu.  The counts of the kLgHot longest
 // tree edges, where nearly all edges up to the last one fall, are kept in
 // shared memory; the others go to the L2 cache.
+// PREFIX (the early path): the keys counted are also kept for step 3, with
+// the histogram of their partitions.
+template <bool PREFIX>
 __global__ void __launch_bounds__(kLgCountThreads, 2) k_large_count(const LgArgs A) {
     extern __shared__ __align__(16) unsigned char s_dyn[];
+    __shared__ uint32_t s_hist[PREFIX ? kLgParts : 1];
+    if constexpr (PREFIX)
+        for (int i = threadIdx.x; i < kLgParts; i += kLgCountThreads) s_hist[i] = 0;
     const int np = A.n - 1, hot = np < kLgHot ? np : kLgHot, base = np - hot, tid = threadIdx.x;
     uint64_t *s_key = reinterpret_cast<uint64_t *>(s_dyn);      // [hot]
     uint32_t *s_cnt = reinterpret_cast<uint32_t *>(s_key + hot);  // [hot]
@@ -1066,11 +1150,7 @@ __global__ void __launch_bounds__(kLgCountThreads, 2) k_large_count(const LgArgs
         for (int j = a + 1; j <= b; ++j) s_lut[j] = uint16_t(i);
     }
     __syncthreads();
-    const uint32_t reps = A.h->lg_reps;
-    for (uint32_t q = uint32_t(gtid); q < reps; q += uint32_t(gthreads)) {
-        const LgRepeat r = A.rep[q];
-        if (r.key <= top) atomicAdd(A.dup + lg_place(A.skey, 0, np - 1, r.key), r.extra);
-    }
+    if constexpr (!PREFIX) lg_reps(A, uint32_t(gtid), uint32_t(gthreads));
     auto take = [&](uint64_t key, int64_t e) {
         if (key > top) return;
         int t;
@@ -1109,14 +1189,34 @@ __global__ void __launch_bounds__(kLgCountThreads, 2) k_large_count(const LgArgs
         }
     };
     constexpr int kU = 8;
-    for (int64_t e0 = gtid; e0 < A.m; e0 += kU * gthreads) {
+    for (int64_t b = int64_t(blockIdx.x) * kLgCountThreads; b < A.m; b += kU * gthreads) {
+        const int64_t e0 = b + tid;
         uint64_t key[kU];
 #pragma unroll
         for (int q = 0; q < kU; ++q) key[q] = e0 + q * gthreads < A.m ? __ldcs(A.mat + e0 + q * gthreads) : kNone;
 #pragma unroll
         for (int q = 0; q < kU; ++q) take(key[q], e0 + q * gthreads);
+        if constexpr (PREFIX) {
+            uint32_t mine = 0;
+#pragma unroll
+            for (int q = 0; q < kU; ++q) mine += key[q] <= top;
+            // an addition per warp (of 20,011 uniform points few warps have
+            // any; one per CTA, with its barriers, took 0.93 ms instead of
+            // 0.38 there, and 2.9 instead of 3.1 where a third are kept)
+            if (!__any_sync(0xffffffffu, mine != 0)) continue;
+            uint32_t at = lg_rank(mine, &A.h->lg_keep);
+#pragma unroll
+            for (int q = 0; q < kU; ++q) {
+                if (key[q] > top) continue;
+                A.keep[at++] = key[q];
+                atomicAdd(s_hist + hash_part(part_hash(key[q])), 1u);
+            }
+        }
     }
     __syncthreads();
+    if constexpr (PREFIX)
+        for (int i = tid; i < kLgParts; i += kLgCountThreads)
+            if (s_hist[i]) atomicAdd(&A.h->phist[0][i], s_hist[i]);
     for (int i = tid; i < hot; i += kLgCountThreads)
         if (s_cnt[i]) atomicAdd(A.cnt + base + i, s_cnt[i]);
 }
@@ -1176,12 +1276,13 @@ __global__ void __launch_bounds__(1024) k_large_emit(const LgArgs A) {
     }
     h->inf_vertex = int32_t(v);
     h->kmin = A.skey[0];
-    h->n_distinct = A.m - int64_t(h->direct_dups);
+    const int64_t keys = A.prefix ? int64_t(h->lg_keep) : A.m;
+    h->n_distinct = keys - int64_t(h->direct_dups);
     h->sort_passes = 0;
     h->key_bits = make_plan(h->kmin, h->kmax).bits;
     h->windows = int32_t(h->lg_rounds);
     h->edges_scanned = A.m;
-    h->sorted_edges = A.m;
+    h->sorted_edges = keys;
     h->direct = 1;
     if (A.inf) {
         ph0_inf_bar b;
@@ -1201,17 +1302,22 @@ int large_nsub(int64_t m) {
 
 // The regions of this form within the sorts' (key, value and look-back
 // buffers, candidate lists) and the reduction's.
-LgArgs large_args(void *ws, const Layout &L, ph0_bar *bars, ph0_inf_bar *inf, uint32_t spin_limit, size_t &zero,
-                  size_t &zero_end) {
+LgArgs large_args(void *ws, const Layout &L, ph0_bar *bars, ph0_inf_bar *inf, uint32_t spin_limit, bool prefix,
+                  size_t &zero, size_t &zero_end) {
     LgArgs A;
     const size_t n = size_t(L.n);
     A.m = L.m;
     A.n = int(L.n);
     A.nsub = large_nsub(L.m);
     A.mat = at<uint64_t>(ws, L.key[0]);
-    A.part = at<uint64_t>(ws, L.key[1]);
-    A.bkt = at<uint64_t>(ws, L.val[0]);
-    A.rep = at<LgRepeat>(ws, L.val[0]);
+    // prefix: the kept keys in key[1], by partition in the value buffers, by
+    // bucket in key[1] again; the records in place of the keys by edge, which
+    // only the steps before read
+    A.prefix = prefix;
+    A.keep = at<uint64_t>(ws, L.key[1]);
+    A.part = at<uint64_t>(ws, prefix ? L.val[0] : L.key[1]);
+    A.bkt = at<uint64_t>(ws, prefix ? L.key[1] : L.val[0]);
+    A.rep = at<LgRepeat>(ws, prefix ? L.key[0] : L.val[0]);
     const int64_t wcap = L.m < kMaxWindow ? L.m : kMaxWindow;
     A.lkey = at<uint64_t>(ws, L.candr);
     A.luv = at<uint32_t>(ws, L.cand[0]);
@@ -1261,6 +1367,15 @@ cudaError_t room(K kernel, size_t smem) {
     return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
 }
 
+cudaError_t launch_parts(const LgArgs &A, cudaStream_t s) {
+    const cudaError_t e = room(k_large_move<0>, move_smem(0));
+    if (e != cudaSuccess) return e;
+    const int64_t moves = (A.m + kLgTile - 1) / kLgTile;
+    const int ctas = 2048 / kLgThreads * sm_count();
+    k_large_move<0><<<unsigned(moves < ctas ? moves : ctas), kLgThreads, move_smem(0), s>>>(A);
+    return cudaGetLastError();
+}
+
 }  // namespace
 
 cudaError_t launch_dist(const float *pts, int64_t n, int32_t d, int64_t ld, uint64_t *key, uint32_t *val, Header *h,
@@ -1269,27 +1384,25 @@ cudaError_t launch_dist(const float *pts, int64_t n, int32_t d, int64_t ld, uint
 // Up to the tree's edges in order: *records, n-1 of them ((u << 16) | v), for
 // the reduction.
 cudaError_t launch_large_tree(void *ws, const Layout &L, const float *pts, int64_t n, int32_t d, int64_t ld,
-                              int split16, int tile, uint32_t spin_limit, const uint32_t **records, cudaStream_t s,
-                              cudaEvent_t after_dist, cudaEvent_t after_part) {
+                              int split16, int tile, uint32_t spin_limit, bool prefix, const uint32_t **records,
+                              cudaStream_t s, cudaEvent_t after_dist, cudaEvent_t after_part) {
     size_t zero, zero_end;
-    const LgArgs A = large_args(ws, L, nullptr, nullptr, spin_limit, zero, zero_end);
+    const LgArgs A = large_args(ws, L, nullptr, nullptr, spin_limit, prefix, zero, zero_end);
     if (A.n == 0) return cudaErrorInvalidValue;
     *records = A.suv;
     cudaError_t e = cudaMemsetAsync(at<char>(ws, L.hdr), 0, sizeof(Header), s);
     if (e == cudaSuccess) e = cudaMemsetAsync(at<char>(ws, zero), 0, zero_end - zero, s);
     if (e == cudaSuccess)
         e = launch_dist(pts, n, d, ld, at<uint64_t>(ws, L.key[0]), nullptr, A.h, s, split16, tile, nullptr, false,
-                        kDistHashed);
+                        prefix ? kDistKeys : kDistHashed);
     if (e == cudaSuccess && after_dist) e = cudaEventRecord(after_dist, s);
     if (e == cudaSuccess) e = room(k_large_prep, 32768 * 4);
     if (e != cudaSuccess) return e;
     k_large_sample<<<unsigned((lg_samples(A.n) + 255) / 256), 256, 0, s>>>(A);  // into the list's place
     k_large_prep<<<1, 1024, 32768 * 4, s>>>(A);
-    e = room(k_large_move<0>, move_smem(0));
-    if (e != cudaSuccess) return e;
-    const int64_t moves = (L.m + kLgTile - 1) / kLgTile;
-    const int ctas = 2 * sm_count(), mctas = 2048 / kLgThreads * sm_count();
-    k_large_move<0><<<unsigned(moves < mctas ? moves : mctas), kLgThreads, move_smem(0), s>>>(A);
+    const int ctas = 2 * sm_count();
+    if (prefix) k_large_list<<<unsigned(ctas), 1024, 0, s>>>(A);
+    else if ((e = launch_parts(A, s)) != cudaSuccess) return e;
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if (after_part && (e = cudaEventRecord(after_part, s)) != cudaSuccess) return e;
 
@@ -1307,16 +1420,25 @@ cudaError_t launch_large_tree(void *ws, const Layout &L, const float *pts, int64
 
 // The rest, after the reduction of the tree's edges (its pivots in kill_key,
 // kill_val).
-cudaError_t launch_large_bars(void *ws, const Layout &L, int64_t n, ph0_bar *bars, ph0_inf_bar *inf, cudaStream_t s,
-                              cudaEvent_t after_counts) {
+cudaError_t launch_large_bars(void *ws, const Layout &L, int64_t n, ph0_bar *bars, ph0_inf_bar *inf, bool prefix,
+                              cudaStream_t s, cudaEvent_t after_counts) {
     size_t zero, zero_end;
-    const LgArgs A = large_args(ws, L, bars, inf, 0, zero, zero_end);
+    const LgArgs A = large_args(ws, L, bars, inf, 0, prefix, zero, zero_end);
     const int ctas = 2 * sm_count();
     const int hot = n - 1 < kLgHot ? int(n - 1) : kLgHot;
-    cudaError_t e = room(k_large_count, size_t(kLgHot) * 12);
-    if (e != cudaSuccess) return e;
     const int64_t counts = (L.m + kLgCountThreads * 16 - 1) / (kLgCountThreads * 16);
-    k_large_count<<<unsigned(counts < ctas ? counts : ctas), kLgCountThreads, size_t(hot) * 12, s>>>(A);
+    auto count = [&](auto kernel) {
+        const cudaError_t r = room(kernel, size_t(kLgHot) * 12);
+        if (r != cudaSuccess) return r;
+        kernel<<<unsigned(counts < ctas ? counts : ctas), kLgCountThreads, size_t(hot) * 12, s>>>(A);
+        return cudaGetLastError();
+    };
+    cudaError_t e = prefix ? count(k_large_count<true>) : count(k_large_count<false>);
+    if (e != cudaSuccess) return e;
+    if (prefix) {
+        k_large_places<<<1, 1024, 0, s>>>(A);
+        if ((e = launch_parts(A, s)) != cudaSuccess) return e;
+    }
     if (A.nsub > 1) {
         e = room(k_large_move<1>, move_smem(1));
         if (e != cudaSuccess) return e;

@@ -74,10 +74,10 @@ cudaError_t launch_backward(const float *pts, int64_t n, int32_t d, int64_t ld, 
 
 bool direct_applies(const Layout &L, int32_t d);
 cudaError_t launch_large_tree(void *ws, const Layout &L, const float *pts, int64_t n, int32_t d, int64_t ld,
-                              int split16, int tile, uint32_t spin_limit, const uint32_t **records, cudaStream_t s,
-                              cudaEvent_t after_dist = nullptr, cudaEvent_t after_part = nullptr);
-cudaError_t launch_large_bars(void *ws, const Layout &L, int64_t n, ph0_bar *bars, ph0_inf_bar *inf, cudaStream_t s,
-                              cudaEvent_t after_counts = nullptr);
+                              int split16, int tile, uint32_t spin_limit, bool prefix, const uint32_t **records,
+                              cudaStream_t s, cudaEvent_t after_dist = nullptr, cudaEvent_t after_part = nullptr);
+cudaError_t launch_large_bars(void *ws, const Layout &L, int64_t n, ph0_bar *bars, ph0_inf_bar *inf, bool prefix,
+                              cudaStream_t s, cudaEvent_t after_counts = nullptr);
 cudaError_t launch_direct(void *ws, const Layout &L, const float *pts, int64_t n, int32_t d, int64_t ld,
                           ph0_bar *bars, ph0_inf_bar *inf, cudaStream_t s, cudaEvent_t after_dist = nullptr,
                           cudaEvent_t after_tree = nullptr);
@@ -315,15 +315,17 @@ cudaError_t run_reduce(void *ws, const Layout &L, int64_t n, int64_t m, const ui
 
 // The whole path above kDirectMaxN points without a sort (k_large.cu): the
 // tree's edges in order, their columns' pivots, the counts and the bars.
-// ev: after the distances, the partition, the pivots, the counts; or null.
+// prefix: step 3 on the edges up to the last killing edge only (the early
+// path).  ev: after the distances, the partition, the pivots, the counts; or
+// null.
 cudaError_t run_large(void *ws, const Layout &L, const float *pts, int64_t n, int32_t d, int64_t ld, const Tune &t,
-                      ph0_bar *bars, ph0_inf_bar *inf, cudaStream_t s, const cudaEvent_t *ev = nullptr) {
+                      ph0_bar *bars, ph0_inf_bar *inf, bool prefix, cudaStream_t s, const cudaEvent_t *ev = nullptr) {
     const uint32_t *rec = nullptr;
-    cudaError_t e = launch_large_tree(ws, L, pts, n, d, ld, t.split16, t.tile, t.spin_limit, &rec, s,
+    cudaError_t e = launch_large_tree(ws, L, pts, n, d, ld, t.split16, t.tile, t.spin_limit, prefix, &rec, s,
                                       ev ? ev[0] : nullptr, ev ? ev[1] : nullptr);
     if (e == cudaSuccess) e = run_reduce(ws, L, n, n - 1, rec, rec, nullptr, s, t.spin_limit);
     if (e == cudaSuccess && ev) e = cudaEventRecord(ev[2], s);
-    if (e == cudaSuccess) e = launch_large_bars(ws, L, n, bars, inf, s, ev ? ev[3] : nullptr);
+    if (e == cudaSuccess) e = launch_large_bars(ws, L, n, bars, inf, prefix, s, ev ? ev[3] : nullptr);
     return e;
 }
 
@@ -441,7 +443,7 @@ int barcodes_whole(const float *pts_dev, int64_t n, int32_t d, int64_t ld, ph0_b
     uint32_t *cpref = at<uint32_t>(ws, L.cpref);
     if (t.sortless && direct_applies(L, d))
         return cuda_status(launch_direct(ws, L, pts_dev, n, d, ld, bars_dev, inf_dev, s));
-    if (t.large) return cuda_status(run_large(ws, L, pts_dev, n, d, ld, t, bars_dev, inf_dev, s));
+    if (t.large) return cuda_status(run_large(ws, L, pts_dev, n, d, ld, t, bars_dev, inf_dev, false, s));
     cudaError_t e = begin_call(ws, L, s, t.top_bits);
     if (e == cudaSuccess)
         e = launch_dist(pts_dev, n, d, ld, k0, v0, h, s, t.split16, t.tile, nullptr, t.wide,
@@ -512,7 +514,14 @@ int ph0_barcodes_early_tuned(const float *pts_dev, int64_t n, int32_t d, int64_t
     if (n < 3 || rounds == 0 || (rounds != 1 && L.m < kEarlyMinEdges)) return whole();
     // edge-index records above 65,535 points (or when a test asks for them);
     // the rounds never split the sort (E < 2^32 up to 92,681 points)
-    const Tune t(tuning, n);
+    const Tune t(tuning, n, d);
+    // the built-in choice leaves the sort out, and step 3's work beyond the
+    // last killing edge: no rounds (20,011 uniform points in space: 3.3 ms,
+    // 5.0 in rounds, 4.8 on the whole path)
+    if (rounds != 1 && t.large) {
+        const cudaError_t e = run_large(ws, L, pts_dev, n, d, ld, t, bars_dev, inf_dev, true, s);
+        return e != cudaSuccess ? PH0_ECUDA : ph0_finish(ws, stream, stats);
+    }
     const int64_t m = L.m;
     Header *h = at<Header>(ws, L.hdr);
     Header *sh = at<Header>(ws, L.aux_hdr);  // header of the segment sorts
@@ -708,7 +717,7 @@ int ph0_barcodes_profiled(const float *pts_dev, int64_t n, int32_t d, int64_t ld
     }
     if (t.large) {  // distances, partition, tree and pivots, counts, bars
         const cudaEvent_t at[4] = {ev[1], ev[2], ev[3], ev[4]};
-        if (e == cudaSuccess) e = run_large(ws, L, pts_dev, n, d, ld, t, bars_dev, inf_dev, s, at);
+        if (e == cudaSuccess) e = run_large(ws, L, pts_dev, n, d, ld, t, bars_dev, inf_dev, false, s, at);
         if (e == cudaSuccess) e = cudaEventRecord(ev[5], s);
         if (e == cudaSuccess) e = cudaEventSynchronize(ev[5]);
         if (e == cudaSuccess) {

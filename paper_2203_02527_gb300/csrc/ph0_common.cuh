@@ -94,8 +94,8 @@ constexpr int64_t kLargeMinEdges = int64_t(1) << 24;
 
 // What the distance kernel writes and counts beside the keys: records and
 // the short sort's digit histograms, records and the packed sort's, or the
-// histogram of the keys' hash partitions alone (no records).
-enum DistForm { kDistShort = 0, kDistPacked = 1, kDistHashed = 2 };
+// histogram of the keys' hash partitions alone (no records), or nothing.
+enum DistForm { kDistShort = 0, kDistPacked = 1, kDistHashed = 2, kDistKeys = 3 };
 
 // Multiplicative (Fibonacci) hashing of a key.
 __device__ __forceinline__ uint64_t key_hash(uint64_t key) {
@@ -204,7 +204,7 @@ struct Header {
     uint32_t lg_rounds;
     uint32_t lg_passes;          // (of them over all keys)
     uint32_t lg_offers;          // (edges that bettered a component's best in these)
-    uint32_t lg_pad;
+    uint32_t lg_keep;            // edges up to the last killing edge (the early path)
     // class partition of the early path (radix slot kClassSlot): the key
     // bins of its histogram and the classes' bin ranges [bound[c], bound[c+1])
     uint64_t part_kmin;

@@ -37,3 +37,27 @@ def test_clouds(name):
          "outliers": lambda: inputs.circles_with_outliers(1500, 4, 16, 4, seed=3504),
          "mixture": lambda: inputs.gaussian_mixture(6000, 3, k=8, sigma=0.05, center_range=10.0, seed=3505)}[name]()
     check(x)
+
+
+@pytest.mark.parametrize("name", ["uniform3", "line", "lattice", "mixture", "circles", "one_point"])
+def test_early_path_keeps_only_the_prefix(name):
+    """From 2^27 edges on the early path counts repeated distances only up to
+    the last killing edge: the whole path's bars, the prefix's length and its
+    number of distinct distances (the last bar's a, or more with ties)."""
+    import torch
+
+    from paper_2203_02527_gb300 import ph0
+    x = {"uniform3": lambda: inputs.uniform(16400, 3, seed=3601),
+         "line": lambda: inputs.uniform(16500, 1, seed=3602),
+         "lattice": lambda: inputs.lattice(26, 3),
+         "mixture": lambda: inputs.gaussian_mixture(16411, 5, k=8, sigma=0.05, center_range=10.0, seed=3603),
+         "circles": lambda: inputs.circles_with_outliers(4100, 4, 16, 3, seed=3604),
+         "one_point": lambda: np.full((16390, 2), 0.5, np.float32)}[name]()
+    pts = torch.from_numpy(np.ascontiguousarray(x)).cuda()
+    whole, early = ph0.barcodes(pts), ph0.barcodes_early(pts)
+    assert torch.equal(early.raw, whole.raw) and early.inf == whole.inf
+    bars, m = whole.numpy(), len(x) * (len(x) - 1) // 2
+    assert early.stats["sort_form"] == 3
+    assert int(bars["order"][-1]) < early.stats["sorted_edges"] <= m
+    assert early.stats["n_distinct"] == int(bars["a"][-1]) <= whole.stats["n_distinct"]
+    torch.cuda.empty_cache()
