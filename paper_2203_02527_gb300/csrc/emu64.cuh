@@ -139,6 +139,20 @@ __host__ __device__ __forceinline__ void bit_range_f32(uint32_t bits, int32_t &l
 #endif
 }
 
+// Unsigned integers in the order of the binary32 values.
+__host__ __device__ __forceinline__ uint32_t order_f32(uint32_t bits) {
+    return bits ^ (bits >> 31 ? 0xffffffffu : 0x80000000u);
+}
+#ifdef __CUDACC__
+// Whether values between the two (as order_f32) are less than 2^32 units of
+// 2^g apart (both multiples of the unit, fewer than 2^53 of it).
+__device__ __forceinline__ bool within_32_bits(uint32_t lo, uint32_t hi, int32_t g) {
+    if (lo > hi) return true;  // no values
+    auto value = [](uint32_t o) { return double(__uint_as_float(o ^ (o >> 31 ? 0x80000000u : 0xffffffffu))); };
+    return value(hi) - value(lo) < __longlong_as_double((long long)(g + 32 + 1023) << 52);
+}
+#endif
+
 // The integer X with x = X * 2^g (requires g <= lowest set bit of x and
 // |x| < 2^(g+63)).
 __host__ __device__ __forceinline__ int64_t to_fixed(uint32_t bits, int32_t g) {
@@ -179,7 +193,7 @@ __host__ __device__ __forceinline__ double to_double(F53 s) {
 #endif
 }
 
-// binary64 bit pattern of RN(t*t) for t = a * 2^g with 0 <= a < 2^31.  The
+// binary64 bit pattern of RN(t*t) for t = a * 2^g with 0 <= a < 2^32.  The
 // factor is normalized to bit 31 (one 32-bit count of leading zeros; of the
 // 64-bit product it would be two, and a 64-bit shift), so the exact square p
 // has its leading bit at 62 or 63; adding half of the last place kept less
@@ -214,12 +228,13 @@ __host__ __device__ __forceinline__ double bits_to_double(uint64_t b) {
 }
 
 // RN(t*t) as a binary64 value for t = xv - xu (fixed point in units of
-// 2^g); narrow: every |X| of the dimension is below 2^30, so t fits a 32-bit
-// signed difference of the low words.
+// 2^g); narrow: |t| is below 2^32 for all of the dimension's X, so the high
+// word of t is its sign.
 __host__ __device__ __forceinline__ double square_value(int64_t xu, int64_t xv, int32_t g, bool narrow) {
     if (narrow) {
-        const int32_t t = int32_t(uint32_t(xv)) - int32_t(uint32_t(xu));
-        return bits_to_double(square_bits_narrow(uint32_t(t < 0 ? -t : t), g));
+        const uint64_t t = uint64_t(xv) - uint64_t(xu);
+        const uint32_t sign = uint32_t(t >> 32);
+        return bits_to_double(square_bits_narrow((uint32_t(t) ^ sign) - sign, g));
     }
     const int64_t t = xv - xu;
     return to_double(square53(uint64_t(t < 0 ? -t : t), g));

@@ -28,7 +28,8 @@
 // (dist 15, tree 36, count 14; the short sort's path 480 us), 700 in 2 104 us
 // (470), 2048 in 3 195 us (62, 105, 29; 520), 2896 in 3 273 us (655).  The
 // steps are bound by latency: the tree by its rounds' exchanges and dependent
-// L2 reads.  kDirectMaxN is where the packed sort begins (2^22 edges).
+// L2 reads.  kDirectMaxN ends at 2^22 edges: above, the matrix outgrows the L2
+// cache and one cluster the tree's rounds, and k_large.cu takes over.
 #include <cooperative_groups.h>
 
 #include "emu64.cuh"
@@ -50,7 +51,7 @@ constexpr int kDirOwn = 3;                 // columns per thread of the claim ro
 constexpr int kDirClaimRounds = 64;        // then one thread finishes in order
 static_assert(kDirOwn * kDirMstThreads >= kDirectMaxN, "every column has a thread");
 constexpr uint64_t kNoKey = kKeyBits;      // above every squared distance
-constexpr size_t kDirDistSmem = 220 * 1024;
+constexpr size_t kDirDistSmem = 221 * 1024;
 constexpr size_t kDirMstSmem = 224 * 1024;  // beside the static words, below the 227 KB of a CTA
 
 struct DirectArgs {
@@ -125,8 +126,9 @@ __global__ void __launch_bounds__(kDirThreads) k_direct_dist(const DirectArgs A)
     uint64_t *s_colk = s_strip + kDirStrip * (bt + 1);                               // [bt]
     int32_t *s_g = reinterpret_cast<int32_t *>(s_colk + bt);
     int32_t *s_lo = s_g + d, *s_hi = s_lo + d;
-    uint32_t *s_narrow30 = reinterpret_cast<uint32_t *>(s_hi + d);  // [(d+31)/32]
-    uint16_t *s_colv = reinterpret_cast<uint16_t *>(s_narrow30 + (d + 31) / 32);  // [bt]
+    uint32_t *s_first = reinterpret_cast<uint32_t *>(s_hi + d), *s_last = s_first + d;
+    uint32_t *s_narrow = s_last + d;  // [(d+31)/32]
+    uint16_t *s_colv = reinterpret_cast<uint16_t *>(s_narrow + (d + 31) / 32);  // [bt]
     // a crowded strip's hash table of the places of its distinct keys, and
     // their occurrences (two 16-bit counts per word; bt is even)
     uint16_t *s_tab = s_colv + bt;                                                // [2 * 32 * bt]
@@ -147,6 +149,8 @@ __global__ void __launch_bounds__(kDirThreads) k_direct_dist(const DirectArgs A)
     for (int k = tid; k < d; k += kDirThreads) {
         s_lo[k] = 1 << 30;
         s_hi[k] = -(1 << 30);
+        s_first[k] = ~0u;
+        s_last[k] = 0;
     }
     for (int j = tid; j < bt; j += kDirThreads) s_colk[j] = kNoKey;
     // the trace of an earlier call's reduction (this form keeps one record)
@@ -163,11 +167,18 @@ __global__ void __launch_bounds__(kDirThreads) k_direct_dist(const DirectArgs A)
         const uint32_t b = __float_as_uint(x);
         if ((b & 0x7f800000u) == 0x7f800000u) {
             bad = true;
-        } else if (b & 0x7fffffffu) {
-            int32_t lo, hi;
-            emu::bit_range_f32(b, lo, hi);
-            atomicMin(s_lo + k, lo);
-            atomicMax(s_hi + k, hi);
+        } else {
+            if (row < n) {
+                const uint32_t o = emu::order_f32(b);
+                if (o < *(volatile uint32_t *)(s_first + k)) atomicMin(s_first + k, o);
+                if (o > *(volatile uint32_t *)(s_last + k)) atomicMax(s_last + k, o);
+            }
+            if (b & 0x7fffffffu) {
+                int32_t lo, hi;
+                emu::bit_range_f32(b, lo, hi);
+                if (lo < *(volatile int32_t *)(s_lo + k)) atomicMin(s_lo + k, lo);
+                if (hi > *(volatile int32_t *)(s_hi + k)) atomicMax(s_hi + k, hi);
+            }
         }
         (side ? xv : xu)[k * bt + p] = int64_t(b);
     }
@@ -183,10 +194,10 @@ __global__ void __launch_bounds__(kDirThreads) k_direct_dist(const DirectArgs A)
                 s_g[k] = zero ? 0 : s_lo[k];
                 const int span = zero ? 0 : s_hi[k] + 1 - s_lo[k];
                 if (span > 52) wide = true;
-                nar = span <= 30;
+                nar = span <= 52 && emu::within_32_bits(s_first[k], s_last[k], s_g[k]);
             }
             const unsigned bits = __ballot_sync(0xffffffffu, nar);
-            if (lane == 0) s_narrow30[w] = bits;
+            if (lane == 0) s_narrow[w] = bits;
         }
         wide = __any_sync(0xffffffffu, wide);
         if (lane == 0) {
@@ -207,7 +218,7 @@ __global__ void __launch_bounds__(kDirThreads) k_direct_dist(const DirectArgs A)
 
     const int j = tid % bt, v = v0 + j, rpp = kDirThreads / bt;
     const bool diag = bi == bj;
-    const uint32_t nw = s_narrow30[0];
+    const uint32_t nw = s_narrow[0];
     uint64_t kmin = ~0ull, kmax = 0;
     constexpr int kPer = kDirStrip * 128 / kDirThreads;  // keys per thread and strip, at most
     for (int s0 = 0; s0 < bt; s0 += kDirStrip) {
@@ -220,7 +231,7 @@ __global__ void __launch_bounds__(kDirThreads) k_direct_dist(const DirectArgs A)
             if (u < n && v < n && u != v) {
                 if (fixed) {
                     if constexpr (D > 0) kb = emu::sq_dist_mixed_ct<D, BT>(xu + i, xv + j, s_g, nw);
-                    else kb = emu::sq_dist_mixed_st<BT>(xu + i, xv + j, s_g, d, s_narrow30);
+                    else kb = emu::sq_dist_mixed_st<BT>(xu + i, xv + j, s_g, d, s_narrow);
                 } else {
                     double s = 0.0;
                     for (int k = 0; k < d; ++k) {
@@ -1001,7 +1012,7 @@ namespace {
 int direct_tile(int64_t n) { return n <= 32 * kDirectChunks ? 32 : n <= 64 * kDirectChunks ? 64 : 128; }
 
 size_t direct_dist_smem(int bt, int d) {
-    return size_t(2) * bt * d * 8 + size_t(kDirStrip) * (bt + 1) * 8 + size_t(bt) * 8 + size_t(3) * d * 4 +
+    return size_t(2) * bt * d * 8 + size_t(kDirStrip) * (bt + 1) * 8 + size_t(bt) * 8 + size_t(5) * d * 4 +
            size_t((d + 31) / 32) * 4 + size_t(bt) * 2 + size_t(6) * kDirStrip * bt;
 }
 
