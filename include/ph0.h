@@ -446,6 +446,33 @@ int ph0_barcodes_backward(const float *pts_dev, int64_t n, int32_t d,
                           const double *dl_ddeath_dev, float *grad_dev,
                           void *ws, size_t ws_bytes, void *stream);
 
+/* ---- many clouds at once ---- */
+
+/* One cloud of ph0_barcodes_many() and ph0_backward_many(): the arguments of
+ * ph0_barcodes_tuned() (tuning may be NULL) and, for the backward,
+ * dl_ddeath_dev and grad_dev of ph0_barcodes_backward() with its n-1 bars. */
+typedef struct {
+    const float *pts_dev;
+    int64_t n, ld;
+    int32_t d, _pad;
+    ph0_bar *bars_dev;
+    ph0_inf_bar *inf_dev;
+    void *ws;                   /* each cloud's own: clouds run at the same time */
+    size_t ws_bytes;
+    const ph0_tuning *tuning;
+    const double *dl_ddeath_dev;
+    float *grad_dev;
+} ph0_cloud;
+
+/* ph0_barcodes_tuned() of `count` clouds, cloud i on streams[i % n_streams]
+ * (queued by one call: a host loop over separate calls takes longer than the
+ * GPU does for small clouds).  Returns the first error of a call; the clouds
+ * before it are queued. */
+int ph0_barcodes_many(const ph0_cloud *clouds, int64_t count, void *const *streams, int32_t n_streams);
+
+/* ph0_barcodes_backward() of the same clouds, likewise. */
+int ph0_backward_many(const ph0_cloud *clouds, int64_t count, void *const *streams, int32_t n_streams);
+
 #ifdef __cplusplus
 }
 #endif

@@ -121,6 +121,14 @@ class InfBar(ctypes.Structure):
 INF_BAR_BYTES = ctypes.sizeof(InfBar)  # 24
 
 
+class Cloud(ctypes.Structure):
+    _fields_ = [("pts_dev", ctypes.c_void_p), ("n", ctypes.c_int64), ("ld", ctypes.c_int64),
+                ("d", ctypes.c_int32), ("_pad", ctypes.c_int32), ("bars_dev", ctypes.c_void_p),
+                ("inf_dev", ctypes.c_void_p), ("ws", ctypes.c_void_p), ("ws_bytes", ctypes.c_size_t),
+                ("tuning", ctypes.POINTER(Tuning)), ("dl_ddeath_dev", ctypes.c_void_p),
+                ("grad_dev", ctypes.c_void_p)]
+
+
 class Result(ctypes.Structure):
     _fields_ = [
         ("tag", ctypes.c_uint64), ("status", ctypes.c_int32), ("n", ctypes.c_int32),
@@ -163,6 +171,8 @@ SIGNATURES = {
     "ph0_reduce": (ctypes.c_int, [_I64, _VP, _VP, _VP, _VP, _VP, _SZ, _VP]),
     "ph0_barcodes_backward": (ctypes.c_int, [_VP, _I64, _I32, _I64, _VP, _I64, _VP, _VP,
                                              _VP, _SZ, _VP]),
+    "ph0_barcodes_many": (ctypes.c_int, [ctypes.POINTER(Cloud), _I64, ctypes.POINTER(_VP), _I32]),
+    "ph0_backward_many": (ctypes.c_int, [ctypes.POINTER(Cloud), _I64, ctypes.POINTER(_VP), _I32]),
     "ph0_h1_workspace_bytes": (_SZ, [_I64, _I32]),
     "ph0_h1": (ctypes.c_int, [_VP, _I64, _I32, _I64, _VP, _VP, _SZ, _VP, ctypes.POINTER(H1Stats)]),
 }

@@ -912,6 +912,28 @@ int ph0_barcodes_backward(const float *pts_dev, int64_t n, int32_t d, int64_t ld
                                        at<double>(ws, L.grad), s));
 }
 
+int ph0_barcodes_many(const ph0_cloud *clouds, int64_t count, void *const *streams, int32_t n_streams) {
+    if (count < 0 || n_streams < 1 || !streams || (count > 0 && !clouds)) return PH0_EINVAL;
+    for (int64_t i = 0; i < count; ++i) {
+        const ph0_cloud &c = clouds[i];
+        const int rc = ph0_barcodes_tuned(c.pts_dev, c.n, c.d, c.ld, c.bars_dev, c.inf_dev, c.ws, c.ws_bytes,
+                                          streams[i % n_streams], c.tuning);
+        if (rc != PH0_OK) return rc;
+    }
+    return PH0_OK;
+}
+
+int ph0_backward_many(const ph0_cloud *clouds, int64_t count, void *const *streams, int32_t n_streams) {
+    if (count < 0 || n_streams < 1 || !streams || (count > 0 && !clouds)) return PH0_EINVAL;
+    for (int64_t i = 0; i < count; ++i) {
+        const ph0_cloud &c = clouds[i];
+        const int rc = ph0_barcodes_backward(c.pts_dev, c.n, c.d, c.ld, c.bars_dev, c.n - 1, c.dl_ddeath_dev,
+                                             c.grad_dev, c.ws, c.ws_bytes, streams[i % n_streams]);
+        if (rc != PH0_OK) return rc;
+    }
+    return PH0_OK;
+}
+
 size_t ph0_h1_workspace_bytes(int64_t n, int32_t d) {
     if (check_sizes(n, d, d, kH1MaxN) != PH0_OK) return 0;
     const Layout L(n, d);

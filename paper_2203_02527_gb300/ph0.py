@@ -318,38 +318,70 @@ class DeathValuesBatch(torch.autograd.Function):
     @staticmethod
     def forward(ctx, workspaces, streams, *pts):
         cur = torch.cuda.current_stream()
-        bars = []
-        for i, p in enumerate(pts):
-            s = streams[i % len(streams)]
-            s.wait_stream(cur)
-            with torch.cuda.stream(s):
-                bars.append(barcodes(p, workspaces[i], sync=False))
-        if not torch.cuda.is_current_stream_capturing():
-            for i, ws in enumerate(workspaces[:len(pts)]):
-                with torch.cuda.stream(streams[i % len(streams)]):
-                    finish(ws)  # waits for that stream; raises on a device error
-        for s in streams:
-            cur.wait_stream(s)
-        out = [b.death for b in bars]  # on the current stream, after every cloud finished
+        shaped = [_points(p) for p in pts]  # a copy where the rows need one
+        sizes = [max(n - 1, 0) for _, n, _, _ in shaped]
+        device = pts[0].device if pts else None
+        # every buffer is made on the current stream, which the others follow
+        # and which waits for them below
+        raw = torch.empty((sum(sizes), BAR_BYTES), dtype=torch.uint8, device=device)
+        inf = torch.empty((len(pts), _lib.INF_BAR_BYTES), dtype=torch.uint8, device=device)
+        clouds = (_lib.Cloud * len(pts))()
+        tunings, at = [], 0
+        for i, (p, n, d, ld) in enumerate(shaped):
+            c, ws = clouds[i], workspaces[i]
+            c.pts_dev, c.n, c.ld, c.d = p.data_ptr(), n, ld, d
+            c.bars_dev = raw.data_ptr() + at * BAR_BYTES
+            c.inf_dev = inf.data_ptr() + i * _lib.INF_BAR_BYTES
+            c.ws, c.ws_bytes = ws.buf.data_ptr(), ws.nbytes
+            t = _tuning(n, d, None)
+            if t is not None:
+                tunings.append(t)  # kept until the call is made
+                c.tuning = ctypes.pointer(t)
+            at += sizes[i]
+        _many(_lib.load().ph0_barcodes_many, "ph0_barcodes", clouds, streams, cur)
+        if pts and not torch.cuda.is_current_stream_capturing():
+            for st in statuses(workspaces[:len(pts)]):  # waits for the current stream
+                check(int(st), "device status")
+        off, size, dt = _FIELDS["death"]
+        deaths = raw[:, off:off + size].contiguous().view(dt).reshape(at)
         ctx.save_for_backward(*pts)
-        ctx.bars, ctx.workspaces, ctx.streams = bars, workspaces, streams
-        return tuple(out)
+        ctx.raw, ctx.sizes, ctx.workspaces, ctx.streams = raw, sizes, workspaces, streams
+        return tuple(torch.split_with_sizes_copy(deaths, sizes))
 
     @staticmethod
     def backward(ctx, *grads):
-        pts = ctx.saved_tensors
         cur = torch.cuda.current_stream()
-        out = []
-        for i, (p, g) in enumerate(zip(pts, grads)):
-            s = ctx.streams[i % len(ctx.streams)]
-            s.wait_stream(cur)
-            with torch.cuda.stream(s):
-                gp = backward(p, ctx.bars[i], g.contiguous(), ctx.workspaces[i])
-            gp.record_stream(cur)  # made on s, used on the current stream
+        clouds = (_lib.Cloud * len(grads))()
+        keep, out, at = [], [], 0
+        for i, (p, g) in enumerate(zip(ctx.saved_tensors, grads)):
+            p, n, d, ld = _points(p)
+            g = g.to(dtype=torch.float64).contiguous()
+            gp = torch.empty((n, d), dtype=torch.float32, device=p.device)
+            c, ws = clouds[i], ctx.workspaces[i]
+            c.pts_dev, c.n, c.ld, c.d = p.data_ptr(), n, ld, d
+            c.bars_dev = ctx.raw.data_ptr() + at * BAR_BYTES
+            c.ws, c.ws_bytes = ws.buf.data_ptr(), ws.nbytes
+            c.dl_ddeath_dev, c.grad_dev = g.data_ptr(), gp.data_ptr()
+            keep.append((p, g))
             out.append(gp)
-        for s in ctx.streams:
-            cur.wait_stream(s)
+            at += ctx.sizes[i]
+        _many(_lib.load().ph0_backward_many, "ph0_barcodes_backward", clouds, ctx.streams, cur)
         return (None, None, *out)
+
+
+def _many(call, what, clouds, streams, cur):
+    """One call that queues work for many clouds on `streams`, after the
+    current stream's work; the current stream then waits for all of it."""
+    if not len(clouds):
+        return
+    used = streams[:len(clouds)]
+    for s in used:
+        s.wait_stream(cur)
+    handles = (ctypes.c_void_p * len(used))(*[s.cuda_stream for s in used])
+    rc = call(clouds, len(clouds), handles, len(used))
+    for s in used:
+        cur.wait_stream(s)
+    check(rc, what)
 
 
 class Batch:
