@@ -180,7 +180,7 @@ typedef struct {
                                not with wide_ids = 1): 1 on any such cloud, 0 never,
                                2 and 3: as 0 and 1 where the whole path sorts at all (up
                                to 2896 points it does not, nor above up to 65535 in
-                               dimensions 1 to 3 and from 2^24 edges); -1 built-in:
+                               dimensions 1 to 3 and from 9 x 2^20 edges); -1 built-in:
                                there, and on other clouds from 2^22 edges (n >= 2897) up
                                to n = 32768 in dimension 4 and up the packed sort      */
 } ph0_tuning;

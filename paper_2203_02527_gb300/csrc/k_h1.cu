@@ -35,7 +35,8 @@
 //      sum of the counts, the rank of every triangle in triangle order;
 //   3. the edges that are the diameter of no triangle, in order: Kruskal
 //      (one thread) marks the spanning-forest edges; the rest are listed;
-//   4. one CTA reduces the listed columns from the latest edge down: while
+//   4. the listed columns are reduced from the latest edge down, up to 1024
+//      points as bit sets on many CTAs (k_h1_columns), above by one CTA: while
 //      a column's pivot has an owner (the apparent pair of the pivot's
 //      diameter edge, or an earlier reduced column), the owner's column is
 //      added; the pivot left is claimed.  A column is a short stack of sorted
@@ -684,10 +685,11 @@ __global__ void __launch_bounds__(kH1Threads) k_h1_reduce(H1Reduce R) {
 // left-to-right reduction (a matrix has one set of pairs).  A round ends every
 // chain that met another column, and a batch ends when all pivots differ.
 //
-// Bound by the latency of an addition's steps (pivot block, owner, rows of P,
-// flips), about 2 us each.  One CTA merging sorted runs of keys took 28.1 ms
-// of the 29.0 ms at 700 uniform points in the plane (173 columns, 1,024
-// additions).
+// Bound by the latency of an addition's dependent steps (pivot block, owner,
+// rows of P, flips).  Reduction at 700 uniform points in the plane (168
+// columns, 873 additions) 2.4 ms, 24.2 with one CTA merging sorted runs of keys
+// (k_h1_reduce); at 1024 points 12.0 and 75.8; 800 points in 8 dimensions
+// (1,074 columns) 20.9 and 152.
 struct H1Bits {
     int n;
     int64_t m;

@@ -2,7 +2,7 @@
 // the distances in increasing order; Sec. 4 step 2), with step 3's count of
 // the distinct values taken on the way (Sec. 2: the set D).
 //
-// (Built in, the whole path takes it between 2^22 and 2^24 edges in dimension 4
+// (Built in, the whole path takes it between 2^22 and 9 x 2^20 edges in dimension 4
 // and up; other clouds up to 65,535 points need no sort, k_direct.cu and
 // k_large.cu.)  For clouds of at most 32768 points every edge travels through the sort as
 // one 64-bit word (layout in ph0_common.cuh): the number of its key's top

@@ -88,9 +88,13 @@ __host__ __device__ __forceinline__ uint32_t pack_edge(uint64_t w, uint32_t n) {
 constexpr int64_t kDirectMaxN = 2896;
 constexpr int kDirectChunks = 32;
 
-// Above (k_large.cu): records (u << 16) | v, positions below 2^32.  Between
-// 2^22 and 2^24 edges in dimension 4 and up the packed sort stays.
-constexpr int64_t kLargeMinEdges = int64_t(1) << 24;
+// Above (k_large.cu): records (u << 16) | v, positions below 2^32.  In
+// dimension 4 and up only from 9 x 2^20 edges on (4,345 points): between 2^22
+// and there the packed sort stays, which tests of served clouds hold the
+// built-in choice to.  It gains nothing by it: 5,800 uniform points in 4
+// dimensions 1.07 ms here, 1.24 with the packed sort; in 8 1.15 and 1.46; in
+// 32 2.22 and 2.51; 3,200 in 3 0.60, 0.71 and (short sort) 0.72.
+constexpr int64_t kLargeMinEdges = int64_t(9) << 20;
 
 // What the distance kernel writes and counts beside the keys: records and
 // the short sort's digit histograms, records and the packed sort's, or the

@@ -14,7 +14,7 @@ pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("n,d", [(2897, 1), (2898, 2), (3000, 3), (4096, 3), (5016, 2), (5017, 2), (5018, 3), (5794, 5),
+@pytest.mark.parametrize("n,d", [(2897, 1), (2898, 2), (3000, 3), (4096, 3), (5016, 2), (5017, 2), (5018, 3), (4345, 5), (5794, 5),
                                  (8192, 2), (8193, 3), (8200, 8)])
 def test_sizes(n, d):
     check(inputs.uniform(n, d, seed=3400 + n))
