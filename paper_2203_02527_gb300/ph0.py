@@ -186,7 +186,9 @@ def h1(pts: torch.Tensor):
     bars = torch.empty((max(nb, 1), _lib.H1_BAR_BYTES), dtype=torch.uint8, device=pts.device)
     st = _lib.H1Stats()
     check(lib.ph0_h1(_ptr(pts), n, d, ld, _ptr(bars), _ptr(ws), nbytes, _stream(), ctypes.byref(st)), "ph0_h1")
-    out = bars[:nb].cpu().numpy().reshape(-1).view(_lib.H1_DTYPE)  # host memory of its own
+    out = np.empty(nb, _lib.H1_DTYPE)
+    if nb:
+        torch.from_numpy(out.view(np.uint8).reshape(nb, _lib.H1_BAR_BYTES)).copy_(bars[:nb])
     return out, st.as_dict()
 
 
