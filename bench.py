@@ -41,7 +41,10 @@ WORKLOAD = "circles32768"
 # the top pass), the fix-up.
 PHASE_TRAFFIC_PER_EDGE = {"k_dist": 10.24, "k_onesweep": 25.31, "k_sort_fixup": 8.18}
 ONESWEEP_TRAFFIC_PER_EDGE = PHASE_TRAFFIC_PER_EDGE["k_onesweep"]
-# The packed sort (clouds up to 32768 points, the benchmark's form): DRAM
+# Without a sort (k_large.cu, the benchmark's form): the key written, read and
+# written to its partition
+SORTLESS_BYTES_PER_EDGE = 24
+# The packed sort (clouds up to 32768 points, on request): DRAM
 # bytes per edge of the distance kernel, its four passes and its fix-up with
 # the fix-up's second kernel (whose key gathers grow with the share of edges
 # in groups of equal key >> 22), from ncu on the benchmark cloud itself
@@ -292,7 +295,7 @@ def run_ours(args, rank, world, local_rank):
         early = {"value": job_throughput(m, world, early_t), "unit": "edges/s", "ms_per_step": early_t,
                  "sorted_edges": int(eb.stats["sorted_edges"]), "identical_to_whole_path": early_same,
                  "timing": "host clock around the synchronous call, L2 flushed before each",
-                 "choice": "built-in (sorts in rounds from 2^27 edges on)"}
+                 "choice": "built-in (no sort, step 3 up to the last killing edge, from 2^27 edges on)"}
         if rank == 0 and world == 1:
             early["configs"] = time_early_configs(args, dev, flush)
 
@@ -301,7 +304,8 @@ def run_ours(args, rank, world, local_rank):
     # roofline of the dominant kernel
     mean = lambda k: float(np.mean([p[k] for p in profs]))  # noqa: E731
     passes = int(st["sort_passes"])
-    packed = int(st.get("sort_form", 0)) == 1
+    form = int(st.get("sort_form", 0))
+    packed, sortless = form == 1, form == 3
     # the short sort runs the passes from slot 2 on (the slots below sort key
     # bits 0..15, which the fix-up completes), so slots 0 and 1 stay empty;
     # the packed sort's four passes take slots 0-3
@@ -310,7 +314,7 @@ def run_ours(args, rank, world, local_rank):
     stages = {"dist_ms": mean("dist_ms"), "sort_ms": mean("sort_ms"), "pass_ms": pass_ms,
               "fixup_ms": mean("fixup_ms"), "dedupe_ms": mean("dedupe_ms"),
               "reduce_ms": mean("reduce_ms"), "emit_ms": mean("emit_ms"),
-              "sort_form": "packed" if packed else "short"}
+              "sort_form": ("short", "packed", "complete", "none")[form]}
     hbm, hbm_src = peaks()
     per_pass_ms = float(np.mean(ran)) if ran else 0.0
     if packed:
@@ -331,7 +335,7 @@ def run_ours(args, rank, world, local_rank):
     else:
         # the radix passes: 24 algorithmic bytes per edge per pass, against HBM
         achieved = 24.0 * m / (per_pass_ms * 1e-3) / 1e9 if per_pass_ms > 0 else 0.0
-        roof_sort = {"kernel": "k_onesweep", "bound": "hbm", "achieved": achieved, "peak": hbm,
+        roof_sort = {"kernel": "k_onesweep" if ran else "none: no sort", "bound": "hbm", "achieved": achieved, "peak": hbm,
                      "unit": "GB/s", "frac": achieved / hbm,
                      "traffic": ONESWEEP_TRAFFIC_PER_EDGE * m,
                      "traffic_source": "ncu on the 8192-point cloud (slots 4-6), scaled by edges",
@@ -369,6 +373,10 @@ def run_ours(args, rank, world, local_rank):
         phase_bytes = m * (PACKED_TRAFFIC_PER_EDGE["k_dist"] + sum(PACKED_TRAFFIC_PER_EDGE["k_psweep"])
                            + PACKED_TRAFFIC_PER_EDGE["k_pfixup"])
         phase_kernels = "k_dist, k_psweep x4, k_pfixup"
+    elif sortless:
+        # no sort: the keys written once, then moved to their hash partitions
+        phase_bytes = m * SORTLESS_BYTES_PER_EDGE
+        phase_kernels = "k_dist, k_large_move<0>"
     else:
         phase_bytes = m * (PHASE_TRAFFIC_PER_EDGE["k_dist"] + len(ran) * PHASE_TRAFFIC_PER_EDGE["k_onesweep"]
                            + PHASE_TRAFFIC_PER_EDGE["k_sort_fixup"])
@@ -380,7 +388,7 @@ def run_ours(args, rank, world, local_rank):
              "floor_per_edge": PHASE_FLOOR_PER_EDGE,
              "floor_frac": PHASE_FLOOR_PER_EDGE * m / (phase_ms * 1e-3) / 1e9 / hbm,
              "traffic_source": ("ncu dram bytes per edge of each kernel on the benchmark cloud"
-                                if packed else
+                                if packed else "bytes the two kernels write and read" if sortless else
                                 "ncu dram bytes per edge of each kernel on the 8192-point cloud, scaled by edges"),
              "peak_source": hbm_src}
     # sort init, distances, the short sort (passes from slot 2: 8 launches
@@ -395,6 +403,10 @@ def run_ours(args, rank, world, local_rank):
     launches_per_step = 1 + 1 + (8 + 2) + (1 + 1 + 10 + 1) + 1 + 2 + (1 + 1 + 10) + 1 + 1
     if packed:
         launches_per_step += 1 + 4 + 2 + 1
+    if sortless:
+        # distances, sample, threshold, first move, tree, its order (2),
+        # reduction (2), count, bucket counts, second move, repeats, bars
+        launches_per_step = 14
     cpu = cpu_all = cpu_full = None
     if world == 1 and not args.no_cpu_baseline:
         r, dt, ns, ms_ = time_oracle(x)
