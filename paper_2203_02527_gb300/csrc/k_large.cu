@@ -56,6 +56,8 @@ constexpr int kLgPass = 14336;                 // keys of a bucket looked at at 
 constexpr int kLgWords = 20480;                // of a bucket's bit table, slots of its hash table
 constexpr int kLgSuspects = 512, kLgSusSlots = 2048, kLgSusKeys = 1024;
 constexpr int kLgPart = 5120;                  // keys of a larger bucket looked at together
+constexpr int kLgFew = 6144;                   // ... unless it holds at most this many distances: 512 threads
+static_assert(kLgFew + 8 * 512 <= kLgWords / 2, "insert up to eight each after the last look at the count");
 constexpr int kLgRepThreads = 512;
 constexpr int kLgListPerPoint = 64;            // edges per point the list aims at
 constexpr int kLgListRoom = 512;               // ... and has room for
@@ -662,6 +664,49 @@ __global__ void __launch_bounds__(kLgRepThreads, 2) k_large_repeats(const LgArgs
             continue;
         }
         unsigned long long *tab = reinterpret_cast<unsigned long long *>(s_tab);
+        // a bucket this size holds distances repeated often, as a rule few of
+        // them: one table of all; the occurrences beyond the first are the
+        // keys less the table's entries (lattices: 27,000 points of a 30^3
+        // lattice, 1,546 distances, took 428 ms in parts)
+        clear();
+        if (tid == 0) s_ns = s_nk = 0;
+        __syncthreads();
+        bool below = false;  // keys up to the last tree edge's
+        for (uint32_t i0 = tid; i0 < size; i0 += kU * kLgRepThreads) {
+            uint64_t key[kU];
+#pragma unroll
+            for (int q = 0; q < kU; ++q) key[q] = i0 + q * kLgRepThreads < size ? keys[i0 + q * kLgRepThreads] : kNone;
+            if (*(volatile uint32_t *)&s_ns > uint32_t(kLgFew)) break;  // the table fills: in parts
+#pragma unroll
+            for (int q = 0; q < kU; ++q) {
+                if (key[q] == kNone) continue;
+                below |= key[q] <= top;
+                uint32_t slot = __umulhi(uint32_t(key_hash(key[q])) * 0x9E3779B9u, uint32_t(kLgWords / 2));
+                for (int pr = 0; pr < kLgWords / 2; ++pr) {
+                    unsigned long long old = *(volatile unsigned long long *)(tab + slot);
+                    if (old == 0) {
+                        old = atomicCAS(tab + slot, 0ull, (unsigned long long)(key[q] + 1));
+                        if (old == 0) atomicAdd(&s_ns, 1u);
+                    }
+                    if (old == 0 || old == key[q] + 1) break;
+                    slot = slot + 1 == kLgWords / 2 ? 0 : slot + 1;
+                }
+            }
+        }
+        below = __syncthreads_or(below);
+        const uint32_t distinct = s_ns;
+        __syncthreads();
+        if (distinct <= uint32_t(kLgFew)) {
+            if (tid == 0) dups += size - distinct;
+            if (below) {
+                for (uint32_t i = tid; i < size; i += kLgRepThreads)
+                    if (keys[i] <= top) atomicAdd(A.dup + lg_place(A.skey, 0, np - 1, keys[i]), 1u);
+                for (int i = tid; i < kLgWords / 2; i += kLgRepThreads)
+                    if (tab[i] != 0 && tab[i] - 1 <= top) atomicSub(A.dup + lg_place(A.skey, 0, np - 1, tab[i] - 1), 1u);
+                __syncthreads();
+            }
+            continue;
+        }
         const uint32_t parts = (size + kLgPart - 1) / kLgPart;
         for (uint32_t part = 0; part < parts; ++part) {
             clear();
@@ -1151,6 +1196,18 @@ __global__ void __launch_bounds__(kLgCountThreads, 2) k_large_count(const LgArgs
     }
     __syncthreads();
     if constexpr (!PREFIX) lg_reps(A, uint32_t(gtid), uint32_t(gthreads));
+    uint64_t gap_key = kNone;
+    uint32_t gap_from = 0, gap_to = 0, gap_n = 0;
+    int gap_t = 0, gap_s = 0;
+    auto flush = [&]() {
+        if (gap_n == 0) return;
+        if (gap_s < np) atomicAdd(gap_s >= base ? s_cnt + (gap_s - base) : A.cnt + gap_s, gap_n);
+        if (gap_s != gap_t) {
+            atomicAdd(A.corr + gap_t, gap_n);
+            if (gap_s < np) atomicSub(A.corr + gap_s, gap_n);
+        }
+        gap_n = 0;
+    };
     auto take = [&](uint64_t key, int64_t e) {
         if (key > top) return;
         int t;
@@ -1172,21 +1229,28 @@ __global__ void __launch_bounds__(kLgCountThreads, 2) k_large_count(const LgArgs
                 return;
             }
         }
-        // as long as a tree edge: its place among them by (u, v)
+        // as long as a tree edge: its place among them by (u, v).  The gap
+        // between tree edges it falls in is remembered with the edges counted
+        // there (20,000 equal points, whose 200M edges all come here: 128 ms
+        // without)
         uint32_t u, v;
         edge_uv(e, A.n, u, v);
         const uint32_t uv = (u << 16) | v;
-        int lo = t, hi = np;
-        while (lo < hi) {
-            const int mid = (lo + hi) >> 1;
-            if (lg_before(A.skey[mid], A.suv[mid], key, uv)) lo = mid + 1;
-            else hi = mid;
+        if (key != gap_key || uv < gap_from || uv > gap_to) {
+            flush();
+            int lo = t, hi = np;
+            while (lo < hi) {
+                const int mid = (lo + hi) >> 1;
+                if (lg_before(A.skey[mid], A.suv[mid], key, uv)) lo = mid + 1;
+                else hi = mid;
+            }
+            gap_key = key;
+            gap_t = t;
+            gap_s = lo;
+            gap_from = lo > t ? A.suv[lo - 1] + 1 : 0u;
+            gap_to = lo < np && A.skey[lo] == key ? A.suv[lo] : 0xffffffffu;
         }
-        if (lo < np) atomicAdd(lo >= base ? s_cnt + (lo - base) : A.cnt + lo, 1u);
-        if (lo != t) {
-            atomicAdd(A.corr + t, 1u);
-            if (lo < np) atomicSub(A.corr + lo, 1u);
-        }
+        ++gap_n;
     };
     constexpr int kU = 8;
     for (int64_t b = int64_t(blockIdx.x) * kLgCountThreads; b < A.m; b += kU * gthreads) {
@@ -1213,6 +1277,7 @@ __global__ void __launch_bounds__(kLgCountThreads, 2) k_large_count(const LgArgs
             }
         }
     }
+    flush();
     __syncthreads();
     if constexpr (PREFIX)
         for (int i = tid; i < kLgParts; i += kLgCountThreads)

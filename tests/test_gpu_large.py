@@ -20,13 +20,15 @@ def test_sizes(n, d):
     check(inputs.uniform(n, d, seed=3400 + n))
 
 
-@pytest.mark.parametrize("name", ["lattice", "lattice3", "one_point", "integers", "duplicates", "exponents",
+@pytest.mark.parametrize("name", ["lattice", "lattice3", "lattice3_20", "bytes", "one_point", "integers", "duplicates", "exponents",
                                   "signed_zeros", "chain", "crowded", "outliers", "mixture"])
 def test_clouds(name):
     rng = np.random.default_rng(3500)
     crowded = rng.random((3200, 3)) * 1e-12
     crowded[1600:, 1] = 1.0
     x = {"lattice": lambda: inputs.lattice(75, 2), "lattice3": lambda: inputs.lattice(15, 3),
+         "lattice3_20": lambda: inputs.lattice(20, 3),
+         "bytes": lambda: rng.integers(0, 256, (6000, 3)).astype(np.float32),
          "one_point": lambda: np.full((3000, 2), 0.5, np.float32),
          "integers": lambda: rng.integers(0, 3000, (5200, 1)).astype(np.float32),
          "duplicates": lambda: inputs.with_duplicates(3100, 3, 700, seed=3501),
