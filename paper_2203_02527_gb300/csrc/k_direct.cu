@@ -1171,11 +1171,14 @@ cudaError_t launch_direct(void *ws, const Layout &L, const float *pts, int64_t n
     if (e == cudaSuccess && after_tree) e = cudaEventRecord(after_tree, s);
     if (e != cudaSuccess) return e;
 
-    const size_t csm = size_t(20) * size_t(n);
-    if (csm > 48 * 1024) {
-        e = cudaFuncSetAttribute(k_direct_count, cudaFuncAttributeMaxDynamicSharedMemorySize, int(csm));
-        if (e != cudaSuccess) return e;
-    }
+    // the kernel's limit is one for the whole process: the largest size it
+    // needs, on every call (a call's own size could lower it between another
+    // thread's setting and launch; the 48 KB it has unset include its static
+    // shared memory, so 2,451 points already need it)
+    constexpr size_t kPerPoint = 20;
+    e = cudaFuncSetAttribute(k_direct_count, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kPerPoint * kDirectMaxN));
+    if (e != cudaSuccess) return e;
+    const size_t csm = kPerPoint * size_t(n);
     // two CTAs per SM, or fewer with at least 2048 edges each
     int grid = int((L.m + 2047) / 2048);
     if (grid > 2 * sm_count()) grid = 2 * sm_count();
