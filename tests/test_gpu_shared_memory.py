@@ -7,7 +7,6 @@ import subprocess
 import sys
 import threading
 
-import numpy as np
 import pytest
 
 import oracle
@@ -39,41 +38,48 @@ def test_counts_around_48_kb_in_a_fresh_process():
     assert out.returncode == 0 and "all equal" in out.stdout, out.stderr[-2000:]
 
 
-def run_side_by_side(sizes, call, rounds):
-    """call(x) for each size in a thread of its own; the exceptions."""
-    failed = []
+def queue_side_by_side(clouds, rounds=40, each=128, tuning=None):
+    """A thread per cloud, each queueing `each` calls on it by one call of
+    ph0_barcodes_many, `rounds` times; what went wrong."""
+    import ctypes
 
-    def work(n):
+    from paper_2203_02527_gb300 import _lib, ph0
+    lib, failed, t = _lib.load(), [], _lib.Tuning.make(**tuning) if tuning else None
+
+    def work(x):
+        torch.cuda.set_device(0)
+        n, d = x.shape
+        pts, ws = torch.from_numpy(x).cuda(), ph0.Workspace(n, d)
+        raw = torch.empty((n - 1, _lib.BAR_BYTES), dtype=torch.uint8, device="cuda")
+        torch.cuda.synchronize()
+        stream = torch.cuda.Stream()
+        calls = (_lib.Cloud * each)()
+        for c in calls:
+            c.pts_dev, c.n, c.ld, c.d, c.bars_dev = pts.data_ptr(), n, d, d, raw.data_ptr()
+            c.ws, c.ws_bytes = ws.buf.data_ptr(), ws.nbytes
+            if t is not None:
+                c.tuning = ctypes.pointer(t)
+        handles = (ctypes.c_void_p * 1)(stream.cuda_stream)
+        for _ in range(rounds):
+            rc = lib.ph0_barcodes_many(calls, each, handles, 1)
+            stream.synchronize()
+            if rc != 0:
+                failed.append((n, rc))
+                return
+        got = raw.cpu().numpy().reshape(-1).view(_lib.BAR_DTYPE)
         try:
-            torch.cuda.set_device(0)
-            x = torch.from_numpy(inputs.uniform(n, 2, seed=4100 + n)).cuda()
-            with torch.cuda.stream(torch.cuda.Stream()):
-                for _ in range(rounds):
-                    call(x)
-        except Exception as e:  # noqa: BLE001
-            failed.append((n, repr(e)))
+            assert_bars_equal(got, oracle.barcodes(x)[0])
+        except AssertionError as e:
+            failed.append((n, str(e)))
 
-    threads = [threading.Thread(target=work, args=(n,)) for n in sizes]
-    for t in threads:
-        t.start()
-    for t in threads:
-        t.join()
+    threads = [threading.Thread(target=work, args=(x,)) for x in clouds]
+    for th in threads:
+        th.start()
+    for th in threads:
+        th.join()
     return failed
 
 
 def test_counts_of_two_sizes_in_two_threads():
-    """A thread with 2,896 points and one with 2,500: neither's launches are
-    refused, and the bars stay right."""
-    from paper_2203_02527_gb300 import ph0
-    ws = {n: ph0.Workspace(n, 2) for n in (2500, 2896)}
-    want = {n: oracle.barcodes(inputs.uniform(n, 2, seed=4100 + n))[0] for n in ws}
-
-    def call(x):
-        got = ph0.barcodes(x, ws[len(x)])
-        if not np.array_equal(got.numpy()["order"], want[len(x)]["order"]):
-            raise AssertionError("order")
-
-    assert run_side_by_side(list(ws), call, 300) == []
-    for n in ws:
-        x = torch.from_numpy(inputs.uniform(n, 2, seed=4100 + n)).cuda()
-        assert_bars_equal(ph0.barcodes(x, ws[n]).numpy(), want[n])
+    """A thread with 2,896 points and one with 2,500: neither's launches are refused."""
+    assert queue_side_by_side([inputs.uniform(n, 2, seed=4100 + n) for n in (2896, 2500)]) == []
