@@ -653,9 +653,12 @@ cudaError_t launch_reduce(const ReduceArgs &A, cudaStream_t s) {
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess || A.m <= A.start) return e;
 
+    // the kernel's limit holds for the whole process: the largest size it
+    // needs, not this call's (which could lower it between another thread's
+    // setting and launch)
     const size_t smem = reduce_dyn_smem(A.n, A.wide);
     const void *fn = A.wide ? (const void *)k_reduce<true> : (const void *)k_reduce<false>;
-    e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+    e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, int(reduce_dyn_smem(kMaxN, A.wide)));
     if (e != cudaSuccess) return e;
     int per_sm = 0;
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kReduceThreads, smem);

@@ -83,3 +83,10 @@ def queue_side_by_side(clouds, rounds=40, each=128, tuning=None):
 def test_counts_of_two_sizes_in_two_threads():
     """A thread with 2,896 points and one with 2,500: neither's launches are refused."""
     assert queue_side_by_side([inputs.uniform(n, 2, seed=4100 + n) for n in (2896, 2500)]) == []
+
+
+def test_reductions_of_two_sizes_in_two_threads():
+    """The reduction after a sort, of 300 points and of 2,800: neither's
+    launches are refused."""
+    clouds = [inputs.uniform(n, 2, seed=4200 + n) for n in (2800, 300)]
+    assert queue_side_by_side(clouds, rounds=20, each=64, tuning={"packed_sort": 0}) == []
