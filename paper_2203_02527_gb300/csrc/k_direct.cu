@@ -1115,7 +1115,7 @@ cudaError_t launch_direct(void *ws, const Layout &L, const float *pts, int64_t n
     const unsigned tiles = unsigned(A.nch) * unsigned(A.nch + 1) / 2;
     const size_t dsm = direct_dist_smem(A.bt, d);
     auto go = [&](auto kernel) {
-        cudaError_t r = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kDirDistSmem));
+        cudaError_t r = smem_limit<kDirDistSmem>(kernel);
         if (r != cudaSuccess) return r;
         kernel<<<tiles, kDirThreads, dsm, s>>>(A);
         return cudaGetLastError();
@@ -1162,7 +1162,7 @@ cudaError_t launch_direct(void *ws, const Layout &L, const float *pts, int64_t n
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     auto tree = [&](auto kernel) {
-        cudaError_t r = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kDirMstSmem));
+        cudaError_t r = smem_limit<kDirMstSmem>(kernel);
         if (r == cudaSuccess && cl > 8) r = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
         if (r == cudaSuccess) r = cudaLaunchKernelEx(&cfg, kernel, (const DirectArgs)A);
         return r;
@@ -1171,12 +1171,10 @@ cudaError_t launch_direct(void *ws, const Layout &L, const float *pts, int64_t n
     if (e == cudaSuccess && after_tree) e = cudaEventRecord(after_tree, s);
     if (e != cudaSuccess) return e;
 
-    // the kernel's limit is one for the whole process: the largest size it
-    // needs, on every call (a call's own size could lower it between another
-    // thread's setting and launch; the 48 KB it has unset include its static
-    // shared memory, so 2,451 points already need it)
+    // (the 48 KB a kernel has without it include its static shared memory, so
+    // 2,451 points already need it)
     constexpr size_t kPerPoint = 20;
-    e = cudaFuncSetAttribute(k_direct_count, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kPerPoint * kDirectMaxN));
+    e = smem_limit<kPerPoint * kDirectMaxN>(k_direct_count);
     if (e != cudaSuccess) return e;
     const size_t csm = kPerPoint * size_t(n);
     // two CTAs per SM, or fewer with at least 2048 edges each

@@ -262,10 +262,12 @@ size_t dist_smem(int bt, int d) {
            size_t((d + 31) / 32) * sizeof(uint32_t);
 }
 
+constexpr size_t kDistSmem = 160 * 1024;
+
 // Tile edge for dimension d: the staged blocks must fit in shared memory.
 int dist_tile(int d, int want) {
     int bt = (want == 32 || want == 64) ? want : 128;
-    while (bt > 8 && dist_smem(bt, d) > 160 * 1024) bt /= 2;
+    while (bt > 8 && dist_smem(bt, d) > kDistSmem) bt /= 2;
     return bt;
 }
 
@@ -275,12 +277,12 @@ cudaError_t launch_dist(const float *pts, int64_t n, int32_t d, int64_t ld, uint
     if (n < 2) return cudaSuccess;
     const int bt = dist_tile(d, tile);
     const size_t smem = dist_smem(bt, d);
-    if (smem > 160 * 1024) return cudaErrorInvalidValue;
+    if (smem > kDistSmem) return cudaErrorInvalidValue;
     const int64_t T = (n + bt - 1) / bt;
     const int64_t tiles = T * (T + 1) / 2;
     const int hw16 = (split16 >= 0 && split16 <= 16) ? split16 : kDefaultDistSplit16;
     auto go = [&](auto kernel) {
-        cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024);
+        cudaError_t e = smem_limit<kDistSmem>(kernel);
         if (e != cudaSuccess) return e;
         kernel<<<unsigned(tiles), kDistThreads, smem, s>>>(pts, int(n), int(d), ld, bt, hw16, key, val, h, gate,
                                                            wide ? 1 : 0, int(form));

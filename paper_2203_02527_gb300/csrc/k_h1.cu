@@ -1066,6 +1066,12 @@ int sm_count();
 // holds the sorted edges (buffer by esort's plan) and the de-duplication
 // chunk prefixes; bars: n(n-1)/2 - (n-1) entries.  Asynchronous on s;
 // after_scan / after_reduce (may be null) are recorded after steps 2 and 4.
+// Shared memory of k_h1_columns: a bit per edge and one per block of a bit set.
+static constexpr size_t h1_columns_smem(int64_t m, size_t bit_stride) {
+    const size_t blocks = bit_stride * 8 / kH1BlockBits;
+    return 4 * (size_t(m + 31) / 32 + (blocks + 31) / 32);
+}
+
 cudaError_t run_h1(void *ws, const H1Layout &H, int64_t n, const uint64_t *ek0, const uint64_t *ek1,
                    const uint32_t *ev0, const uint32_t *ev1, const Header *esort, const uint32_t *cpref,
                    Header *h, ph0_h1bar *bars, cudaStream_t s, cudaEvent_t after_scan, cudaEvent_t after_reduce) {
@@ -1131,9 +1137,9 @@ cudaError_t run_h1(void *ws, const H1Layout &H, int64_t n, const uint64_t *ek0, 
         R.c = c;
         R.h = h;
         R.spin_limit = kSpinLimit;
-        const size_t blocks = R.bit_words * 32 / kH1BlockBits;
-        const size_t smem = 4 * (size_t(m + 31) / 32 + (blocks + 31) / 32);
-        e = cudaFuncSetAttribute(k_h1_columns, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+        const size_t smem = h1_columns_smem(m, H.bit_stride);
+        constexpr int64_t kMaxM = kH1BitsMaxN * (kH1BitsMaxN - 1) / 2;
+        e = smem_limit<h1_columns_smem(kMaxM, h1_bit_stride(kMaxM, kH1BitsMaxN))>(k_h1_columns);
         void *args[] = {&R};
         if (e == cudaSuccess)
             e = cudaLaunchCooperativeKernel((const void *)k_h1_columns, dim3(unsigned(ctas)), dim3(kH1Threads), args,

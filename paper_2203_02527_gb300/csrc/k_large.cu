@@ -481,7 +481,7 @@ __global__ void __launch_bounds__(kLgThreads, 2048 / kLgThreads) k_large_move(co
     }
 }
 
-size_t move_smem(int level) {
+constexpr size_t move_smem(int level) {
     return size_t(kLgTile) * 8 + size_t(level == 0 ? kLgParts : kLgMaxSub) * 16;
 }
 
@@ -1427,13 +1427,8 @@ LgArgs large_args(void *ws, const Layout &L, ph0_bar *bars, ph0_inf_bar *inf, ui
     return A;
 }
 
-template <typename K>
-cudaError_t room(K kernel, size_t smem) {
-    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
-}
-
 cudaError_t launch_parts(const LgArgs &A, cudaStream_t s) {
-    const cudaError_t e = room(k_large_move<0>, move_smem(0));
+    const cudaError_t e = smem_limit<move_smem(0)>(k_large_move<0>);
     if (e != cudaSuccess) return e;
     const int64_t moves = (A.m + kLgTile - 1) / kLgTile;
     const int ctas = 2048 / kLgThreads * sm_count();
@@ -1461,7 +1456,7 @@ cudaError_t launch_large_tree(void *ws, const Layout &L, const float *pts, int64
         e = launch_dist(pts, n, d, ld, at<uint64_t>(ws, L.key[0]), nullptr, A.h, s, split16, tile, nullptr, false,
                         prefix ? kDistKeys : kDistHashed);
     if (e == cudaSuccess && after_dist) e = cudaEventRecord(after_dist, s);
-    if (e == cudaSuccess) e = room(k_large_prep, 32768 * 4);
+    if (e == cudaSuccess) e = smem_limit<32768 * 4>(k_large_prep);
     if (e != cudaSuccess) return e;
     k_large_sample<<<unsigned((lg_samples(A.n) + 255) / 256), 256, 0, s>>>(A);  // into the list's place
     k_large_prep<<<1, 1024, 32768 * 4, s>>>(A);
@@ -1493,7 +1488,7 @@ cudaError_t launch_large_bars(void *ws, const Layout &L, int64_t n, ph0_bar *bar
     const int hot = n - 1 < kLgHot ? int(n - 1) : kLgHot;
     const int64_t counts = (L.m + kLgCountThreads * 16 - 1) / (kLgCountThreads * 16);
     auto count = [&](auto kernel) {
-        const cudaError_t r = room(kernel, size_t(kLgHot) * 12);
+        const cudaError_t r = smem_limit<size_t(kLgHot) * 12>(kernel);
         if (r != cudaSuccess) return r;
         kernel<<<unsigned(counts < ctas ? counts : ctas), kLgCountThreads, size_t(hot) * 12, s>>>(A);
         return cudaGetLastError();
@@ -1505,12 +1500,12 @@ cudaError_t launch_large_bars(void *ws, const Layout &L, int64_t n, ph0_bar *bar
         if ((e = launch_parts(A, s)) != cudaSuccess) return e;
     }
     if (A.nsub > 1) {
-        e = room(k_large_move<1>, move_smem(1));
+        e = smem_limit<move_smem(1)>(k_large_move<1>);
         if (e != cudaSuccess) return e;
         k_large_sub<<<kLgParts * kLgSubCtas, kLgThreads, 0, s>>>(A);
         k_large_move<1><<<kLgParts * kLgSubCtas, kLgThreads, move_smem(1), s>>>(A);
     }
-    e = room(k_large_repeats, size_t(kLgWords) * 4);
+    e = smem_limit<size_t(kLgWords) * 4>(k_large_repeats);
     if (e != cudaSuccess) return e;
     k_large_repeats<<<unsigned(ctas), kLgRepThreads, size_t(kLgWords) * 4, s>>>(A);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;

@@ -636,7 +636,7 @@ cudaError_t launch_inf(Header *h, int64_t n, ph0_inf_bar *inf, cudaStream_t s) {
 
 // Snapshot labels (2 B per vertex, rounded up to 16 B; none for wide
 // records) plus the tail arrays (global ids of 2 or 4 bytes).
-size_t reduce_dyn_smem(int64_t n, bool wide) {
+constexpr size_t reduce_dyn_smem(int64_t n, bool wide) {
     const size_t snap = wide ? 0 : sizeof(uint16_t) * size_t((n + 7) & ~int64_t(7));
     const size_t rid = wide ? 4 : 2;
     const size_t tail = size_t(kTailCap) * (4 + 4 * 2 + rid * 4 + 2 * 4 + 1);
@@ -653,12 +653,9 @@ cudaError_t launch_reduce(const ReduceArgs &A, cudaStream_t s) {
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess || A.m <= A.start) return e;
 
-    // the kernel's limit holds for the whole process: the largest size it
-    // needs, not this call's (which could lower it between another thread's
-    // setting and launch)
     const size_t smem = reduce_dyn_smem(A.n, A.wide);
     const void *fn = A.wide ? (const void *)k_reduce<true> : (const void *)k_reduce<false>;
-    e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, int(reduce_dyn_smem(kMaxN, A.wide)));
+    e = A.wide ? smem_limit<reduce_dyn_smem(kMaxN, true)>(fn) : smem_limit<reduce_dyn_smem(kMaxN, false)>(fn);
     if (e != cudaSuccess) return e;
     int per_sm = 0;
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kReduceThreads, smem);

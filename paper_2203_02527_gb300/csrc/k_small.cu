@@ -300,7 +300,7 @@ int small_max_d() { return kSmallMaxD; }
 // task count is read on the device so that a captured launch can be replayed
 // for any batch.
 cudaError_t prepare_small_kernel() {
-    return cudaFuncSetAttribute(k_small, cudaFuncAttributeMaxDynamicSharedMemorySize, int(sizeof(SmallSmem)));
+    return smem_limit<sizeof(SmallSmem)>(k_small);
 }
 
 cudaError_t launch_small(const SmallTask *tasks, const int32_t *ntasks_dev, uint32_t *counter, int grid,

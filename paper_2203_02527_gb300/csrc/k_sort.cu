@@ -779,20 +779,12 @@ cudaError_t launch_keystats(const uint64_t *keys, int64_t m, Header *h, cudaStre
 template <int RADIX, int SLOT>
 static cudaError_t set_attr() {
     constexpr int TT = slot_threads<RADIX>();
-    const int bytes = int(sort_smem<RADIX>());
-    const int tbytes = int(sort_smem<RADIX, TT>());
-    cudaError_t e = cudaFuncSetAttribute(k_onesweep<RADIX, SLOT, true, false, TT>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, tbytes);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_onesweep<RADIX, SLOT, false, false, TT>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, tbytes);
+    constexpr size_t kBytes = sort_smem<RADIX>(), kTBytes = sort_smem<RADIX, TT>();
+    cudaError_t e = smem_limit<kTBytes>(k_onesweep<RADIX, SLOT, true, false, TT>);
+    if (e == cudaSuccess) e = smem_limit<kTBytes>(k_onesweep<RADIX, SLOT, false, false, TT>);
     if constexpr (SLOT != kClassSlot) {
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(k_onesweep<RADIX, SLOT, false, true>,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(k_onesweep<RADIX, SLOT, true, true>,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+        if (e == cudaSuccess) e = smem_limit<kBytes>(k_onesweep<RADIX, SLOT, false, true>);
+        if (e == cudaSuccess) e = smem_limit<kBytes>(k_onesweep<RADIX, SLOT, true, true>);
     }
     return e;
 }

@@ -116,6 +116,15 @@ __device__ __forceinline__ uint32_t part_hash(uint64_t key) {
 }
 __device__ __forceinline__ uint32_t hash_part(uint32_t x) { return x >> 23; }
 
+// Lets a kernel be launched with up to kBytes of dynamic shared memory.  The
+// limit holds for the whole process, so it must not be a call's own size
+// (which could lower it between another thread's setting and launch): a
+// template argument cannot be.
+template <size_t kBytes, typename K>
+inline cudaError_t smem_limit(K kernel) {
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kBytes));
+}
+
 // Bounded device-side waits: about a second at most, then the kernel records
 // PH0_ETIMEOUT in the status word and returns cleanly.
 constexpr uint32_t kSpinLimit = 1u << 24;
@@ -332,6 +341,11 @@ constexpr int kH1BitsCtas = 128;
 constexpr size_t kH1BitsBytes = size_t(1) << 31;
 constexpr int kH1BlockBits = 1024;  // bits per touched block
 
+// Bytes of one bit set: a bit per (edge, vertex), in whole blocks.
+constexpr size_t h1_bit_stride(int64_t m, int64_t n) {
+    return align_up((size_t(m) * size_t(n) + 7) / 8, kH1BlockBits / 8) + kH1BlockBits / 8;
+}
+
 // The first-homology regions of a workspace, after the dimension-0 layout.
 // Up to kH1BitsMaxN points a column under reduction is a bit set (bits, one
 // per CTA of k_h1_columns, with its list of edges in pub) and pool_cap bounds
@@ -358,7 +372,7 @@ struct H1Layout {
         ctas = 0;
         bit_stride = 0;
         if (n <= kH1BitsMaxN) {
-            bit_stride = align_up((size_t(m) * size_t(n) + 7) / 8, kH1BlockBits / 8) + kH1BlockBits / 8;
+            bit_stride = h1_bit_stride(m, n);
             const size_t fit = kH1BitsBytes / (bit_stride + 4 * size_t(m + 1));
             ctas = fit < size_t(kH1BitsCtas) ? int(fit) : kH1BitsCtas;
             col_cap = 0;

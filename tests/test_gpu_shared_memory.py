@@ -90,3 +90,4 @@ def test_reductions_of_two_sizes_in_two_threads():
     launches are refused."""
     clouds = [inputs.uniform(n, 2, seed=4200 + n) for n in (2800, 300)]
     assert queue_side_by_side(clouds, rounds=20, each=64, tuning={"packed_sort": 0}) == []
+
