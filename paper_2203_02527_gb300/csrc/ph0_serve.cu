@@ -173,6 +173,13 @@ struct ph0_ctx {
         finished.push_back(r);
     }
 
+    // A launch that failed part of the way: what it queued before still uses
+    // the request's memory, which the next one may get on another stream.
+    void fail_launch(Request *r, int k) {
+        cudaStreamSynchronize(streams[k]);
+        complete(r, PH0_ECUDA);
+    }
+
     // Launch one large request on stream slot `k`.  The first launch leaves
     // out the whole path's gated fallback (about 14 launches that return at
     // once on almost every cloud) and copies the fix-up's fallback flag back
@@ -256,7 +263,7 @@ struct ph0_ctx {
                     const cudaError_t e = launch_large(r, int(k));
                     if (e == cudaSuccess) continue;
                     error = e;
-                    complete(r, PH0_ECUDA);
+                    fail_launch(r, int(k));
                 } else if (q == cudaSuccess) {
                     complete_ok(r);
                 } else {
@@ -314,7 +321,7 @@ struct ph0_ctx {
                 cudaError_t e = launch_large(r, int(k));
                 if (e != cudaSuccess) {
                     error = e;
-                    complete(r, PH0_ECUDA);
+                    fail_launch(r, int(k));
                     slot_req[k] = nullptr;
                     cv_done.notify_all();
                 }
