@@ -161,7 +161,9 @@ __device__ __forceinline__ int lg_place(const uint64_t *skey, int lo, int hi, ui
 // list's threshold from a sample of the keys (evenly spread, jittered):
 // a bin of key >> 48 (sixteen to the octave) and within it one of the next 15
 // bits, so that about kLgListPerPoint n edges lie below; and the bin below
-// which at most a sixteenth of those do (for the rounds on the list).
+// which at most a sixteenth of those do (for the rounds on the list).  More
+// zeros than that (copies of a few points): the list leaves them out, and the
+// tree's first round, over all keys, joins the points that are equal.
 __host__ __device__ __forceinline__ int lg_samples(int n) {
     // four keys per point, so that a few hundred lie below the threshold
     const int S = 4 * n;
@@ -191,12 +193,13 @@ __global__ void __launch_bounds__(1024) k_large_places(const LgArgs A) {
 __global__ void __launch_bounds__(1024) k_large_prep(const LgArgs A) {
     extern __shared__ uint32_t s_bin[];  // [32768]
     __shared__ uint32_t s_w[33];
-    __shared__ uint32_t s_at, s_below;
+    __shared__ uint32_t s_at, s_below, s_zeros;
     const int tid = threadIdx.x;
+    if (tid == 0) s_zeros = 0;
     lg_places(A, s_w);
     const int S = lg_samples(A.n);
     const double want = double(kLgListPerPoint) * double(A.n) * double(S) / double(A.m);
-    uint64_t limit = 0;
+    uint64_t limit = 0, lo = 0;
     uint32_t target = uint32_t(want);
     uint64_t prefix = 0;
     for (int level = 0; level < 2; ++level) {
@@ -209,6 +212,16 @@ __global__ void __launch_bounds__(1024) k_large_prep(const LgArgs A) {
             else if ((k >> 48) == prefix) atomicAdd(s_bin + ((k >> 33) & 32767), 1u);
         }
         __syncthreads();
+        if (prefix == 0 && s_bin[0] > uint32_t(want)) {  // (few clouds; the same for all threads)
+            if (level == 0) {
+                for (uint32_t i = tid; i < uint32_t(S); i += 1024)
+                    if (A.lkey[i] == 0) atomicAdd(&s_zeros, 1u);
+            }
+            __syncthreads();
+            lo = s_zeros > uint32_t(want);
+            if (tid == 0 && lo) s_bin[0] -= s_zeros;
+            __syncthreads();
+        }
         // the bin in which the running count passes the target
         uint32_t sum = 0;
         for (int i = 0; i < 32; ++i) sum += s_bin[tid * 32 + ((i + tid) & 31)];
@@ -254,7 +267,10 @@ __global__ void __launch_bounds__(1024) k_large_prep(const LgArgs A) {
         }
         __syncthreads();
     }
-    if (tid == 0) A.h->lg_limit = limit;
+    if (tid == 0) {
+        A.h->lg_limit = limit > lo ? limit : lo;
+        A.h->lg_lo = uint32_t(lo);
+    }
 }
 
 // A thread's place for the `mine` entries it appends, by one addition per
@@ -282,14 +298,14 @@ __device__ __forceinline__ void lg_room(uint32_t *counter, uint32_t *s_n, uint32
         *s_n = 0;
     }
 }
-// The keys of a thread below the limit, with their edges, to the list from
-// place `at` on.  (kNone, past the end, is below no limit.)
+// The keys of a thread from lo on and below the limit, with their edges, to
+// the list from place `at` on.  (kNone, past the end, is below no limit.)
 template <int N>
 __device__ __forceinline__ void lg_list_put(const LgArgs &A, const uint64_t (&key)[N], int64_t e0, int64_t step,
-                                            uint64_t limit, uint32_t at) {
+                                            uint64_t lo, uint64_t limit, uint32_t at) {
 #pragma unroll
     for (int q = 0; q < N; ++q) {
-        if (key[q] >= limit) continue;
+        if (key[q] >= limit || key[q] < lo) continue;
         if (at < A.lcap) {
             uint32_t u, v;
             edge_uv(e0 + q * step, A.n, u, v);
@@ -304,23 +320,27 @@ __device__ __forceinline__ void lg_list_put(const LgArgs &A, const uint64_t (&ke
 __global__ void __launch_bounds__(1024, 2) k_large_list(const LgArgs A) {
     __shared__ uint32_t s_n, s_base;
     constexpr int kU = 8;
-    const uint64_t limit = A.h->lg_limit;
+    const uint64_t lo = A.h->lg_lo, limit = A.h->lg_limit;
     const int64_t stride = int64_t(gridDim.x) * 1024;
     if (threadIdx.x == 0) s_n = 0;
     __syncthreads();
     for (int64_t b = int64_t(blockIdx.x) * 1024; b < A.m; b += kU * stride) {  // the same for a whole CTA
         const int64_t e0 = b + threadIdx.x;
         uint64_t key[kU];
-        uint32_t mine = 0;
 #pragma unroll
         for (int q = 0; q < kU; ++q) key[q] = e0 + q * stride < A.m ? A.mat[e0 + q * stride] : kNone;
+        uint32_t mine = 0;
 #pragma unroll
         for (int q = 0; q < kU; ++q) mine += key[q] < limit;
+        if (lo && mine) {
+#pragma unroll
+            for (int q = 0; q < kU; ++q) mine -= key[q] < lo;
+        }
         const uint32_t at = lg_rank(mine, &s_n);
         __syncthreads();
         lg_room(&A.h->lg_list, &s_n, &s_base);
         __syncthreads();
-        if (mine) lg_list_put<kU>(A, key, e0, stride, limit, s_base + at);
+        if (mine) lg_list_put<kU>(A, key, e0, stride, lo, limit, s_base + at);
     }
 }
 
@@ -361,7 +381,8 @@ __global__ void __launch_bounds__(kLgThreads, 2048 / kLgThreads) k_large_move(co
         if (tid < kDig) s_base[tid] = run;
         if (tid < ndig && first == 0) A.boff[size_t(p) * ndig + tid] = run;
     }
-    const uint64_t limit = LEVEL == 0 && !A.prefix ? A.h->lg_limit : 0;
+    const bool listing = LEVEL == 0 && !A.prefix;
+    const uint64_t lo = listing ? A.h->lg_lo : 0, limit = listing ? A.h->lg_limit : 0;
     if (tid == 0) s_nlist = 0;
     auto digit = [&](uint64_t k) { return LEVEL == 0 ? hash_part(part_hash(k)) : hash_sub(part_hash(k), ndig); };
     for (int64_t t0 = begin + first * kLgTile; t0 < end; t0 += step * kLgTile) {
@@ -386,7 +407,7 @@ __global__ void __launch_bounds__(kLgThreads, 2048 / kLgThreads) k_large_move(co
         uint32_t mine = 0, at = 0;  // for the list
         if constexpr (LEVEL == 0) {
 #pragma unroll
-            for (int q = 0; q < kLgPer; ++q) mine += key[q] < limit;
+            for (int q = 0; q < kLgPer; ++q) mine += key[q] - lo < limit - lo;
             at = lg_rank(mine, &s_nlist);
         }
         const bool dedupe = __syncthreads_or(crowded);
@@ -466,7 +487,7 @@ __global__ void __launch_bounds__(kLgThreads, 2048 / kLgThreads) k_large_move(co
             }
         }
         __syncthreads();
-        if (LEVEL == 0 && mine) lg_list_put<kLgPer>(A, key, t0 + tid, kLgThreads, limit, s_list + at);
+        if (LEVEL == 0 && mine) lg_list_put<kLgPer>(A, key, t0 + tid, kLgThreads, lo, limit, s_list + at);
 #pragma unroll
         for (int q = 0; q < kLgPer; ++q) {
             if (place[q] == 0xffffffffu) continue;
@@ -744,9 +765,19 @@ __device__ __forceinline__ uint32_t lg_other(const LgArgs &A, uint32_t c) {
     return a == c ? b : a;
 }
 
+// Edges of equal keys meet at one component in their millions (two distances
+// between 20,000 points: 10^8 edges for two components), so an atomic is only
+// made by an edge that comes before the one found so far: the tree of that
+// cloud takes 1.2 ms, 13.0 with every edge's atomics.
+__device__ __forceinline__ void lg_first(uint32_t *best, uint32_t uv) {
+    if (uv < __ldcg(best)) atomicMin(best, uv);
+}
+__device__ __forceinline__ void lg_less(unsigned long long *best, uint64_t key) {
+    if (key < __ldcg(best)) atomicMin(best, (unsigned long long)key);
+}
 __device__ __forceinline__ void lg_offer(const LgArgs &A, uint64_t key, uint32_t uv, uint32_t cu, uint32_t cv) {
-    if (key == __ldcg(A.best + cu)) atomicMin(A.buv + cu, uv);
-    if (key == __ldcg(A.best + cv)) atomicMin(A.buv + cv, uv);
+    if (key == __ldcg(A.best + cu)) lg_first(A.buv + cu, uv);
+    if (key == __ldcg(A.best + cv)) lg_first(A.buv + cv, uv);
 }
 
 // First row and column of 128 x 128 tile w of the upper triangle (T tiles a
@@ -784,7 +815,8 @@ __global__ void __launch_bounds__(kLgTreeThreads, 2) k_large_tree(const LgArgs A
     uint32_t joined = 0, rounds = 0, passes = 0;
     uint32_t live = uint32_t(gtid) < list ? (list - gtid - 1) / gthreads + 1 : 0u;  // entries of this thread
     const uint64_t first = __ldcg(&h->lg_first);
-    bool on_list = list > 0;
+    // (a list without zeros serves once equal points are joined)
+    bool later = list > 0 && __ldcg(&h->lg_lo) != 0, on_list = list > 0 && !later;
     const int64_t T = (n + 127) / 128, tiles = T * (T + 1) / 2;
     const int warps = gthreads >> 5, gwarp = gtid >> 5;
     while (joined < uint32_t(n - 1)) {
@@ -867,8 +899,8 @@ __global__ void __launch_bounds__(kLgTreeThreads, 2) k_large_tree(const LgArgs A
 #pragma unroll
                 for (int q = 0; q < 4; ++q) {
                     if (cu[q] == cv[q]) continue;
-                    if (k[q] == bu[q]) atomicMin(A.buv + cu[q], uv[q]);
-                    if (k[q] == bv[q]) atomicMin(A.buv + cv[q], uv[q]);
+                    if (k[q] == bu[q]) lg_first(A.buv + cu[q], uv[q]);
+                    if (k[q] == bv[q]) lg_first(A.buv + cv[q], uv[q]);
                 }
             }
         } else {
@@ -959,6 +991,7 @@ __global__ void __launch_bounds__(kLgTreeThreads, 2) k_large_tree(const LgArgs A
                 // whole tiles off the diagonal need no look at u < v < n
                 const bool inner = u0 + 31 < v0 && v0 + 127 < n;
                 const uint64_t *line = A.mat + (edge_index(n, u0, 0) + v0 + lane);
+                uint32_t rowc = 0xffffffffu, colc = 0xffffffffu;  // row u0 + lane's edge: column; the columns': rows
                 for (int i0 = 0; i0 < 32; i0 += 4) {
                     uint64_t key[4][4];
 #pragma unroll
@@ -990,7 +1023,6 @@ __global__ void __launch_bounds__(kLgTreeThreads, 2) k_large_tree(const LgArgs A
                         for (int q = 0; q < 4; ++q) hit |= key[r][q] < bu || key[r][q] < bv[q];
                         if (!__any_sync(0xffffffffu, hit)) continue;
                         const uint32_t cu = __shfl_sync(0xffffffffu, cul, i0 + r);
-                        const int64_t e0 = edge_index(n, u0 + i0 + r, 0) + v0 + lane;
                         // the row's smallest key and the first edge that has it
                         uint64_t mine = kNone;
                         uint32_t at = 0xffffffffu;
@@ -1005,27 +1037,43 @@ __global__ void __launch_bounds__(kLgTreeThreads, 2) k_large_tree(const LgArgs A
                         const uint32_t ml = __reduce_min_sync(0xffffffffu, lo);
                         const uint64_t mn = (uint64_t(mh) << 32) | ml;
                         at = __reduce_min_sync(0xffffffffu, mine == mn ? at : 0xffffffffu);
-                        const bool row = mn < bu;
-                        if (row) {
-                            if (lane == 0) atomicMin(A.best + cu, (unsigned long long)mn);
+                        if (mn < bu) {
+                            if (lane == 0) lg_less(A.best + cu, mn);
                             if (cul == cu && mn < bul) bul = mn;
+                            if (lane == i0 + r) rowc = at;
                         }
 #pragma unroll
                         for (int q = 0; q < 4; ++q) {
-                            const bool col = key[r][q] < bv[q];
-                            if (col) {
+                            if (key[r][q] < bv[q]) {
                                 bv[q] = key[r][q];
-                                atomicMin(A.best + cv[q], (unsigned long long)bv[q]);
+                                lg_less(A.best + cv[q], bv[q]);
+                                colc = (colc & ~(0xffu << (8 * q))) | uint32_t(i0 + r) << (8 * q);
                             }
-                            const bool take = col || (row && at == uint32_t(q * 32 + lane));
-                            const unsigned who = __ballot_sync(0xffffffffu, take);
-                            if (!who) continue;
-                            uint32_t j = 0;
-                            if (lane == 0) j = atomicAdd(&h->lg_cand, uint32_t(__popc(who)));
-                            j = __shfl_sync(0xffffffffu, j, 0) + __popc(who & ((1u << lane) - 1u));
-                            if (take && j < A.ccap) A.cand[j] = uint32_t(e0 + q * 32);
                         }
                     }
+                }
+                // the edges that bettered a row's component, and the last
+                // that bettered a column's (it has that column's smallest
+                // key), with one addition to the counter (one per row and 32
+                // columns: clouds of many equal keys waited for it alone)
+                uint32_t total = 0, at[5];
+                bool has[5];
+#pragma unroll
+                for (int q = 0; q < 5; ++q) {
+                    has[q] = q < 4 ? ((colc >> (8 * q)) & 0xffu) != 0xffu : rowc != 0xffffffffu;
+                    const unsigned who = __ballot_sync(0xffffffffu, has[q]);
+                    at[q] = total + __popc(who & ((1u << lane) - 1u));
+                    total += __popc(who);
+                }
+                if (total == 0) continue;
+                uint32_t j = 0;
+                if (lane == 0) j = atomicAdd(&h->lg_cand, total);
+                j = __shfl_sync(0xffffffffu, j, 0);
+#pragma unroll
+                for (int q = 0; q < 5; ++q) {
+                    if (!has[q] || j + at[q] >= A.ccap) continue;
+                    const int u = q < 4 ? u0 + int((colc >> (8 * q)) & 0xffu) : u0 + lane;
+                    A.cand[j + at[q]] = uint32_t(edge_index(n, u, v0 + (q < 4 ? q * 32 + lane : int(rowc))));
                 }
             }
             if (!grid_barrier(h, &s_ok, A.spin_limit)) return;
@@ -1092,6 +1140,8 @@ __global__ void __launch_bounds__(kLgTreeThreads, 2) k_large_tree(const LgArgs A
             }
             on_list = false;
         }
+        if (later) on_list = true;
+        later = false;
         joined = now;
     }
     if (gtid == 0) {

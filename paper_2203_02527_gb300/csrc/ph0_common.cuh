@@ -218,6 +218,7 @@ struct Header {
     uint32_t lg_passes;          // (of them over all keys)
     uint32_t lg_offers;          // (edges that bettered a component's best in these)
     uint32_t lg_keep;            // edges up to the last killing edge (the early path)
+    uint32_t lg_lo;              // 1: the list leaves out keys of zero
     // class partition of the early path (radix slot kClassSlot): the key
     // bins of its histogram and the classes' bin ranges [bound[c], bound[c+1])
     uint64_t part_kmin;
