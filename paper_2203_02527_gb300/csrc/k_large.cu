@@ -66,6 +66,7 @@ constexpr int kLgTreeThreads = 512;
 constexpr int kLgRun = 2048;                   // tree edges sorted by a CTA
 constexpr int kLgHot = 8192;                   // longest tree edges whose counts stay in shared memory
 constexpr int kLgCountThreads = 512;
+constexpr int kLgRuns = 256;                   // runs of equal tree edges remembered by a CTA
 constexpr int kLgLutBits = 11, kLgLut = 1 << kLgLutBits;
 constexpr int kLgSubCtas = 4;                  // CTAs per partition
 // keys of a tile in one partition that only repeated distances explain: the
@@ -98,7 +99,7 @@ struct LgArgs {
     const unsigned long long *kill_key;  // [n] k_reduce's pivots: position,
     const uint32_t *kill_val;            //     row
     uint32_t *low;             // [n] pivot row by position
-    uint32_t *cnt, *corr, *dup;  // [n] counts per place among the tree's edges
+    uint32_t *cnt, *late, *dup;  // [n] counts per place among the tree's edges
     uint32_t *poff, *pcur;     // [512 + 1], [512] places of the partitions, their ends
     uint32_t *bcnt, *bcur;     // [512][nsub] keys per bucket, filled
     uint32_t *boff;            // [512][nsub]
@@ -1206,9 +1207,20 @@ __global__ void __launch_bounds__(256) k_large_merge(const LgArgs A) {
 static_assert(32 * kLgRun >= kMaxN - 1, "a lane per run");
 
 // ---------------------------------------------------------- counts, bars ---
-// s(e), t(e), order and a as in k_direct.cu.  The counts of the kLgHot longest
-// tree edges, where nearly all edges up to the last one fall, are kept in
-// shared memory; the others go to the L2 cache.
+// s(e), t(e), order and a as in k_direct.cu.  cnt[s] counts the edges at s(e);
+// those as long as a run of tree edges of one key but behind the run's last
+// are counted apart, in late[end of the run] (a(p) takes them, where order(p)
+// has them only from the run's end on).  The counts of the kLgHot longest tree
+// edges, where nearly all edges up to the last one fall, are kept in shared
+// memory; the others go to the L2 cache.
+// An edge as long as a tree edge: its run comes from a table of the CTA
+// (kLgRuns runs, by a hash of the key, filled as they are met), and most such
+// edges are behind the run's last (copies of few points: the tree joins them
+// in the rows of the first copies), which the table counts; the others are
+// searched for in the run, and the gap between two of its edges is remembered
+// with the edges counted there.  20,000 points of two kinds, whose 200M edges
+// all come here: 1.0 ms; 64 with a search over the tree's edges and three
+// atomics on the L2 cache's words for every edge.
 // PREFIX (the early path): the keys counted are also kept for step 3, with
 // the histogram of their partitions.
 template <bool PREFIX>
@@ -1221,10 +1233,22 @@ __global__ void __launch_bounds__(kLgCountThreads, 2) k_large_count(const LgArgs
     uint64_t *s_key = reinterpret_cast<uint64_t *>(s_dyn);      // [hot]
     uint32_t *s_cnt = reinterpret_cast<uint32_t *>(s_key + hot);  // [hot]
     // where to look: the first hot key at or beyond each of kLgLut steps of
-    // the way from the first to the last (a search over them all takes a warp
+    // the way from the second to the last (a search over them all takes a warp
     // with a few keys to place 13 steps: 3.0 ms instead of 1.15 at 30,000
     // points in eight clusters, 450M keys)
     __shared__ uint16_t s_lut[kLgLut + 2];
+    // runs of equal tree edges: key (kNone: a free slot), first and end,
+    // number of the last edge (kUnknown until all three are written), edges
+    // behind it
+    constexpr uint32_t kUnknown = 0xffffffffu;
+    __shared__ unsigned long long s_rkey[kLgRuns];
+    __shared__ int s_rfirst[kLgRuns], s_rend[kLgRuns];
+    __shared__ uint32_t s_rlast[kLgRuns], s_late[kLgRuns];
+    for (int i = tid; i < kLgRuns; i += kLgCountThreads) {
+        s_rkey[i] = kNone;
+        s_rlast[i] = kUnknown;
+        s_late[i] = 0;
+    }
     for (int i = tid; i < hot; i += kLgCountThreads) {
         s_key[i] = A.skey[base + i];
         s_cnt[i] = 0;
@@ -1235,72 +1259,100 @@ __global__ void __launch_bounds__(kLgCountThreads, 2) k_large_count(const LgArgs
         if (p < (unsigned long long)np) A.low[p] = A.kill_val[j];
     }
     __syncthreads();
+    // the steps go from the second key on: many tree edges may have the first,
+    // zero, whose distance from the others would leave these in one step
     const uint64_t top = s_key[hot - 1], bottom = s_key[0];
-    int shift = bitlen64(top - bottom) - kLgLutBits;
+    const uint64_t second = s_key[lg_place(s_key, 0, hot - 1, bottom + 1)];
+    int shift = bitlen64(top - second) - kLgLutBits;
     if (shift < 0) shift = 0;
     for (int i = tid; i < kLgLut + 2; i += kLgCountThreads) s_lut[i] = uint16_t(hot - 1);
     __syncthreads();
     for (int i = tid; i < hot; i += kLgCountThreads) {
-        const int b = int((s_key[i] - bottom) >> shift), a = i > 0 ? int((s_key[i - 1] - bottom) >> shift) : -1;
+        if (s_key[i] < second) continue;
+        const int b = int((s_key[i] - second) >> shift);
+        const int a = i > 0 && s_key[i - 1] >= second ? int((s_key[i - 1] - second) >> shift) : -1;
         for (int j = a + 1; j <= b; ++j) s_lut[j] = uint16_t(i);
     }
     __syncthreads();
     if constexpr (!PREFIX) lg_reps(A, uint32_t(gtid), uint32_t(gthreads));
     uint64_t gap_key = kNone;
     uint32_t gap_from = 0, gap_to = 0, gap_n = 0;
-    int gap_t = 0, gap_s = 0;
+    int gap_s = 0;
     auto flush = [&]() {
-        if (gap_n == 0) return;
-        if (gap_s < np) atomicAdd(gap_s >= base ? s_cnt + (gap_s - base) : A.cnt + gap_s, gap_n);
-        if (gap_s != gap_t) {
-            atomicAdd(A.corr + gap_t, gap_n);
-            if (gap_s < np) atomicSub(A.corr + gap_s, gap_n);
-        }
+        if (gap_n) atomicAdd(gap_s >= base ? s_cnt + (gap_s - base) : A.cnt + gap_s, gap_n);
         gap_n = 0;
     };
-    auto take = [&](uint64_t key, int64_t e) {
-        if (key > top) return;
-        int t;
-        bool tie;
-        if (key > bottom || base == 0) {
-            const int b = key > bottom ? int((key - bottom) >> shift) : 0;
-            const int i = lg_place(s_key, s_lut[b], s_lut[b + 1], key);
-            tie = s_key[i] == key;
-            t = base + i;
-            if (!tie) {
-                atomicAdd(s_cnt + i, 1u);
+    // a key as long as tree edge t (-1: not known, nor whether there is one)
+    auto tie = [&](uint64_t key, int64_t e, int t) {
+        const uint32_t h = (uint32_t(key >> 32) * 0x9E3779B9u + uint32_t(key) * 0x7F4A7C15u) >> 24;
+        static_assert(kLgRuns == 256, "eight bits of the hash");
+        const uint32_t known = *(volatile uint64_t *)&s_rkey[h] == key ? *(volatile uint32_t *)&s_rlast[h] : kUnknown;
+        int end;
+        if (known != kUnknown) {
+            if (uint32_t(e) > known) {
+                atomicAdd(s_late + h, 1u);
                 return;
             }
+            __threadfence_block();
+            t = *(volatile int *)&s_rfirst[h];
+            end = *(volatile int *)&s_rend[h];
         } else {
-            t = lg_place(A.skey, 0, base, key);
-            tie = A.skey[t] == key;
-            if (!tie) {
-                atomicAdd(A.cnt + t, 1u);
+            if (t < 0) {
+                t = lg_place(A.skey, 0, base, key);
+                if (A.skey[t] != key) {
+                    atomicAdd(A.cnt + t, 1u);
+                    return;
+                }
+            }
+            end = t + 1;
+            if (end < np && A.skey[end] == key) {
+                int hi = np;
+                while (end < hi) {
+                    const int mid = (end + hi) >> 1;
+                    if (A.skey[mid] <= key) end = mid + 1;
+                    else hi = mid;
+                }
+            }
+            const uint32_t last = A.suv[end - 1], elast = uint32_t(edge_index(A.n, last >> 16, last & 0xffffu));
+            if (atomicCAS(&s_rkey[h], (unsigned long long)kNone, (unsigned long long)key) == kNone) {
+                s_rfirst[h] = t;
+                s_rend[h] = end;
+                __threadfence_block();
+                *(volatile uint32_t *)&s_rlast[h] = elast;  // from now on the run is known
+            }
+            if (uint32_t(e) > elast) {
+                atomicAdd(A.late + end, 1u);
                 return;
             }
         }
-        // as long as a tree edge: its place among them by (u, v).  The gap
-        // between tree edges it falls in is remembered with the edges counted
-        // there (20,000 equal points, whose 200M edges all come here: 128 ms
-        // without)
         uint32_t u, v;
         edge_uv(e, A.n, u, v);
         const uint32_t uv = (u << 16) | v;
         if (key != gap_key || uv < gap_from || uv > gap_to) {
             flush();
-            int lo = t, hi = np;
+            int lo = t, hi = end - 1;  // suv[end - 1] >= uv
             while (lo < hi) {
                 const int mid = (lo + hi) >> 1;
-                if (lg_before(A.skey[mid], A.suv[mid], key, uv)) lo = mid + 1;
+                if (A.suv[mid] < uv) lo = mid + 1;
                 else hi = mid;
             }
             gap_key = key;
-            gap_t = t;
             gap_s = lo;
             gap_from = lo > t ? A.suv[lo - 1] + 1 : 0u;
-            gap_to = lo < np && A.skey[lo] == key ? A.suv[lo] : 0xffffffffu;
+            gap_to = A.suv[lo];
         }
         ++gap_n;
+    };
+    auto take = [&](uint64_t key, int64_t e) {
+        if (key > top) return;
+        if (key > bottom) {
+            const int b = key > second ? int((key - second) >> shift) : 0;
+            const int i = lg_place(s_key, s_lut[b], s_lut[b + 1], key);
+            if (s_key[i] == key) tie(key, e, base + i);
+            else atomicAdd(s_cnt + i, 1u);
+        } else {
+            tie(key, e, base == 0 ? 0 : -1);  // base 0: the first tree edge has the least key of all
+        }
     };
     constexpr int kU = 8;
     for (int64_t b = int64_t(blockIdx.x) * kLgCountThreads; b < A.m; b += kU * gthreads) {
@@ -1334,21 +1386,27 @@ __global__ void __launch_bounds__(kLgCountThreads, 2) k_large_count(const LgArgs
             if (s_hist[i]) atomicAdd(&A.h->phist[0][i], s_hist[i]);
     for (int i = tid; i < hot; i += kLgCountThreads)
         if (s_cnt[i]) atomicAdd(A.cnt + base + i, s_cnt[i]);
+    for (int i = tid; i < kLgRuns; i += kLgCountThreads)
+        if (s_late[i]) atomicAdd(A.late + s_rend[i], s_late[i]);
 }
 
 // Each CTA adds up the counts before its 1024 tree edges, then writes their
-// bars; the last one to finish writes the bar that never dies.
+// bars; the last one to finish writes the bar that never dies.  order(p): the
+// edges counted up to place p; a(p): those up to the end of p's run of equal
+// keys and the late ones there, less the repeated ones.
 __global__ void __launch_bounds__(1024) k_large_emit(const LgArgs A) {
-    __shared__ uint32_t s_w[33], s_pre[2];
-    __shared__ int s_last;
+    __shared__ uint32_t s_w[33], s_pre[2], s_upto[1025], s_beyond;
+    __shared__ int s_last, s_end;
     const int tid = threadIdx.x, np = A.n - 1, base = blockIdx.x * 1024, p = base + tid;
+    const int stop = base + 1024 < np ? base + 1024 : np;  // of this CTA's
     if (tid < 2) s_pre[tid] = 0;
+    if (tid == 0) s_beyond = 0;
     __syncthreads();
     uint32_t so = 0, sa = 0;
     for (int i = tid; i < base; i += 1024) {
-        const uint32_t c = A.cnt[i];
+        const uint32_t c = A.cnt[i] + A.late[i];
         so += c;
-        sa += c + A.corr[i] - A.dup[i];
+        sa += c - A.dup[i];
     }
     so = __reduce_add_sync(0xffffffffu, so);
     sa = __reduce_add_sync(0xffffffffu, sa);
@@ -1356,11 +1414,30 @@ __global__ void __launch_bounds__(1024) k_large_emit(const LgArgs A) {
         atomicAdd(s_pre, so);
         atomicAdd(s_pre + 1, sa);
     }
+    const uint64_t key = p < np ? A.skey[p] : kNone;
+    int end = p + 1;  // of p's run
+    if (end < np && A.skey[end] == key) {
+        int hi = np;
+        while (end < hi) {
+            const int mid = (end + hi) >> 1;
+            if (A.skey[mid] <= key) end = mid + 1;
+            else hi = mid;
+        }
+    }
+    if (p == stop - 1) s_end = end;
     __syncthreads();
-    const uint32_t c = p < np ? A.cnt[p] : 0u, a = p < np ? c + A.corr[p] - A.dup[p] : 0u;
+    const uint32_t c = p < np ? A.cnt[p] + A.late[p] : 0u, a = p < np ? c - A.dup[p] : 0u;
     uint32_t total;
     const uint32_t order = s_pre[0] + block_scan<1024>(c, s_w, total) + c;
-    const uint32_t aval = s_pre[1] + block_scan<1024>(a, s_w, total) + a;
+    s_upto[tid] = s_pre[1] + block_scan<1024>(a, s_w, total);
+    if (tid == 0) s_upto[1024] = s_pre[1] + total;
+    // the last run, beyond this CTA's places
+    sa = 0;
+    for (int i = stop + tid; i < s_end; i += 1024) sa += A.cnt[i] + A.late[i] - A.dup[i];
+    sa = __reduce_add_sync(0xffffffffu, sa);
+    if ((tid & 31) == 0 && sa) atomicAdd(&s_beyond, sa);
+    __syncthreads();
+    const uint32_t aval = p < np ? (end > stop ? s_upto[1024] + s_beyond : s_upto[end - base]) + A.late[end] : 0u;
     uint32_t low = 0;
     if (p < np) {
         const uint32_t uv = A.suv[p];
@@ -1371,7 +1448,7 @@ __global__ void __launch_bounds__(1024) k_large_emit(const LgArgs A) {
         b.a = aval;
         b.low = int32_t(low);
         b.order = int64_t(order) - 1;
-        b.death_sq = __longlong_as_double((long long)A.skey[p]);
+        b.death_sq = __longlong_as_double((long long)key);
         b.death = __dsqrt_rn(b.death_sq);
         A.bars[p] = b;
     }
@@ -1455,7 +1532,7 @@ LgArgs large_args(void *ws, const Layout &L, ph0_bar *bars, ph0_inf_bar *inf, ui
     const size_t nb = size_t(kLgParts) * size_t(A.nsub);
     zero = off;
     A.cnt = at<uint32_t>(ws, take(4 * n));
-    A.corr = at<uint32_t>(ws, take(4 * n));
+    A.late = at<uint32_t>(ws, take(4 * n));
     A.dup = at<uint32_t>(ws, take(4 * n));
     A.bcnt = at<uint32_t>(ws, take(4 * nb));
     A.bcur = at<uint32_t>(ws, take(4 * nb));

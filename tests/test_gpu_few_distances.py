@@ -71,8 +71,25 @@ def test_bars(name):
     assert got.stats["n_distinct"] == want.stats["n_distinct"]
 
 
+@pytest.mark.parametrize("name", sorted(k for k in CLOUDS if "5000" not in k))
+def test_early_path(name):
+    from paper_2203_02527_gb300 import ph0
+    x, ((want, _), _) = measured(name)
+    got = ph0.barcodes_early(x)
+    assert got.stats["sort_form"] == 3
+    assert torch.equal(got.raw, want.raw) and got.inf == want.inf
+    assert got.stats["n_distinct"] == int(want.a[-1])
+
+
 @pytest.mark.parametrize("name", ["two_points", "two_points_in_order", "cube_corners", "copies_256", "two_points_5000"])
 def test_tree_among_equal_distances(name):
     """The tree and its pivots: less than half the sorted form's whole path."""
     _, ((_, form), (_, whole)) = measured(name)
     assert form["reduce_ms"] < 0.5 * whole["total_ms"], (form, whole)
+
+
+@pytest.mark.parametrize("name", ["two_points", "two_points_in_order", "cube_corners", "copies_256", "two_points_5000"])
+def test_counts_among_equal_distances(name):
+    """The counts and the repeated distances: less than half the sorted form's whole path."""
+    _, ((_, form), (_, whole)) = measured(name)
+    assert form["dedupe_ms"] < 0.5 * whole["total_ms"], (form, whole)
