@@ -55,9 +55,8 @@ constexpr int kLgBucket = 10240;               // keys per bucket on average, at
 constexpr int kLgPass = 14336;                 // keys of a bucket looked at at once (14 bits)
 constexpr int kLgWords = 20480;                // of a bucket's bit table, slots of its hash table
 constexpr int kLgSuspects = 512, kLgSusSlots = 2048, kLgSusKeys = 1024;
-constexpr int kLgPart = 5120;                  // keys of a larger bucket looked at together
-constexpr int kLgFew = 6144;                   // ... unless it holds at most this many distances: 512 threads
-static_assert(kLgFew + 8 * 512 <= kLgWords / 2, "insert up to eight each after the last look at the count");
+constexpr int kLgSlots = 6784, kLgProbes = 64; // larger buckets: keys with their occurrences
+static_assert(3 * kLgSlots <= kLgWords, "in the same room");
 constexpr int kLgRepThreads = 512;
 constexpr int kLgListPerPoint = 64;            // edges per point the list aims at
 constexpr int kLgListRoom = 512;               // ... and has room for
@@ -547,12 +546,12 @@ __device__ __forceinline__ void lg_reps(const LgArgs &A, uint32_t first, uint32_
 // table compares.  Where more than kLgSuspects are, a hash table of all keys
 // (32-bit slots: the key's place in the bucket and 18 bits of its hash, so an
 // occupied slot needs the key itself only when those agree); a bucket of more
-// than kLgPass keys in parts of kLgPart by another piece of the hash, with the
-// keys in the slots.  (The hash tables alone took 8.3 ps per key: a warp waits
+// than kLgPass keys by one of the distinct keys and their occurrences, in as
+// many parts as those need.  (The hash tables alone took 8.3 ps per key: a warp waits
 // for its lane with the most probes.)
 __global__ void __launch_bounds__(kLgRepThreads, 2) k_large_repeats(const LgArgs A) {
     extern __shared__ __align__(16) unsigned char s_dyn[];
-    uint32_t *s_tab = reinterpret_cast<uint32_t *>(s_dyn);  // [kLgWords] bits, slots, or keys + 1 in half as many
+    uint32_t *s_tab = reinterpret_cast<uint32_t *>(s_dyn);  // [kLgWords] bits, slots, or keys + 1 and occurrences
     __shared__ uint64_t s_key[kLgSusKeys];
     __shared__ uint32_t s_sus[kLgSusSlots], s_ns, s_nk;
     const int tid = threadIdx.x, np = A.n - 1;
@@ -685,74 +684,71 @@ __global__ void __launch_bounds__(kLgRepThreads, 2) k_large_repeats(const LgArgs
             crowded = __syncthreads_count(dups != found) > kLgRepThreads / 4;
             continue;
         }
+        // a bucket this size holds distances repeated often beside about as
+        // many others as any bucket: a table of the distinct keys and (up to
+        // the last tree edge) how often each comes again, of one part of the
+        // hash's values at a time (all at first; a part whose keys do not fit
+        // is taken in two halves, which a one-to-one hash ends at one key).
+        // 50,000 points, a fifth of them equal: 16.0 ms for all buckets, 56.8
+        // when the number of parts followed a bucket's size; half of them on a
+        // line, at 300 places: 4.8 and 9.8.  (Of 6,784 slots 64 probes fail
+        // from about 5,500 keys on; with 128 the first of these took 21.8.)
         unsigned long long *tab = reinterpret_cast<unsigned long long *>(s_tab);
-        // a bucket this size holds distances repeated often, as a rule few of
-        // them: one table of all; the occurrences beyond the first are the
-        // keys less the table's entries (lattices: 27,000 points of a 30^3
-        // lattice, 1,546 distances, took 428 ms in parts)
-        clear();
-        if (tid == 0) s_ns = s_nk = 0;
-        __syncthreads();
-        bool below = false;  // keys up to the last tree edge's
-        for (uint32_t i0 = tid; i0 < size; i0 += kU * kLgRepThreads) {
-            uint64_t key[kU];
-#pragma unroll
-            for (int q = 0; q < kU; ++q) key[q] = i0 + q * kLgRepThreads < size ? keys[i0 + q * kLgRepThreads] : kNone;
-            if (*(volatile uint32_t *)&s_ns > uint32_t(kLgFew)) break;  // the table fills: in parts
-#pragma unroll
-            for (int q = 0; q < kU; ++q) {
-                if (key[q] == kNone) continue;
-                below |= key[q] <= top;
-                uint32_t slot = __umulhi(uint32_t(key_hash(key[q])) * 0x9E3779B9u, uint32_t(kLgWords / 2));
-                for (int pr = 0; pr < kLgWords / 2; ++pr) {
-                    unsigned long long old = *(volatile unsigned long long *)(tab + slot);
-                    if (old == 0) {
-                        old = atomicCAS(tab + slot, 0ull, (unsigned long long)(key[q] + 1));
-                        if (old == 0) atomicAdd(&s_ns, 1u);
-                    }
-                    if (old == 0 || old == key[q] + 1) break;
-                    slot = slot + 1 == kLgWords / 2 ? 0 : slot + 1;
-                }
-            }
-        }
-        below = __syncthreads_or(below);
-        const uint32_t distinct = s_ns;
-        __syncthreads();
-        if (distinct <= uint32_t(kLgFew)) {
-            if (tid == 0) dups += size - distinct;
-            if (below) {
-                for (uint32_t i = tid; i < size; i += kLgRepThreads)
-                    if (keys[i] <= top) atomicAdd(A.dup + lg_place(A.skey, 0, np - 1, keys[i]), 1u);
-                for (int i = tid; i < kLgWords / 2; i += kLgRepThreads)
-                    if (tab[i] != 0 && tab[i] - 1 <= top) atomicSub(A.dup + lg_place(A.skey, 0, np - 1, tab[i] - 1), 1u);
-                __syncthreads();
-            }
-            continue;
-        }
-        const uint32_t parts = (size + kLgPart - 1) / kLgPart;
-        for (uint32_t part = 0; part < parts; ++part) {
+        uint32_t *occ = reinterpret_cast<uint32_t *>(tab + kLgSlots);
+        int bits = 0;
+        uint64_t part = 0;
+        for (;;) {
             clear();
+            if (tid == 0) s_ns = 0;
+            uint32_t more = 0;  // beyond the first of each distance
             __syncthreads();
-            for (uint32_t i = tid; i < size; i += kLgRepThreads) {
-                const uint64_t key = keys[i], x = key_hash(key);
-                if (__umulhi(uint32_t(x) * 2654435761u, parts) != part) continue;
-                uint32_t slot = __umulhi(uint32_t(x) * 0x9E3779B9u, uint32_t(kLgWords / 2));
-                for (int pr = 0;; ++pr) {
+            for (uint32_t i0 = tid; i0 < size; i0 += kU * kLgRepThreads) {
+                uint64_t key[kU];
+#pragma unroll
+                for (int q = 0; q < kU; ++q) key[q] = i0 + q * kLgRepThreads < size ? keys[i0 + q * kLgRepThreads] : kNone;
+                if (*(volatile uint32_t *)&s_ns) break;  // a key found no slot
+#pragma unroll
+                for (int q = 0; q < kU; ++q) {
+                    if (key[q] == kNone) continue;
+                    const uint64_t x = key_hash(key[q]);
+                    if (bits && x >> (64 - bits) != part) continue;
+                    uint32_t slot = __umulhi(uint32_t(x) * 0x9E3779B9u, uint32_t(kLgSlots));
+                    const unsigned long long tag = key[q] + 1;
                     unsigned long long old = *(volatile unsigned long long *)(tab + slot);
-                    if (old == 0) old = atomicCAS(tab + slot, 0ull, (unsigned long long)(key + 1));
-                    if (old == 0) break;
-                    if (old == key + 1) {
-                        again(key);
-                        break;
+                    int pr = 0;
+                    while (old != tag) {
+                        if (old == 0 && (old = atomicCAS(tab + slot, 0ull, tag)) == 0) break;
+                        if (old == tag) break;
+                        slot = slot + 1 == kLgSlots ? 0 : slot + 1;
+                        if (++pr == kLgProbes) break;
+                        old = *(volatile unsigned long long *)(tab + slot);
                     }
-                    slot = slot + 1 == kLgWords / 2 ? 0 : slot + 1;
-                    if (pr == kLgWords) {  // more distinct keys than slots: the hash does not spread them
-                        set_status(A.h, PH0_EINTERNAL);
-                        break;
+                    if (old == tag) {
+                        ++more;
+                        if (key[q] <= top) atomicAdd(occ + slot, 1u);
                     }
+                    if (pr == kLgProbes) *(volatile uint32_t *)&s_ns = 1;
                 }
             }
             __syncthreads();
+            const bool full = s_ns != 0;
+            if (!full) {
+                dups += more;
+                for (int i = tid; i < kLgSlots; i += kLgRepThreads)
+                    if (occ[i]) atomicAdd(A.dup + lg_place(A.skey, 0, np - 1, tab[i] - 1), occ[i]);
+            }
+            __syncthreads();  // before the table is cleared again
+            if (full) {
+                ++bits;
+                part <<= 1;
+                continue;
+            }
+            while (bits > 0 && (part & 1)) {
+                part >>= 1;
+                --bits;
+            }
+            if (bits == 0) break;
+            part |= 1;
         }
     }
     dups = __reduce_add_sync(0xffffffffu, dups);
@@ -1284,9 +1280,14 @@ __global__ void __launch_bounds__(kLgCountThreads, 2) k_large_count(const LgArgs
     };
     // a key as long as tree edge t (-1: not known, nor whether there is one)
     auto tie = [&](uint64_t key, int64_t e, int t) {
-        const uint32_t h = (uint32_t(key >> 32) * 0x9E3779B9u + uint32_t(key) * 0x7F4A7C15u) >> 24;
+        uint32_t h = (uint32_t(key >> 32) * 0x9E3779B9u + uint32_t(key) * 0x7F4A7C15u) >> 24, known = kUnknown;
         static_assert(kLgRuns == 256, "eight bits of the hash");
-        const uint32_t known = *(volatile uint64_t *)&s_rkey[h] == key ? *(volatile uint32_t *)&s_rlast[h] : kUnknown;
+        for (int pr = 0; pr < 4; ++pr) {
+            const uint64_t k = *(volatile uint64_t *)&s_rkey[h];
+            if (k == key) known = *(volatile uint32_t *)&s_rlast[h];
+            if (k == key || k == kNone) break;
+            h = (h + 1) & (kLgRuns - 1);
+        }
         int end;
         if (known != kUnknown) {
             if (uint32_t(e) > known) {

@@ -36,6 +36,15 @@ def hot(n, k):
     return x
 
 
+def line_and_plane(n, places):
+    """Half of n points at whole places on a line, half in the plane, in random order."""
+    rng = np.random.default_rng(75)
+    x = rng.random((n, 2)).astype(np.float32) * places
+    at = rng.permutation(n)[:n // 2]
+    x[at, 0], x[at, 1] = rng.integers(0, places, len(at)), 0.0
+    return x
+
+
 CLOUDS = {
     "two_points": lambda: halves(N, True),
     "two_points_in_order": lambda: halves(N, False),
@@ -44,6 +53,9 @@ CLOUDS = {
     "copies_64": lambda: copies(N, 64),
     "copies_16": lambda: copies(N, 16),
     "a_fifth_equal": lambda: hot(N, N // 5),
+    "half_on_a_line_50000": lambda: line_and_plane(50000, 300),
+    "a_fifth_equal_50000": lambda: hot(50000, 10000),
+    "uniform_50000": lambda: hot(50000, 1),
     "one_point": lambda: np.full((N, 2), 0.25, np.float32),
     "two_points_5000": lambda: halves(5000, True),
     "copies_64_5000": lambda: copies(5000, 64),
@@ -60,6 +72,7 @@ def measured(name):
         runs = [ph0.barcodes_profiled(x, tuning=tuning) for _ in range(4)]
         times = {k: min(p[k] for _, p in runs[1:]) for k in ("total_ms", "reduce_ms", "dedupe_ms", "sort_ms")}
         out.append((ph0.barcodes(x, tuning=tuning), times))
+    torch.cuda.empty_cache()
     return x, out
 
 
@@ -71,7 +84,7 @@ def test_bars(name):
     assert got.stats["n_distinct"] == want.stats["n_distinct"]
 
 
-@pytest.mark.parametrize("name", sorted(k for k in CLOUDS if "5000" not in k))
+@pytest.mark.parametrize("name", sorted(k for k in CLOUDS if "000" not in k))
 def test_early_path(name):
     from paper_2203_02527_gb300 import ph0
     x, ((want, _), _) = measured(name)
@@ -93,3 +106,13 @@ def test_counts_among_equal_distances(name):
     """The counts and the repeated distances: less than half the sorted form's whole path."""
     _, ((_, form), (_, whole)) = measured(name)
     assert form["dedupe_ms"] < 0.5 * whole["total_ms"], (form, whole)
+
+
+def test_distances_repeated_among_distinct_ones():
+    """16,000 distances that come ten thousand times each, too few of one in a
+    tile of 8,192 edges to be taken out there, in buckets of ten thousand
+    others: the counts and the repeated distances take less than 2.5 times as
+    long as without any repeated (a bucket is not read once per 5,000 keys)."""
+    _, ((_, form), _) = measured("a_fifth_equal_50000")
+    _, ((_, plain), _) = measured("uniform_50000")
+    assert form["dedupe_ms"] < 2.5 * plain["dedupe_ms"], (form, plain)
