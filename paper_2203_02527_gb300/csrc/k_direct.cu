@@ -44,6 +44,10 @@ constexpr int kDirCountThreads = 512;
 constexpr int kDirMaxBuckets = 512;        // of kDirBucketLarge keys up to kDirectMaxN points
 constexpr int kDirBucketSmall = 4096, kDirBucketLarge = 8192;
 constexpr int kDirStrip = 32;              // rows of a tile staged at a time
+#ifndef PH0_DIR_PROBES
+#define PH0_DIR_PROBES 512
+#endif
+constexpr int kDirProbes = PH0_DIR_PROBES; // of a bucket's table, at most half full but for repeated distances
 constexpr double kDirCrowd = 6.0;          // standard deviations over the mean that crowd a bucket
 constexpr int kDirMaxRounds = 13;          // 2^12 > kDirectMaxN components halve each round
 constexpr int kDirMstThreads = 1024;
@@ -445,16 +449,23 @@ struct DirMst {
 // did not fit its room (distances that occur many times, but seldom within a
 // strip) takes the upper triangle's keys from the matrix instead, with the
 // repeats that crowded strips recorded taken off.  The hash spreads distinct
-// keys evenly (the mean is at most half the table), so a free slot ends every
-// probe.
+// keys evenly, the mean is at most half the table, and a bucket whose distinct
+// keys do not fit all the same (a key finds no slot in kDirProbes) is taken in
+// two halves by bits of the hash, and so on: a one-to-one hash ends that
+// at one key.
 __device__ void direct_repeats(const DirectArgs &A, unsigned char *s_dyn, int first, int step) {
     unsigned long long *s_key = reinterpret_cast<unsigned long long *>(s_dyn);
     uint32_t *s_occ = reinterpret_cast<uint32_t *>(s_key + A.table);
     const int tid = threadIdx.x, T = blockDim.x, lane = tid & 31;
+    int bits = 0;  // of the hash, those of the part looked at
+    uint64_t part = 0;
+    bool full = false;
+    // (the bucket comes from the hash's high word, the slot from bits 8 to 21)
+    auto within = [&](uint64_t x) { return bits == 0 || (x << 32 | x >> 32) >> (64 - bits) == part; };
     auto insert = [&](uint64_t key, uint64_t x) {
         const unsigned long long tag = key + 1;
         uint32_t slot = hash_slot(x, A.table);
-        for (int pr = 0; pr < A.table; ++pr) {
+        for (int pr = 0; pr < kDirProbes; ++pr) {
             unsigned long long old = *(volatile unsigned long long *)(s_key + slot);
             if (old == 0) old = atomicCAS(s_key + slot, 0ull, tag);
             if (old == 0 || old == tag) {
@@ -463,20 +474,21 @@ __device__ void direct_repeats(const DirectArgs &A, unsigned char *s_dyn, int fi
             }
             slot = (slot + 1) & uint32_t(A.table - 1);
         }
-        set_status(A.h, PH0_EINTERNAL);
+        full = true;
     };
-    for (int b = first; b < A.buckets; b += step) {
+    for (int b = first; b < A.buckets;) {
         for (int i = tid; i < A.table; i += T) {
             s_key[i] = 0;
             s_occ[i] = 0;
         }
         __syncthreads();
         const uint32_t cnt = A.bcount[b];
-        if (cnt <= uint32_t(A.bcap)) {
+        const bool stored = cnt <= uint32_t(A.bcap);
+        if (stored) {
             const uint64_t *keys = A.bkeys + size_t(b) * A.bcap;
             for (uint32_t i = tid; i < cnt; i += T) {
-                const uint64_t k = keys[i];
-                insert(k, key_hash(k));
+                const uint64_t k = keys[i], x = key_hash(k);
+                if (within(x)) insert(k, x);
             }
         } else {
             const uint32_t n = uint32_t(A.n), items = n * n;
@@ -490,20 +502,28 @@ __device__ void direct_repeats(const DirectArgs &A, unsigned char *s_dyn, int fi
 #pragma unroll
                 for (int q = 0; q < 8; ++q) {
                     const uint64_t x = key_hash(key[q]);
-                    if (key[q] != kNoKey && hash_bucket(x, A.buckets) == uint32_t(b)) insert(key[q], x);
+                    if (key[q] != kNoKey && hash_bucket(x, A.buckets) == uint32_t(b) && within(x)) insert(key[q], x);
                 }
             }
-            __syncthreads();
+        }
+        full = __syncthreads_or(full);
+        if (full) {
+            full = false;
+            ++bits;
+            part <<= 1;
+            continue;
+        }
+        if (!stored) {
             const uint32_t strips = A.h->direct_strips;
             for (uint32_t r = tid; r < strips; r += T) {
                 const uint64_t k = A.repk[r], x = key_hash(k);
-                if (hash_bucket(x, A.buckets) != uint32_t(b)) continue;
+                if (hash_bucket(x, A.buckets) != uint32_t(b) || !within(x)) continue;
                 uint32_t slot = hash_slot(x, A.table);
                 for (int pr = 0; pr < A.table && s_key[slot] != k + 1; ++pr) slot = (slot + 1) & uint32_t(A.table - 1);
                 if (s_key[slot] == k + 1) atomicSub(s_occ + slot, A.repx[r]);
             }
+            __syncthreads();
         }
-        __syncthreads();
         uint32_t extra = 0;
         for (int i = tid; i < A.table; i += T) {
             const uint32_t o = s_occ[i];
@@ -517,6 +537,13 @@ __device__ void direct_repeats(const DirectArgs &A, unsigned char *s_dyn, int fi
         extra = __reduce_add_sync(0xffffffffu, extra);
         if (lane == 0 && extra) atomicAdd(&A.h->direct_dups, extra);
         __syncthreads();
+        // the next half, or bucket
+        while (bits > 0 && (part & 1)) {
+            part >>= 1;
+            --bits;
+        }
+        if (bits > 0) part |= 1;
+        else b += step;
     }
 }
 

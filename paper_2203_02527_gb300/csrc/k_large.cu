@@ -55,7 +55,10 @@ constexpr int kLgBucket = 10240;               // keys per bucket on average, at
 constexpr int kLgPass = 14336;                 // keys of a bucket looked at at once (14 bits)
 constexpr int kLgWords = 20480;                // of a bucket's bit table, slots of its hash table
 constexpr int kLgSuspects = 512, kLgSusSlots = 2048, kLgSusKeys = 1024;
-constexpr int kLgSlots = 6784, kLgProbes = 64; // larger buckets: keys with their occurrences
+#ifndef PH0_LG_PROBES
+#define PH0_LG_PROBES 64
+#endif
+constexpr int kLgSlots = 6784, kLgProbes = PH0_LG_PROBES; // larger buckets: keys with their occurrences
 static_assert(3 * kLgSlots <= kLgWords, "in the same room");
 constexpr int kLgRepThreads = 512;
 constexpr int kLgListPerPoint = 64;            // edges per point the list aims at
