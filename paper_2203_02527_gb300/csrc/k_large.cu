@@ -1260,9 +1260,11 @@ __global__ void __launch_bounds__(kLgCountThreads, 2) k_large_count(const LgArgs
     __syncthreads();
     // the steps go from the second key on: many tree edges may have the first,
     // zero, whose distance from the others would leave these in one step
-    const uint64_t top = s_key[hot - 1], bottom = s_key[0];
-    const uint64_t second = s_key[lg_place(s_key, 0, hot - 1, bottom + 1)];
-    int shift = bitlen64(top - second) - kLgLutBits;
+    // (a tree that a wait's end left unfinished has kNone for its missing
+    // edges: what is read past the last key must not count as one up to it)
+    const uint64_t top = s_key[hot - 1] < kNone ? s_key[hot - 1] : kNone - 1, bottom = s_key[0];
+    const uint64_t second = s_key[lg_place(s_key, 0, hot - 1, bottom < kNone ? bottom + 1 : kNone)];
+    int shift = bitlen64(s_key[hot - 1] - second) - kLgLutBits;
     if (shift < 0) shift = 0;
     for (int i = tid; i < kLgLut + 2; i += kLgCountThreads) s_lut[i] = uint16_t(hot - 1);
     __syncthreads();
