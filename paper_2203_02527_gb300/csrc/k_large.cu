@@ -113,6 +113,12 @@ struct LgArgs {
     uint32_t spin_limit;
 };
 
+// All distances zero, the points all equal: the tree is vertex 0's edges and
+// every count is known, so the kernels that read the keys leave them alone
+// (20,000 points: 1.07 ms a call; 3.8 with the keys moved and counted, 2.0
+// by the sorted form, whose passes see that no digit varies).
+__device__ __forceinline__ bool lg_all_equal(const LgArgs &A) { return __ldcg(&A.h->kmax) == 0; }
+
 __device__ __forceinline__ uint32_t hash_sub(uint32_t x, int nsub) { return __umulhi(x << 9, uint32_t(nsub)); }
 
 // Exclusive prefix sum over the CTA (T threads); s_w: T / 32 + 1 words.
@@ -322,6 +328,7 @@ __device__ __forceinline__ void lg_list_put(const LgArgs &A, const uint64_t (&ke
 // The list alone (the early path, whose keys are not all moved).
 __global__ void __launch_bounds__(1024, 2) k_large_list(const LgArgs A) {
     __shared__ uint32_t s_n, s_base;
+    if (lg_all_equal(A)) return;
     constexpr int kU = 8;
     const uint64_t lo = A.h->lg_lo, limit = A.h->lg_limit;
     const int64_t stride = int64_t(gridDim.x) * 1024;
@@ -362,6 +369,7 @@ __global__ void __launch_bounds__(kLgThreads, 2048 / kLgThreads) k_large_move(co
     uint32_t *s_off = s_cnt + kDig, *s_to = s_off + kDig, *s_base = s_to + kDig;  // s_base: LEVEL 1
     __shared__ uint32_t s_w[kLgThreads / 32 + 1], s_nrep, s_rbase, s_extra, s_nlist, s_list;
     const int tid = threadIdx.x;
+    if (LEVEL == 0 && lg_all_equal(A)) return;  // the partitions stay empty
     int64_t begin = 0, end = A.prefix ? int64_t(A.h->lg_keep) : A.m, first = blockIdx.x, step = gridDim.x;
     const uint64_t *src = A.prefix ? A.keep : A.mat;
     uint64_t *dst = A.part;
@@ -805,6 +813,17 @@ __global__ void __launch_bounds__(kLgTreeThreads, 2) k_large_tree(const LgArgs A
     const int n = A.n, tid = threadIdx.x, lane = tid & 31;
     const int gthreads = gridDim.x * kLgTreeThreads, gtid = blockIdx.x * kLgTreeThreads + tid;
     Header *h = A.h;
+    if (lg_all_equal(A)) {
+        for (int j = gtid; j < n - 1; j += gthreads) {
+            A.tkey[j] = 0;
+            A.tuv[j] = uint32_t(j) + 1;  // (0, j + 1)
+        }
+        if (gtid == 0) {
+            h->lg_tree = uint32_t(n - 1);
+            h->lg_rounds = 1;
+        }
+        return;
+    }
     for (int v = gtid; v < n; v += gthreads) {
         A.comp[v] = A.parent[v] = uint32_t(v);
         A.best[v] = kNone;
@@ -1256,6 +1275,15 @@ __global__ void __launch_bounds__(kLgCountThreads, 2) k_large_count(const LgArgs
     for (int64_t j = gtid; j < np; j += gthreads) {
         const unsigned long long p = A.kill_key[j];
         if (p < (unsigned long long)np) A.low[p] = A.kill_val[j];
+    }
+    if (lg_all_equal(A)) {
+        for (int64_t j = gtid; j < np; j += gthreads) A.cnt[j] = 1;
+        if (gtid == 0) {
+            A.late[np] = uint32_t(A.m - np);
+            A.dup[0] = A.h->direct_dups = uint32_t(A.m - 1);
+            A.h->lg_keep = uint32_t(A.m);
+        }
+        return;
     }
     __syncthreads();
     // the steps go from the second key on: many tree edges may have the first,

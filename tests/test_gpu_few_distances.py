@@ -59,6 +59,7 @@ CLOUDS = {
     "one_point": lambda: np.full((N, 2), 0.25, np.float32),
     "two_points_5000": lambda: halves(5000, True),
     "copies_64_5000": lambda: copies(5000, 64),
+    "one_point_5000": lambda: np.full((5000, 2), 0.25, np.float32),
 }
 
 
@@ -116,3 +117,10 @@ def test_distances_repeated_among_distinct_ones():
     _, ((_, form), _) = measured("a_fifth_equal_50000")
     _, ((_, plain), _) = measured("uniform_50000")
     assert form["dedupe_ms"] < 2.5 * plain["dedupe_ms"], (form, plain)
+
+
+@pytest.mark.parametrize("name", sorted(CLOUDS))
+def test_whole_path(name):
+    """The whole path: no longer than the sorted form's."""
+    _, ((_, form), (_, whole)) = measured(name)
+    assert form["total_ms"] < whole["total_ms"], (form, whole)
