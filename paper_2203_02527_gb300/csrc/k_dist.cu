@@ -262,13 +262,15 @@ size_t dist_smem(int bt, int d) {
            size_t((d + 31) / 32) * sizeof(uint32_t);
 }
 
-constexpr size_t kDistSmem = 160 * 1024;
-
-// Tile edge for dimension d: the staged blocks must fit in shared memory.
+// Tile edge for dimension d: the largest that fits 160 KB; 8 only where 16
+// points do not fit 168 (6,000 points in 610 dimensions 77 ms with tiles of 16,
+// 127 with 8; the larger tiles gain nothing by the same room: in 312 dimensions
+// 32 points take 32.7 ms, 16 take 23.3; in 158, 64 take 11.9, 32 take 10.3).
+constexpr size_t kDistTileSmem = 160 * 1024, kDistSmem = 168 * 1024;
 int dist_tile(int d, int want) {
     int bt = (want == 32 || want == 64) ? want : 128;
-    while (bt > 8 && dist_smem(bt, d) > kDistSmem) bt /= 2;
-    return bt;
+    while (bt > 16 && dist_smem(bt, d) > kDistTileSmem) bt /= 2;
+    return bt == 16 && dist_smem(bt, d) > kDistSmem ? 8 : bt;
 }
 
 cudaError_t launch_dist(const float *pts, int64_t n, int32_t d, int64_t ld, uint64_t *key,
