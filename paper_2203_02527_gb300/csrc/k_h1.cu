@@ -78,7 +78,7 @@ __device__ __forceinline__ bool h1_uv(const uint32_t *vals, int64_t p, int64_t n
 }
 
 // Column additions of one call before it stops with PH0_ETOOBIG (776 at 700
-// uniform points in the plane).
+// uniform points in the plane); of one CTA where several reduce columns.
 constexpr unsigned long long kH1MaxAdditions = 1ull << 22;
 
 // Counters of the last run (device; read back by h1_counters).
@@ -840,9 +840,18 @@ __global__ void __launch_bounds__(kH1Threads, 1) k_h1_columns(const H1Bits R) {
         __syncthreads();
     };
 
+    // the reduction ends with an error (the whole CTA returns): the others see
+    // it at their next grid barrier
+    auto stop = [&](int32_t status) {
+        if (tid != 0) return;
+        set_status(R.h, status);
+        atomicExch(&R.h->abort, 1);
+    };
+
     for (int64_t base = 0; base < K; base += G) {
         const int64_t col = base + me;  // in processing order: from the latest edge down
-        bool active = col < K, running = active;
+        const bool active = col < K;
+        bool running = active;
         uint32_t p = 0, piv = kH1NoPivot, len = 0;
         reset();
         if (active) {
@@ -900,10 +909,8 @@ __global__ void __launch_bounds__(kH1Threads, 1) k_h1_columns(const H1Bits R) {
                     __syncthreads();
                     if (op == kNone) break;
                     if (op == kError || adds >= kH1MaxAdditions) {
-                        if (tid == 0) set_status(R.h, op == kError ? PH0_EINTERNAL : PH0_ETOOBIG);
-                        active = false;
-                        piv = kH1NoPivot;
-                        break;
+                        stop(op == kError ? PH0_EINTERNAL : PH0_ETOOBIG);
+                        return;
                     }
                     ++adds;
                     if (op == kApparent) add_edge(e, uv);
@@ -967,25 +974,30 @@ __global__ void __launch_bounds__(kH1Threads, 1) k_h1_columns(const H1Bits R) {
             h1_block_scan(cnt, s_warp, keys);
             if (tid == 0) {
                 const uint64_t off = atomicAdd(&R.c->list_used, (unsigned long long)len);
-                const bool fits = off + len <= uint64_t(R.pool_cap);
-                if (!fits) set_status(R.h, PH0_ETOOBIG);
-                s_len = fits ? len : 0u;
+                s_ok = off + len <= uint64_t(R.pool_cap);
                 s_off = off;
+            }
+            __syncthreads();
+            if (!s_ok) {  // no room for its list: it claims nothing
+                stop(PH0_ETOOBIG);
+                return;
+            }
+            if (tid == 0) {
                 const int32_t q = int32_t(col);
                 R.node_key[q] = h1_key(dp, a2, b2, w);
                 R.node_pos[q] = p;
                 R.node_within[q] = uint32_t(within);
                 R.own_node[p] = uint32_t(q);
-                R.own_off[p] = off;
-                R.own_len[p] = s_len;
+                R.own_off[p] = s_off;
+                R.own_len[p] = len;
                 R.node_next[q] = atomicExch(R.head + dp, q);
                 atomicAdd(R.claims + dp, 1u);
                 atomicAdd(&R.c->nodes, 1ull);
                 atomicAdd(&R.c->pool_used, (unsigned long long)keys);
                 atomicMax(&R.c->max_len, (unsigned long long)keys);
             }
-            __syncthreads();
-            for (uint32_t i = tid; i < s_len; i += T) R.pool[s_off + i] = __ldcg(mine + i);
+            for (uint32_t i = tid; i < len; i += T) R.pool[s_off + i] = __ldcg(mine + i);
+            __syncthreads();  // before s_off is used again
         }
         if (base + G < K && !grid_barrier(R.h, &s_ok, R.spin_limit)) return;
     }

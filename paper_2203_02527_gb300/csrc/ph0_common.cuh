@@ -378,6 +378,9 @@ struct H1Layout {
             ctas = fit < size_t(kH1BitsCtas) ? int(fit) : kH1BitsCtas;
             col_cap = 0;
             pool_cap *= 2;  // 4-byte entries
+#ifdef PH0_H1_POOL  // (a build that tests what a full pool does)
+            pool_cap = PH0_H1_POOL;
+#endif
         }
         size_t off = base;
         auto take = [&](size_t bytes) {

@@ -4,10 +4,7 @@ With the library's tables only keys that a hash crowds on purpose would show
 it, so this builds both units with so few probes that nearly every bucket is
 halved several times, and compares every field of every bar with the oracle
 (integers and keys, so there is no tolerance)."""
-import concurrent.futures as cf
 import ctypes
-import os
-import subprocess
 
 import numpy as np
 import pytest
@@ -15,6 +12,7 @@ import pytest
 import oracle
 from paper_2203_02527_gb300 import inputs
 from tests.test_gpu_parity import assert_bars_equal
+from tests.variants import build_variant
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
@@ -22,23 +20,8 @@ pytestmark = pytest.mark.gpu
 
 @pytest.fixture(scope="module")
 def few_probes(tmp_path_factory):
-    from paper_2203_02527_gb300 import _lib, build
-    build.build()
-    out = tmp_path_factory.mktemp("few_probes")
-    units, flags = ("k_direct", "k_large"), ["-DPH0_DIR_PROBES=3", "-DPH0_LG_PROBES=4"]
-
-    def compile_unit(name):
-        subprocess.check_call([build._nvcc(), *build.NVCC_FLAGS, *flags, "-c", os.path.join(build.CSRC, name + ".cu"),
-                               "-o", str(out / (name + ".o"))])
-
-    with cf.ThreadPoolExecutor(len(units)) as ex:
-        list(ex.map(compile_unit, units))
-    rest = [os.path.join(build.OUT_DIR, os.path.basename(s)[:-3] + ".o") for s in build.sources()]
-    rest = [o for o in rest if os.path.basename(o)[:-2] not in units]
-    lib = str(out / "libph0_few_probes.so")
-    subprocess.check_call([build._nvcc(), *build.ARCH, "-shared", "-o", lib, *(str(out / (u + ".o")) for u in units),
-                           *rest, "-lpthread"])
-    return _lib.load(lib)
+    return build_variant(tmp_path_factory.mktemp("few_probes"), ("k_direct", "k_large"),
+                         ["-DPH0_DIR_PROBES=3", "-DPH0_LG_PROBES=4"])
 
 
 def _cases():
