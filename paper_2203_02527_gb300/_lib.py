@@ -174,6 +174,7 @@ SIGNATURES = {
     "ph0_barcodes_many": (ctypes.c_int, [ctypes.POINTER(Cloud), _I64, ctypes.POINTER(_VP), _I32]),
     "ph0_backward_many": (ctypes.c_int, [ctypes.POINTER(Cloud), _I64, ctypes.POINTER(_VP), _I32]),
     "ph0_h1_workspace_bytes": (_SZ, [_I64, _I32]),
+    "ph0_h1_workspace_best_bytes": (_SZ, [_I64, _I32]),
     "ph0_h1": (ctypes.c_int, [_VP, _I64, _I32, _I64, _VP, _VP, _SZ, _VP, ctypes.POINTER(H1Stats)]),
 }
 

@@ -937,6 +937,12 @@ int ph0_backward_many(const ph0_cloud *clouds, int64_t count, void *const *strea
 size_t ph0_h1_workspace_bytes(int64_t n, int32_t d) {
     if (check_sizes(n, d, d, kH1MaxN) != PH0_OK) return 0;
     const Layout L(n, d);
+    return H1Layout::least(n, L.total);
+}
+
+size_t ph0_h1_workspace_best_bytes(int64_t n, int32_t d) {
+    if (check_sizes(n, d, d, kH1MaxN) != PH0_OK) return 0;
+    const Layout L(n, d);
     return H1Layout(n, L.total).total;
 }
 
@@ -948,8 +954,8 @@ int ph0_h1(const float *pts_dev, int64_t n, int32_t d, int64_t ld, ph0_h1bar *ba
     if (!pts_dev || !ws || (nbars > 0 && !bars_dev)) return PH0_EINVAL;
     if (!aligned(ws, 256) || !aligned(pts_dev, 4) || !aligned(bars_dev, 8)) return PH0_EINVAL;
     const Layout L(n, d);
-    const H1Layout H(n, L.total);
-    if (ws_bytes < H.total) return PH0_ENOMEM;
+    if (ws_bytes < H1Layout::least(n, L.total)) return PH0_ENOMEM;
+    const H1Layout H = H1Layout::in_room(n, L.total, ws_bytes);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const Tune t(nullptr, n);
     Header *h = at<Header>(ws, L.hdr);

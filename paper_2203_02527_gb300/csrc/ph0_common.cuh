@@ -341,6 +341,7 @@ constexpr int64_t kH1BitsMaxN = 1024;
 constexpr int kH1BitsCtas = 128;
 constexpr size_t kH1BitsBytes = size_t(1) << 31;
 constexpr int kH1BlockBits = 1024;  // bits per touched block
+constexpr int kH1FewSets = 5;       // fewer: one CTA with runs instead
 
 // Bytes of one bit set: a bit per (edge, vertex), in whole blocks.
 constexpr size_t h1_bit_stride(int64_t m, int64_t n) {
@@ -360,7 +361,9 @@ struct H1Layout {
     size_t bits, pub, pub_piv;
     size_t cnt, aof, posof, pmat, tcount, tfirst, scan_in, zpref, tpref, bsum, zlist, rlist, head, claims,
         node_key, node_pos, node_next, node_within, own_node, own_off, own_len, col_x, col_m, pool, total;
-    H1Layout(int64_t n, size_t base) {
+    // room: the workspace's bytes, which bound the columns at a time (one at
+    // least); runs: the form with runs at any n
+    H1Layout(int64_t n, size_t base, size_t room = ~size_t(0), bool runs = false) {
         const int64_t m = n_edges(n);
         T = n * (n - 1) * (n - 2) / 6;
         blocks = (m + kH1ScanItems - 1) / kH1ScanItems;
@@ -372,10 +375,9 @@ struct H1Layout {
         pool_cap = clamp(8 * T, int64_t(1) << 20, int64_t(1) << 26) + n + 1;
         ctas = 0;
         bit_stride = 0;
-        if (n <= kH1BitsMaxN) {
+        const bool sets = n <= kH1BitsMaxN && !runs;
+        if (sets) {
             bit_stride = h1_bit_stride(m, n);
-            const size_t fit = kH1BitsBytes / (bit_stride + 4 * size_t(m + 1));
-            ctas = fit < size_t(kH1BitsCtas) ? int(fit) : kH1BitsCtas;
             col_cap = 0;
             pool_cap *= 2;  // 4-byte entries
 #ifdef PH0_H1_POOL  // (a build that tests what a full pool does)
@@ -412,11 +414,30 @@ struct H1Layout {
         own_len = take(4 * M1);
         col_x = take(8 * size_t(col_cap));
         col_m = take(8 * size_t(col_cap));
-        pool = take(ctas ? 4 * size_t(pool_cap) : 8 * size_t(pool_cap));
+        pool = take(sets ? 4 * size_t(pool_cap) : 8 * size_t(pool_cap));
+        if (sets) {
+            const size_t one = bit_stride + 4 * M1 + 12, left = room > off + 768 ? room - off - 768 : 0;  // 768: alignment
+            const size_t best = kH1BitsBytes / (bit_stride + 4 * M1), fit = left / one < best ? left / one : best;
+            ctas = fit < 1 ? 1 : fit < size_t(kH1BitsCtas) ? int(fit) : kH1BitsCtas;
+        }
         bits = take(size_t(ctas) * bit_stride);
         pub = take(size_t(ctas) * 4 * M1);
         pub_piv = take(size_t(ctas) * 3 * 4);  // pivots (by the round's parity), lengths
         total = off;
+    }
+    // The least room that serves: the form with runs needs no more, nor do as
+    // many bit sets as can be used.
+    static size_t least(int64_t n, size_t base) {
+        const size_t runs = H1Layout(n, base, ~size_t(0), true).total, best = H1Layout(n, base).total;
+        return runs < best ? runs : best;
+    }
+    // The layout for a room of at least that: bit sets, unless it holds so few
+    // that one column in runs is faster (700 points in the plane, seven sets:
+    // 11.7 ms, 23.4 in runs; 800 in 8 dimensions, four: 169 and 148; 1024 in
+    // the plane, one: 193 and 46).
+    static H1Layout in_room(int64_t n, size_t base, size_t room) {
+        const H1Layout sets(n, base, room);
+        return sets.ctas > 0 && sets.ctas < kH1FewSets ? H1Layout(n, base, room, true) : sets;
     }
 };
 

@@ -178,10 +178,14 @@ def h1(pts: torch.Tensor):
     positive edge is paired, zero-length bars included; n <= 4096."""
     pts, n, d, ld = _points(pts)
     lib = _lib.load()
-    nbytes = int(lib.ph0_h1_workspace_bytes(n, d))
+    nbytes = int(lib.ph0_h1_workspace_best_bytes(n, d))
     if nbytes == 0:
         raise _lib.Ph0Error(3, f"ph0_h1_workspace_bytes(n={n}, d={d})")
-    ws = torch.empty(nbytes, dtype=torch.uint8, device=pts.device)
+    try:
+        ws = torch.empty(nbytes, dtype=torch.uint8, device=pts.device)
+    except torch.cuda.OutOfMemoryError:  # less serves too, with fewer columns at a time
+        nbytes = int(lib.ph0_h1_workspace_bytes(n, d))
+        ws = torch.empty(nbytes, dtype=torch.uint8, device=pts.device)
     nb = max(n * (n - 1) // 2 - (n - 1), 0)
     bars = torch.empty((max(nb, 1), _lib.H1_BAR_BYTES), dtype=torch.uint8, device=pts.device)
     st = _lib.H1Stats()
