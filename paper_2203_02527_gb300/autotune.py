@@ -2,14 +2,18 @@
 
 For a dimension d it times candidate settings on a synthetic cloud of that
 dimension (the stages they affect, with CUDA events between the stages of
-ph0_barcodes_profiled) and keeps the fastest:
+ph0_barcodes_profiled) and keeps the fastest, all on the forms that sort the
+edges or read their keys: the distance matrix of clouds of up to 2896 points,
+the built-in form there, has no settings.
   * dist_split16  -- rows of each 16 of a distance tile that take the running
                      sums on the binary64 units (the rest all in integers),
   * dist_tile     -- points per side of a distance tile (32, 64, 128),
   * sort_top_bits -- width of the single top radix pass (8 or 9),
   * packed_sort   -- the packed sort (1) or the short sort (0), timed on the
                      whole path (clouds from 2^22 edges up to 32768 points;
-                     in few dimensions the keys often do not pack).
+                     in few dimensions the keys often do not pack), where the
+                     faster one beats the library's own choice, which needs
+                     no sort at all on most clouds; else it is left out.
 Results are cached in a JSON file keyed by GPU name, dimension bucket and
 cloud-size bucket ($PH0_TUNING_CACHE, default ~/.cache/ph0_gb300/tuning.json):
 the best distance tile depends on how many tiles a cloud has to fill the GPU.  No setting
@@ -112,22 +116,28 @@ def tune(d: int, n: int = 8192, repeats: int = 3, seed: int = 7, verbose: bool =
         return best
 
     chosen = {"dist_split16": -1, "dist_tile": -1, "sort_top_bits": -1}
-    # distance kernel: split x tile
+    # distance kernel: split x tile (up to 2896 points that of the forms that
+    # sort, the only ones there that take the settings)
+    small = {"packed_sort": 0} if len(x) <= 2896 else {}
     dist = {}
     for split in (0, 4, 8, 12, 16):
         for tile in (64, 128):
-            t = dict(chosen, dist_split16=split, dist_tile=tile)
+            t = dict(chosen, dist_split16=split, dist_tile=tile, **small)
             dist[(split, tile)] = stage_ms(t, "dist_ms")
     (split, tile), _ = min(dist.items(), key=lambda kv: kv[1])
     chosen.update(dist_split16=split, dist_tile=tile)
     # top radix pass width (the short sort's)
     sort = {bits: stage_ms(dict(chosen, sort_top_bits=bits, packed_sort=0), "sort_ms") for bits in (8, 9)}
     chosen["sort_top_bits"] = min(sort, key=sort.get)
-    # the packed sort against the short sort, on the whole path
+    # the packed sort against the short sort, on the whole path; the built-in
+    # choice stays unless it sorts as well or loses to one of them
     whole = {}
     if len(x) * (len(x) - 1) // 2 >= 1 << 22 and len(x) <= 32768:
-        whole = {p: stage_ms(dict(chosen, packed_sort=p), "total_ms") for p in (0, 1)}
-        chosen["packed_sort"] = min(whole, key=whole.get)
+        whole = {p: stage_ms(dict(chosen, packed_sort=p), "total_ms") for p in (0, 1, -1)}
+        best = min((0, 1), key=whole.get)
+        sorts = ph0.barcodes(pts, ws, tuning=dict(chosen)).stats["sort_form"] != 3
+        if sorts or whole[best] < whole[-1]:
+            chosen["packed_sort"] = best
     if verbose:
         print({"d": d, "dist_ms": {f"{k[0]}/{k[1]}": v for k, v in dist.items()},
                "sort_ms": sort, "whole_ms": whole, "chosen": chosen})

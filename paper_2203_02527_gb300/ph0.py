@@ -114,7 +114,7 @@ def _tuning(n: int, d: int, tuning):
     t = autotune.cached(d, n)
     if not t:
         return None
-    if "packed_sort" in t:  # the choice between the sorts, where the call sorts
+    if t.get("packed_sort") in (0, 1):  # the choice between the sorts, where the call sorts
         t = {**t, "packed_sort": t["packed_sort"] + 2}
     return _lib.Tuning.make(**t)
 
