@@ -143,15 +143,29 @@ __host__ __device__ __forceinline__ void bit_range_f32(uint32_t bits, int32_t &l
 __host__ __device__ __forceinline__ uint32_t order_f32(uint32_t bits) {
     return bits ^ (bits >> 31 ? 0xffffffffu : 0x80000000u);
 }
-#ifdef __CUDACC__
 // Whether values between the two (as order_f32) are less than 2^32 units of
 // 2^g apart (both multiples of the unit, fewer than 2^53 of it).
-__device__ __forceinline__ bool within_32_bits(uint32_t lo, uint32_t hi, int32_t g) {
+__host__ __device__ __forceinline__ bool within_32_bits(uint32_t lo, uint32_t hi, int32_t g) {
     if (lo > hi) return true;  // no values
-    auto value = [](uint32_t o) { return double(__uint_as_float(o ^ (o >> 31 ? 0x80000000u : 0xffffffffu))); };
-    return value(hi) - value(lo) < __longlong_as_double((long long)(g + 32 + 1023) << 52);
-}
+    auto value = [](uint32_t o) {
+        const uint32_t b = o ^ (o >> 31 ? 0x80000000u : 0xffffffffu);
+#ifdef __CUDA_ARCH__
+        return double(__uint_as_float(b));
+#else
+        float x;
+        __builtin_memcpy(&x, &b, 4);
+        return double(x);
 #endif
+    };
+    const uint64_t limit = uint64_t(int64_t(g) + 32 + 1023) << 52;  // 2^(g + 32)
+#ifdef __CUDA_ARCH__
+    return value(hi) - value(lo) < __longlong_as_double((long long)limit);
+#else
+    double x;
+    __builtin_memcpy(&x, &limit, 8);
+    return value(hi) - value(lo) < x;
+#endif
+}
 
 // The integer X with x = X * 2^g (requires g <= lowest set bit of x and
 // |x| < 2^(g+63)).
