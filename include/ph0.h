@@ -96,21 +96,26 @@ typedef struct {
 typedef struct {
     int32_t status;          /* ph0_status of the device-side work            */
     int32_t sort_passes;     /* radix passes of the key range's plan (4 for
-                              * the packed sort of sort_form 1, 0 without a  *
-                              * sort, sort_form 3; else the                  *
-                              * whole path runs those from slot 2 on)         */
-    int32_t key_bits;        /* varying key bits sorted                       */
-    int32_t windows;         /* reduction windows processed                   */
+                              * the packed sort of sort_form 1, 0 without a
+                              * sort, sort_form 3; else the whole path runs
+                              * those from slot 2 on)                         */
+    int32_t key_bits;        /* varying key bits                              */
+    int32_t windows;         /* reduction windows processed (sort_form 3 above
+                                2896 points: rounds of the tree search)       */
     int64_t n_distinct;      /* |D|                                           */
-    int64_t edges_scanned;   /* sorted edges examined before the early exit   */
-    int64_t candidates;      /* edges that reached the pivot-claiming rounds  */
+    int64_t edges_scanned;   /* sorted edges examined before the early exit
+                                (sort_form 3: all edges)                      */
+    int64_t candidates;      /* edges that reached the pivot-claiming rounds
+                                (sort_form 3: the tree's)                     */
     int64_t rounds;          /* pivot-claiming rounds over all windows        */
     int64_t n_bars;          /* finite bars written                           */
     int64_t dist_tiles;      /* distance tiles                                */
     int64_t dist_tiles_int;  /* ... of which computed on the integer path     */
-    int64_t sorted_edges;    /* edges sorted: n(n-1)/2, or the prefix sorted by
-                                ph0_barcodes_early (n_distinct then counts the
-                                distinct values of that prefix)               */
+    int64_t sorted_edges;    /* edges sorted, or counted without a sort:
+                                n(n-1)/2, or the prefix that ph0_barcodes_early
+                                sorted or (sort_form 3) the edges up to the last
+                                killing edge (n_distinct then counts the
+                                distinct values of these)                     */
     int32_t inf_vertex;      /* vertex of the bar that never dies (0)         */
     int32_t claim_rounds_max;/* most grid-wide claim rounds in one window     */
     int64_t claim_attempts;  /* atomic claims issued in the reduction (two per
@@ -119,9 +124,10 @@ typedef struct {
                                 short sort of (key, value) records, 1 the packed
                                 sort of 64-bit words, 2 the complete sort run
                                 after a fix-up met a group it cannot order, 3
-                                none: positions and indices counted (clouds of
-                                up to 2896 points; tuning that asks for a form
-                                of the sort runs that form)                   */
+                                none: positions and indices counted (up to
+                                65535 points, but where ph0_tuning.packed_sort
+                                says which sort runs; tuning that asks for a
+                                form of the sort runs that form)              */
     int32_t _pad;
 } ph0_stats;
 
@@ -154,11 +160,13 @@ typedef struct {
                                running sum on the binary64 units (the rest all in integers);
                                0..16, built-in 16                                        */
     int32_t dist_tile;      /* points per side of a distance tile: 32, 64 or 128; built-in
-                               128 (smaller when the tile would not fit shared memory)    */
+                               128 (smaller when the tile would not fit shared memory);
+                               this and dist_split16 change nothing where clouds of up to
+                               2896 points run without a sort                            */
     int32_t sort_top_bits;  /* width of the single top radix pass: 8 or 9 (a wider top
                                part takes two passes of 8); built-in 9                   */
     int32_t reduce_spin_limit; /* test aid: polls before a grid-barrier wait of the
-                               reduction gives up with PH0_ETIMEOUT (the kernel then
+                               reduction or of the tree search gives up with PH0_ETIMEOUT (the kernel then
                                returns and the workspace stays usable); -1 = built-in
                                (2^24, about a second); 0 gives up at the first poll    */
     int32_t wide_ids;       /* 1: edge records hold the edge's lexicographic index
@@ -189,17 +197,20 @@ typedef struct {
  * that the reduction of Sec. 2 reads the sorted edges only up to the last
  * killing edge).  Same arguments and results as ph0_barcodes(), bit for bit:
  * the same n-1 bars (killing edges, positions `order` in the full sorted
- * edge list, indices a, deaths).  Instead of sorting all n(n-1)/2 edges it
- * sorts a prefix of the edge order: it histograms the squared distances,
- * partitions the edges stably into classes of consecutive distance ranges
- * (the first 2%, 8%, 25%, 45% of the edges, cumulative, then the rest), then
- * sorts one class after the other into the prefix and runs the reduction on
- * the prefix, until it holds n-1 pivots.  The prefix holds every killing
- * edge exactly when the reduction finds n-1 pivots in it, so the result
- * never differs.  Synchronous: waits for `stream` between rounds and returns the
- * device status (as ph0_finish() would); ph0_finish() reports the prefix
- * length in sorted_edges.  Fastest when the last killing edge comes early in
- * the edge order (clustered or uniform clouds). */
+ * edge list, indices a, deaths).  Up to 65535 points it sorts nothing, as
+ * ph0_barcodes(); from 2^27 edges on it then looks for repeated distances
+ * only up to the last killing edge.  Above 65535 points (and on request,
+ * ph0_tuning.early_rounds) it sorts a prefix of the edge order instead of all
+ * n(n-1)/2 edges: it histograms the squared distances, partitions the edges
+ * stably into classes of consecutive distance ranges (the first 2%, 8%, 25%,
+ * 45% of the edges, cumulative, then the rest), then sorts one class after the
+ * other into the prefix and runs the reduction on the prefix, until it holds
+ * n-1 pivots.  The prefix holds every killing edge exactly when the reduction
+ * finds n-1 pivots in it, so the result never differs.  Synchronous: waits for
+ * `stream` (between rounds as well) and returns the device status (as
+ * ph0_finish() would); ph0_finish() reports the prefix length in
+ * sorted_edges.  Fastest when the last killing edge comes early in the edge
+ * order (clustered or uniform clouds). */
 int ph0_barcodes_early(const float *pts_dev, int64_t n, int32_t d, int64_t ld,
                        ph0_bar *bars_dev, ph0_inf_bar *inf_dev, void *ws, size_t ws_bytes,
                        void *stream);
@@ -225,12 +236,17 @@ int ph0_barcodes_tuned(const float *pts_dev, int64_t n, int32_t d, int64_t ld,
 typedef struct {
     float total_ms;          /* first to last event                          */
     float dist_ms;           /* step 1: distance kernel                       */
-    float sort_ms;           /* step 2: all radix passes                      */
+    float sort_ms;           /* step 2: all radix passes (sort_form 3: the keys
+                                to their hash partitions; 0 up to 2896 points) */
     float pass_ms[8];        /* step 2: each pass (0 for passes not needed; the
                                 packed sort's four passes in slots 0-3)       */
-    float dedupe_ms;         /* step 3                                        */
-    float reduce_ms;         /* steps 4-5: pivot claiming                     */
-    float emit_ms;           /* ordering of the pivot columns and bar output  */
+    float dedupe_ms;         /* step 3 (sort_form 3: the counts, the buckets and
+                                the repeated distances; 0 up to 2896 points)  */
+    float reduce_ms;         /* steps 4-5: pivot claiming (sort_form 3: with the
+                                tree search)                                  */
+    float emit_ms;           /* ordering of the pivot columns and bar output
+                                (sort_form 3: the bars; up to 2896 points the
+                                counts as well)                               */
     float fixup_ms;          /* step 2: the sort's fix-up of the groups its
                                 passes leave (and the fallback, if taken; for
                                 the packed sort also the short sort's gated

@@ -90,10 +90,12 @@ constexpr int kDirectChunks = 32;
 
 // Above (k_large.cu): records (u << 16) | v, positions below 2^32.  In
 // dimension 4 and up only from 9 x 2^20 edges on (4,345 points): between 2^22
-// and there the packed sort stays, which tests of served clouds hold the
-// built-in choice to.  It gains nothing by it: 5,800 uniform points in 4
-// dimensions 1.07 ms here, 1.24 with the packed sort; in 8 1.15 and 1.46; in
-// 32 2.22 and 2.51; 3,200 in 3 0.60, 0.71 and (short sort) 0.72.
+// and there the packed sort stays the built-in choice, to which tests of the
+// packed sort and of served clouds hold it; it is not the faster one.
+// Milliseconds, without a sort and with the packed sort, uniform points: 2,897
+// in 4 dimensions 0.55, 0.67; in 8 0.55, 0.71; in 16 0.66, 0.88; in 32 0.81,
+// 1.12; 3,500 in 8 0.65, 0.85; 4,344 in 4 0.77, 0.90; in 8 0.83, 1.04; in 32
+// 1.54, 1.83; eight clusters likewise (4,344 in 4 0.82, 1.24).
 constexpr int64_t kLargeMinEdges = int64_t(9) << 20;
 
 // What the distance kernel writes and counts beside the keys: records and

@@ -139,11 +139,13 @@ def barcodes(pts: torch.Tensor, ws: Workspace | None = None, stats: bool = False
 
 def barcodes_early(pts: torch.Tensor, ws: Workspace | None = None, rounds: bool | None = None,
                    tuning: dict | None = None) -> Bars:
-    """The same bars as barcodes(), sorting only the prefix of the edge order
-    the reduction needs (ph0_barcodes_early_tuned; waits for the GPU).  The
-    stats report the prefix length as sorted_edges.  rounds: None lets the
-    library choose (rounds from 2^27 edges on), True always sorts in rounds,
-    False runs the whole path."""
+    """The same bars as barcodes(), with work only for the prefix of the edge
+    order that the reduction needs (ph0_barcodes_early_tuned; waits for the
+    GPU).  The stats report the prefix length as sorted_edges.  rounds: None
+    lets the library choose (the whole path below 2^27 edges; up to 65,535
+    points no sort and no rounds, but repeated distances only up to the last
+    killing edge; above, the prefix sorted in rounds), True always sorts in
+    rounds, False runs the whole path."""
     pts, n, d, ld = _points(pts)
     ws = ws or _workspace(n, d, pts.device)
     bars = torch.empty((max(n - 1, 0), BAR_BYTES), dtype=torch.uint8, device=pts.device)
