@@ -1198,12 +1198,15 @@ cudaError_t launch_direct(void *ws, const Layout &L, const float *pts, int64_t n
     if (e == cudaSuccess && after_tree) e = cudaEventRecord(after_tree, s);
     if (e != cudaSuccess) return e;
 
-    // (the 48 KB a kernel has without it include its static shared memory, so
-    // 2,451 points already need it)
+    // a kernel has 48 KB less its static shared memory without it (2,451
+    // points need more); asked for with a margin, but not by the smallest
+    // calls, which the host's share bounds
     constexpr size_t kPerPoint = 20;
-    e = smem_limit<kPerPoint * kDirectMaxN>(k_direct_count);
-    if (e != cudaSuccess) return e;
     const size_t csm = kPerPoint * size_t(n);
+    if (csm > 40 * 1024) {
+        e = smem_limit<kPerPoint * kDirectMaxN>(k_direct_count);
+        if (e != cudaSuccess) return e;
+    }
     // two CTAs per SM, or fewer with at least 2048 edges each
     int grid = int((L.m + 2047) / 2048);
     if (grid > 2 * sm_count()) grid = 2 * sm_count();
