@@ -68,7 +68,7 @@ constexpr int kLgTreeThreads = 512;
 constexpr int kLgRun = 2048;                   // tree edges sorted by a CTA
 constexpr int kLgHot = 8192;                   // longest tree edges whose counts stay in shared memory
 constexpr int kLgCountThreads = 512;
-constexpr int kLgRuns = 256;                   // runs of equal tree edges remembered by a CTA
+constexpr int kLgRuns = 512;                   // runs of equal tree edges remembered by a CTA
 constexpr int kLgLutBits = 11, kLgLut = 1 << kLgLutBits;
 constexpr int kLgSubCtas = 4;                  // CTAs per partition
 // keys of a tile in one partition that only repeated distances explain: the
@@ -325,33 +325,35 @@ __device__ __forceinline__ void lg_list_put(const LgArgs &A, const uint64_t (&ke
     }
 }
 
-// The list alone (the early path, whose keys are not all moved).
-__global__ void __launch_bounds__(1024, 2) k_large_list(const LgArgs A) {
-    __shared__ uint32_t s_n, s_base;
-    if (lg_all_equal(A)) return;
+// The list alone (the early path, whose keys are not all moved).  ZEROS: they
+// are listed too.
+template <bool ZEROS>
+__device__ __forceinline__ void lg_list_all(const LgArgs &A, uint32_t *s_n, uint32_t *s_base) {
     constexpr int kU = 8;
-    const uint64_t lo = A.h->lg_lo, limit = A.h->lg_limit;
+    const uint64_t lo = ZEROS ? 0 : 1, limit = A.h->lg_limit;
     const int64_t stride = int64_t(gridDim.x) * 1024;
-    if (threadIdx.x == 0) s_n = 0;
-    __syncthreads();
     for (int64_t b = int64_t(blockIdx.x) * 1024; b < A.m; b += kU * stride) {  // the same for a whole CTA
         const int64_t e0 = b + threadIdx.x;
         uint64_t key[kU];
-#pragma unroll
-        for (int q = 0; q < kU; ++q) key[q] = e0 + q * stride < A.m ? A.mat[e0 + q * stride] : kNone;
         uint32_t mine = 0;
 #pragma unroll
-        for (int q = 0; q < kU; ++q) mine += key[q] < limit;
-        if (lo && mine) {
+        for (int q = 0; q < kU; ++q) key[q] = e0 + q * stride < A.m ? A.mat[e0 + q * stride] : kNone;
 #pragma unroll
-            for (int q = 0; q < kU; ++q) mine -= key[q] < lo;
-        }
-        const uint32_t at = lg_rank(mine, &s_n);
+        for (int q = 0; q < kU; ++q) mine += key[q] < limit && key[q] >= lo;
+        const uint32_t at = lg_rank(mine, s_n);
         __syncthreads();
-        lg_room(&A.h->lg_list, &s_n, &s_base);
+        lg_room(&A.h->lg_list, s_n, s_base);
         __syncthreads();
-        if (mine) lg_list_put<kU>(A, key, e0, stride, lo, limit, s_base + at);
+        if (mine) lg_list_put<kU>(A, key, e0, stride, lo, limit, *s_base + at);
     }
+}
+__global__ void __launch_bounds__(1024, 2) k_large_list(const LgArgs A) {
+    __shared__ uint32_t s_n, s_base;
+    if (lg_all_equal(A)) return;
+    if (threadIdx.x == 0) s_n = 0;
+    __syncthreads();
+    if (A.h->lg_lo == 0) lg_list_all<true>(A, &s_n, &s_base);
+    else lg_list_all<false>(A, &s_n, &s_base);
 }
 
 // ----------------------------------------------------- moving keys by hash ---
@@ -712,7 +714,7 @@ __global__ void __launch_bounds__(kLgRepThreads, 2) k_large_repeats(const LgArgs
         // the last tree edge) how often each comes again, of one part of the
         // hash's values at a time (all at first; a part whose keys do not fit
         // is taken in two halves, which a one-to-one hash ends at one key).
-        // 50,000 points, a fifth of them equal: 18.3 ms for all buckets, 56.8
+        // 50,000 points, a fifth of them equal: 16.9 ms for all buckets, 56.8
         // when the number of parts followed a bucket's size; half of them on a
         // line, at 300 places: 4.8 and 9.8.  (Of 6,784 slots 64 probes fail
         // from about 5,500 keys on; with 128 the first of these took 21.8.)
@@ -724,6 +726,7 @@ __global__ void __launch_bounds__(kLgRepThreads, 2) k_large_repeats(const LgArgs
             clear();
             if (tid == 0) s_ns = 0;
             uint32_t more = 0;  // beyond the first of each distance
+            bool placed = false;
             __syncthreads();
             for (uint32_t i0 = tid; i0 < size; i0 += kU * kLgRepThreads) {
                 uint64_t key[kU];
@@ -748,15 +751,18 @@ __global__ void __launch_bounds__(kLgRepThreads, 2) k_large_repeats(const LgArgs
                     }
                     if (old == tag) {
                         ++more;
-                        if (key[q] <= top) atomicAdd(occ + slot, 1u);
+                        if (key[q] <= top) {
+                            atomicAdd(occ + slot, 1u);
+                            placed = true;
+                        }
                     }
                     if (pr == kLgProbes) *(volatile uint32_t *)&s_ns = 1;
                 }
             }
-            __syncthreads();
+            placed = __syncthreads_or(placed);
             const bool full = s_ns != 0;
-            if (!full) {
-                dups += more;
+            if (!full) dups += more;
+            if (!full && placed) {
                 for (int i = tid; i < kLgSlots; i += kLgRepThreads)
                     if (occ[i]) atomicAdd(A.dup + lg_place(A.skey, 0, np - 1, tab[i] - 1), occ[i]);
             }
@@ -1250,8 +1256,92 @@ static_assert(32 * kLgRun >= kMaxN - 1, "a lane per run");
 // in the rows of the first copies), which the table counts; the others are
 // searched for in the run, and the gap between two of its edges is remembered
 // with the edges counted there.  20,000 points of two kinds, whose 200M edges
-// all come here: 1.0 ms; 64 with a search over the tree's edges and three
+// all come here: 0.8 ms; 64 with a search over the tree's edges and three
 // atomics on the L2 cache's words for every edge.
+struct LgRuns {
+    // key (kNone: a free slot), first and end (in the high half) of a run,
+    // number of its last edge (kUnknown until these are written), edges behind
+    unsigned long long key[kLgRuns];
+    uint32_t run[kLgRuns], last[kLgRuns], late[kLgRuns];
+    static constexpr uint32_t kUnknown = 0xffffffffu;
+    static_assert(kMaxN <= 65536, "places below 2^16");
+};
+struct LgGap {  // a thread's: key, (u, v) from and to, edges counted there, place
+    uint64_t key = kNone;
+    uint32_t from = 0, to = 0, n = 0;
+    int s = 0;
+    __device__ void flush(const LgArgs &A, uint32_t *s_cnt, int base) {
+        if (n) atomicAdd(s >= base ? s_cnt + (s - base) : A.cnt + s, n);
+        n = 0;
+    }
+};
+// An edge as long as tree edge t (-1: not known, nor whether there is one)
+// that is not known to lie behind its run; h, known: the key's slot in the
+// table and its run's last edge.  Not inlined: the counting loop holds eight
+// copies of what is, and most warps come by here now and then (20,000 random
+// whole numbers on a line, all counts: 0.63 ms inlined, 0.46).
+__device__ __noinline__ void lg_tie(const LgArgs &A, LgRuns *runs, uint32_t *s_cnt, LgGap &gap, uint64_t key, int64_t e,
+                                    int t, uint32_t h, uint32_t known) {
+    const int np = A.n - 1, base = np - (np < kLgHot ? np : kLgHot);
+    int end;
+    if (known != LgRuns::kUnknown) {
+        __threadfence_block();
+        const uint32_t run = *(volatile uint32_t *)&runs->run[h];
+        t = int(run & 0xffffu);
+        end = int(run >> 16);
+    } else {
+        if (t < 0) {
+            t = lg_place(A.skey, 0, base, key);
+            if (A.skey[t] != key) {
+                atomicAdd(A.cnt + t, 1u);
+                return;
+            }
+        }
+        // the run's end: steps of 1, 2, 4, ... from its first
+        end = t + 1;
+        if (end < np && A.skey[end] == key) {
+            int step = 1;
+            while (end + step < np && A.skey[end + step] == key) {
+                end += step;
+                step *= 2;
+            }
+            int hi = end + step < np ? end + step : np;  // [end] is of the run, [hi] is not
+            while (end + 1 < hi) {
+                const int mid = (end + hi) >> 1;
+                if (A.skey[mid] == key) end = mid;
+                else hi = mid;
+            }
+            end = hi;
+        }
+        const uint32_t last = A.suv[end - 1], elast = uint32_t(edge_index(A.n, last >> 16, last & 0xffffu));
+        if (atomicCAS(&runs->key[h], (unsigned long long)kNone, (unsigned long long)key) == kNone) {
+            *(volatile uint32_t *)&runs->run[h] = uint32_t(t) | uint32_t(end) << 16;
+            __threadfence_block();
+            *(volatile uint32_t *)&runs->last[h] = elast;  // from now on the run is known
+        }
+        if (uint32_t(e) > elast) {
+            atomicAdd(A.late + end, 1u);
+            return;
+        }
+    }
+    uint32_t u, v;
+    edge_uv(e, A.n, u, v);
+    const uint32_t uv = (u << 16) | v;
+    if (key != gap.key || uv < gap.from || uv > gap.to) {
+        gap.flush(A, s_cnt, base);
+        int lo = t, hi = end - 1;  // suv[end - 1] >= uv
+        while (lo < hi) {
+            const int mid = (lo + hi) >> 1;
+            if (A.suv[mid] < uv) lo = mid + 1;
+            else hi = mid;
+        }
+        gap.key = key;
+        gap.s = lo;
+        gap.from = lo > t ? A.suv[lo - 1] + 1 : 0u;
+        gap.to = A.suv[lo];
+    }
+    ++gap.n;
+}
 // PREFIX (the early path): the keys counted are also kept for step 3, with
 // the histogram of their partitions.
 template <bool PREFIX>
@@ -1268,17 +1358,11 @@ __global__ void __launch_bounds__(kLgCountThreads, 2) k_large_count(const LgArgs
     // with a few keys to place 13 steps: 3.0 ms instead of 1.15 at 30,000
     // points in eight clusters, 450M keys)
     __shared__ uint16_t s_lut[kLgLut + 2];
-    // runs of equal tree edges: key (kNone: a free slot), first and end,
-    // number of the last edge (kUnknown until all three are written), edges
-    // behind it
-    constexpr uint32_t kUnknown = 0xffffffffu;
-    __shared__ unsigned long long s_rkey[kLgRuns];
-    __shared__ int s_rfirst[kLgRuns], s_rend[kLgRuns];
-    __shared__ uint32_t s_rlast[kLgRuns], s_late[kLgRuns];
+    __shared__ LgRuns s_runs;
     for (int i = tid; i < kLgRuns; i += kLgCountThreads) {
-        s_rkey[i] = kNone;
-        s_rlast[i] = kUnknown;
-        s_late[i] = 0;
+        s_runs.key[i] = kNone;
+        s_runs.last[i] = LgRuns::kUnknown;
+        s_runs.late[i] = 0;
     }
     for (int i = tid; i < hot; i += kLgCountThreads) {
         s_key[i] = A.skey[base + i];
@@ -1317,78 +1401,18 @@ __global__ void __launch_bounds__(kLgCountThreads, 2) k_large_count(const LgArgs
     }
     __syncthreads();
     if constexpr (!PREFIX) lg_reps(A, uint32_t(gtid), uint32_t(gthreads));
-    uint64_t gap_key = kNone;
-    uint32_t gap_from = 0, gap_to = 0, gap_n = 0;
-    int gap_s = 0;
-    auto flush = [&]() {
-        if (gap_n) atomicAdd(gap_s >= base ? s_cnt + (gap_s - base) : A.cnt + gap_s, gap_n);
-        gap_n = 0;
-    };
-    // a key as long as tree edge t (-1: not known, nor whether there is one)
+    LgGap gap;
     auto tie = [&](uint64_t key, int64_t e, int t) {
-        uint32_t h = (uint32_t(key >> 32) * 0x9E3779B9u + uint32_t(key) * 0x7F4A7C15u) >> 24, known = kUnknown;
-        static_assert(kLgRuns == 256, "eight bits of the hash");
-        for (int pr = 0; pr < 4; ++pr) {
-            const uint64_t k = *(volatile uint64_t *)&s_rkey[h];
-            if (k == key) known = *(volatile uint32_t *)&s_rlast[h];
+        uint32_t h = (uint32_t(key >> 32) * 0x9E3779B9u + uint32_t(key) * 0x7F4A7C15u) >> 23, known = LgRuns::kUnknown;
+        static_assert(kLgRuns == 512, "nine bits of the hash");
+        for (int pr = 0; pr < 2; ++pr) {
+            const uint64_t k = *(volatile uint64_t *)&s_runs.key[h];
+            if (k == key) known = *(volatile uint32_t *)&s_runs.last[h];
             if (k == key || k == kNone) break;
             h = (h + 1) & (kLgRuns - 1);
         }
-        int end;
-        if (known != kUnknown) {
-            if (uint32_t(e) > known) {
-                atomicAdd(s_late + h, 1u);
-                return;
-            }
-            __threadfence_block();
-            t = *(volatile int *)&s_rfirst[h];
-            end = *(volatile int *)&s_rend[h];
-        } else {
-            if (t < 0) {
-                t = lg_place(A.skey, 0, base, key);
-                if (A.skey[t] != key) {
-                    atomicAdd(A.cnt + t, 1u);
-                    return;
-                }
-            }
-            end = t + 1;
-            if (end < np && A.skey[end] == key) {
-                int hi = np;
-                while (end < hi) {
-                    const int mid = (end + hi) >> 1;
-                    if (A.skey[mid] <= key) end = mid + 1;
-                    else hi = mid;
-                }
-            }
-            const uint32_t last = A.suv[end - 1], elast = uint32_t(edge_index(A.n, last >> 16, last & 0xffffu));
-            if (atomicCAS(&s_rkey[h], (unsigned long long)kNone, (unsigned long long)key) == kNone) {
-                s_rfirst[h] = t;
-                s_rend[h] = end;
-                __threadfence_block();
-                *(volatile uint32_t *)&s_rlast[h] = elast;  // from now on the run is known
-            }
-            if (uint32_t(e) > elast) {
-                atomicAdd(A.late + end, 1u);
-                return;
-            }
-        }
-        uint32_t u, v;
-        edge_uv(e, A.n, u, v);
-        const uint32_t uv = (u << 16) | v;
-        if (key != gap_key || uv < gap_from || uv > gap_to) {
-            flush();
-            int lo = t, hi = end - 1;  // suv[end - 1] >= uv
-            while (lo < hi) {
-                const int mid = (lo + hi) >> 1;
-                if (A.suv[mid] < uv) lo = mid + 1;
-                else hi = mid;
-            }
-            gap_key = key;
-            gap_s = lo;
-            gap_from = lo > t ? A.suv[lo - 1] + 1 : 0u;
-            gap_to = A.suv[lo];
-        }
-        ++gap_n;
+        if (known != LgRuns::kUnknown && uint32_t(e) > known) atomicAdd(&s_runs.late[h], 1u);
+        else lg_tie(A, &s_runs, s_cnt, gap, key, e, t, h, known);
     };
     auto take = [&](uint64_t key, int64_t e) {
         if (key > top) return;
@@ -1426,7 +1450,7 @@ __global__ void __launch_bounds__(kLgCountThreads, 2) k_large_count(const LgArgs
             }
         }
     }
-    flush();
+    gap.flush(A, s_cnt, base);
     __syncthreads();
     if constexpr (PREFIX)
         for (int i = tid; i < kLgParts; i += kLgCountThreads)
@@ -1434,7 +1458,7 @@ __global__ void __launch_bounds__(kLgCountThreads, 2) k_large_count(const LgArgs
     for (int i = tid; i < hot; i += kLgCountThreads)
         if (s_cnt[i]) atomicAdd(A.cnt + base + i, s_cnt[i]);
     for (int i = tid; i < kLgRuns; i += kLgCountThreads)
-        if (s_late[i]) atomicAdd(A.late + s_rend[i], s_late[i]);
+        if (s_runs.late[i]) atomicAdd(A.late + (s_runs.run[i] >> 16), s_runs.late[i]);
 }
 
 // Each CTA adds up the counts before its 1024 tree edges, then writes their
