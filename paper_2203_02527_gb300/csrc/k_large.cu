@@ -85,6 +85,9 @@ struct LgRepeat {
 struct LgArgs {
     int64_t m;
     int n, nsub;
+    const float *pts;          // [n][ld] coordinates, d of each row (the tree alone)
+    int64_t ld;
+    int d;
     const uint64_t *mat;       // [m] key of edge e
     uint64_t *part, *bkt;      // [m] keys by partition, by bucket
     LgRepeat *rep;             // [m / 2] records of crowded tiles (in bkt's place, read before it is filled)
@@ -171,8 +174,8 @@ __device__ __forceinline__ int lg_place(const uint64_t *skey, int lo, int hi, ui
 // a bin of key >> 48 (sixteen to the octave) and within it one of the next 15
 // bits, so that about kLgListPerPoint n edges lie below; and the bin below
 // which at most a sixteenth of those do (for the rounds on the list).  More
-// zeros than that (copies of a few points): the list leaves them out, and the
-// tree's first round, over all keys, joins the points that are equal.
+// zeros than an eighth of that (copies of points): the list leaves them out,
+// and the tree joins the points that are equal by their coordinates.
 __host__ __device__ __forceinline__ int lg_samples(int n) {
     // four keys per point, so that a few hundred lie below the threshold
     const int S = 4 * n;
@@ -221,13 +224,13 @@ __global__ void __launch_bounds__(1024) k_large_prep(const LgArgs A) {
             else if ((k >> 48) == prefix) atomicAdd(s_bin + ((k >> 33) & 32767), 1u);
         }
         __syncthreads();
-        if (prefix == 0 && s_bin[0] > uint32_t(want)) {  // (few clouds; the same for all threads)
+        if (prefix == 0 && s_bin[0] > uint32_t(want) / 8) {  // (few clouds; the same for all threads)
             if (level == 0) {
                 for (uint32_t i = tid; i < uint32_t(S); i += 1024)
                     if (A.lkey[i] == 0) atomicAdd(&s_zeros, 1u);
             }
             __syncthreads();
-            lo = s_zeros > uint32_t(want);
+            lo = s_zeros > uint32_t(want) / 8;
             if (tid == 0 && lo) s_bin[0] -= s_zeros;
             __syncthreads();
         }
@@ -795,7 +798,7 @@ __device__ __forceinline__ uint32_t lg_other(const LgArgs &A, uint32_t c) {
 // Edges of equal keys meet at one component in their millions (two distances
 // between 20,000 points: 10^8 edges for two components), so an atomic is only
 // made by an edge that comes before the one found so far: the tree of that
-// cloud takes 1.2 ms, 13.0 with every edge's atomics.
+// cloud takes 0.55 ms, 13.0 with every edge's atomics.
 __device__ __forceinline__ void lg_first(uint32_t *best, uint32_t uv) {
     if (uv < __ldcg(best)) atomicMin(best, uv);
 }
@@ -817,6 +820,67 @@ __device__ __forceinline__ void lg_tile(int64_t w, int64_t T, int &u0, int &v0) 
     while (r < T - 1 && (r + 1) * T - (r + 1) * r / 2 <= w) ++r;
     u0 = int(r) * 128;
     v0 = int(r + w - (r * T - r * (r - 1) / 2)) * 128;
+}
+
+// The tree's edges between equal points, (a, v) for the first a of each group
+// of them and its others: the points by a hash table of their coordinates, in
+// the candidates' place (for clouds with more zeros than the list has room
+// for; a round over all keys did the same: the tree of 20,000 points of two
+// kinds 1.2 ms, 0.55 this way; of 50,000 with 2,500 equal 13.3, 0.87).
+// False when a wait ran out.
+__device__ __noinline__ bool lg_join_equal(const LgArgs &A, int *s_ok) {
+    const int n = A.n, lane = threadIdx.x & 31;
+    const int gthreads = gridDim.x * kLgTreeThreads, gtid = blockIdx.x * kLgTreeThreads + threadIdx.x;
+    uint32_t slots = 2;
+    while (slots < 2u * uint32_t(n)) slots *= 2;  // two tables of at most 2^17, m > 2^22 entries of room
+    uint32_t *tab = A.cand, *low = A.cand + slots;
+    for (uint32_t i = uint32_t(gtid); i < 2 * slots; i += uint32_t(gthreads)) tab[i] = 0xffffffffu;
+    if (!grid_barrier(A.h, s_ok, A.spin_limit)) return false;
+    // by bits, the two zeros alike: whatever is not a number ends in a status anyway
+    auto bits = [&](int v, int k) {
+        const uint32_t b = __float_as_uint(A.pts[int64_t(v) * A.ld + k]);
+        return b << 1 ? b : 0u;
+    };
+    for (int v = gtid; v < n; v += gthreads) {
+        uint32_t x = 0;
+        for (int k = 0; k < A.d; ++k) {
+            x = (x ^ bits(v, k)) * 0x9E3779B1u;
+            x ^= x >> 15;
+        }
+        uint32_t at = x & (slots - 1);
+        for (;;) {  // at most half the slots fill
+            uint32_t old = __ldcg(tab + at);
+            if (old == 0xffffffffu) old = atomicCAS(tab + at, 0xffffffffu, uint32_t(v));
+            if (old == 0xffffffffu) break;
+            int k = 0;
+            while (k < A.d && bits(int(old), k) == bits(v, k)) ++k;
+            if (k == A.d) break;
+            at = (at + 1) & (slots - 1);
+        }
+        A.buv[v] = at;
+        lg_first(low + at, uint32_t(v));
+    }
+    if (!grid_barrier(A.h, s_ok, A.spin_limit)) return false;
+    for (int v0 = gtid - lane; v0 < n; v0 += gthreads) {
+        const int v = v0 + lane;
+        uint32_t a = uint32_t(v);
+        if (v < n) {
+            a = __ldcg(low + A.buv[v]);
+            A.buv[v] = 0xffffffffu;
+            A.comp[v] = A.parent[v] = a;
+        }
+        const bool take = a != uint32_t(v);
+        const unsigned who = __ballot_sync(0xffffffffu, take);
+        if (!who) continue;
+        uint32_t j = 0;
+        if (lane == 0) j = atomicAdd(&A.h->lg_tree, uint32_t(__popc(who)));
+        j = __shfl_sync(0xffffffffu, j, 0) + __popc(who & ((1u << lane) - 1u));
+        if (take && j < uint32_t(n)) {
+            A.tkey[j] = 0;
+            A.tuv[j] = (a << 16) | uint32_t(v);
+        }
+    }
+    return grid_barrier(A.h, s_ok, A.spin_limit);
 }
 
 // Boruvka's rounds, a grid barrier between the steps of a round: every
@@ -853,8 +917,11 @@ __global__ void __launch_bounds__(kLgTreeThreads, 2) k_large_tree(const LgArgs A
     uint32_t joined = 0, rounds = 0, passes = 0;
     uint32_t live = uint32_t(gtid) < list ? (list - gtid - 1) / gthreads + 1 : 0u;  // entries of this thread
     const uint64_t first = __ldcg(&h->lg_first);
-    // (a list without zeros serves once equal points are joined)
-    bool later = list > 0 && __ldcg(&h->lg_lo) != 0, on_list = list > 0 && !later;
+    bool on_list = list > 0;
+    if (__ldcg(&h->lg_lo) != 0) {  // the list has no zeros: equal points first
+        if (!lg_join_equal(A, &s_ok)) return;
+        joined = __ldcg(&h->lg_tree);
+    }
     const int64_t T = (n + 127) / 128, tiles = T * (T + 1) / 2;
     const int warps = gthreads >> 5, gwarp = gtid >> 5;
     while (joined < uint32_t(n - 1)) {
@@ -1178,8 +1245,6 @@ __global__ void __launch_bounds__(kLgTreeThreads, 2) k_large_tree(const LgArgs A
             }
             on_list = false;
         }
-        if (later) on_list = true;
-        later = false;
         joined = now;
     }
     if (gtid == 0) {
@@ -1571,6 +1636,8 @@ LgArgs large_args(void *ws, const Layout &L, ph0_bar *bars, ph0_inf_bar *inf, ui
     const size_t n = size_t(L.n);
     A.m = L.m;
     A.n = int(L.n);
+    A.pts = nullptr;
+    A.ld = A.d = 0;
     A.nsub = large_nsub(L.m);
     A.mat = at<uint64_t>(ws, L.key[0]);
     // prefix: the kept keys in key[1], by partition in the value buffers, by
@@ -1645,8 +1712,11 @@ cudaError_t launch_large_tree(void *ws, const Layout &L, const float *pts, int64
                               int split16, int tile, uint32_t spin_limit, bool prefix, const uint32_t **records,
                               cudaStream_t s, cudaEvent_t after_dist, cudaEvent_t after_part) {
     size_t zero, zero_end;
-    const LgArgs A = large_args(ws, L, nullptr, nullptr, spin_limit, prefix, zero, zero_end);
+    LgArgs A = large_args(ws, L, nullptr, nullptr, spin_limit, prefix, zero, zero_end);
     if (A.n == 0) return cudaErrorInvalidValue;
+    A.pts = pts;
+    A.ld = ld;
+    A.d = d;
     *records = A.suv;
     cudaError_t e = cudaMemsetAsync(at<char>(ws, L.hdr), 0, sizeof(Header), s);
     if (e == cudaSuccess) e = cudaMemsetAsync(at<char>(ws, zero), 0, zero_end - zero, s);

@@ -45,6 +45,11 @@ def line_and_plane(n, places):
     return x
 
 
+def signed(x):
+    """Some of the zeros negative."""
+    return np.where((x == 0) & (np.random.default_rng(76).random(x.shape) < 0.5), np.float32(-0.0), x)
+
+
 CLOUDS = {
     "two_points": lambda: halves(N, True),
     "two_points_in_order": lambda: halves(N, False),
@@ -58,6 +63,8 @@ CLOUDS = {
     "uniform_50000": lambda: hot(50000, 1),
     "one_point": lambda: np.full((N, 2), 0.25, np.float32),
     "two_points_5000": lambda: halves(5000, True),
+    "signed_zeros_5000": lambda: signed(halves(5000, True)),
+    "copies_4_5000": lambda: copies(5000, 4),
     "copies_64_5000": lambda: copies(5000, 64),
     "one_point_5000": lambda: np.full((5000, 2), 0.25, np.float32),
 }
