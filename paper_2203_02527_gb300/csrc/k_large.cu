@@ -555,6 +555,20 @@ __device__ __forceinline__ void lg_reps(const LgArgs &A, uint32_t first, uint32_
     }
 }
 
+// The slot of a tag that is there already, -2 when it was put there, -1 when
+// kLgProbes slots from the first were others'.  (Not inlined: the loop that
+// looks at a table of few distances holds eight copies of what is.)
+__device__ __noinline__ int lg_insert(unsigned long long *tab, uint32_t slot, unsigned long long tag) {
+    for (int pr = 0; pr < kLgProbes; ++pr) {
+        unsigned long long old = *(volatile unsigned long long *)(tab + slot);
+        if (old == 0) old = atomicCAS(tab + slot, 0ull, tag);
+        if (old == 0) return -2;
+        if (old == tag) return int(slot);
+        slot = slot + 1 == kLgSlots ? 0 : slot + 1;
+    }
+    return -1;
+}
+
 // Repeated distances, a bucket at a time.  Few repeats: a bit table in shared
 // memory, one bit per key (10,240 keys set 1.6% of 655,360 bits); a key that
 // finds its bit set is a suspect, and a second look over the bucket's keys
@@ -717,10 +731,10 @@ __global__ void __launch_bounds__(kLgRepThreads, 2) k_large_repeats(const LgArgs
         // the last tree edge) how often each comes again, of one part of the
         // hash's values at a time (all at first; a part whose keys do not fit
         // is taken in two halves, which a one-to-one hash ends at one key).
-        // 50,000 points, a fifth of them equal: 16.9 ms for all buckets, 56.8
+        // 50,000 points, a fifth of them equal: 11.1 ms for all buckets, 59.8
         // when the number of parts followed a bucket's size; half of them on a
         // line, at 300 places: 4.8 and 9.8.  (Of 6,784 slots 64 probes fail
-        // from about 5,500 keys on; with 128 the first of these took 21.8.)
+        // from about 5,500 keys on; 128 took a third longer.)
         unsigned long long *tab = reinterpret_cast<unsigned long long *>(s_tab);
         uint32_t *occ = reinterpret_cast<uint32_t *>(tab + kLgSlots);
         int bits = 0;
@@ -743,23 +757,17 @@ __global__ void __launch_bounds__(kLgRepThreads, 2) k_large_repeats(const LgArgs
                     if (bits && x >> (64 - bits) != part) continue;
                     uint32_t slot = __umulhi(uint32_t(x) * 0x9E3779B9u, uint32_t(kLgSlots));
                     const unsigned long long tag = key[q] + 1;
-                    unsigned long long old = *(volatile unsigned long long *)(tab + slot);
-                    int pr = 0;
-                    while (old != tag) {
-                        if (old == 0 && (old = atomicCAS(tab + slot, 0ull, tag)) == 0) break;
-                        if (old == tag) break;
-                        slot = slot + 1 == kLgSlots ? 0 : slot + 1;
-                        if (++pr == kLgProbes) break;
-                        old = *(volatile unsigned long long *)(tab + slot);
+                    if (*(volatile unsigned long long *)(tab + slot) != tag) {
+                        const int to = lg_insert(tab, slot, tag);
+                        if (to == -1) *(volatile uint32_t *)&s_ns = 1;
+                        if (to < 0) continue;
+                        slot = uint32_t(to);
                     }
-                    if (old == tag) {
-                        ++more;
-                        if (key[q] <= top) {
-                            atomicAdd(occ + slot, 1u);
-                            placed = true;
-                        }
+                    ++more;
+                    if (key[q] <= top) {
+                        atomicAdd(occ + slot, 1u);
+                        placed = true;
                     }
-                    if (pr == kLgProbes) *(volatile uint32_t *)&s_ns = 1;
                 }
             }
             placed = __syncthreads_or(placed);
