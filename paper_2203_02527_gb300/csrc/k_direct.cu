@@ -486,9 +486,16 @@ __device__ void direct_repeats(const DirectArgs &A, unsigned char *s_dyn, int fi
         const bool stored = cnt <= uint32_t(A.bcap);
         if (stored) {
             const uint64_t *keys = A.bkeys + size_t(b) * A.bcap;
-            for (uint32_t i = tid; i < cnt; i += T) {
-                const uint64_t k = keys[i], x = key_hash(k);
-                if (within(x)) insert(k, x);
+            if (bits == 0) {  // nearly always
+                for (uint32_t i = tid; i < cnt; i += T) {
+                    const uint64_t k = keys[i];
+                    insert(k, key_hash(k));
+                }
+            } else {
+                for (uint32_t i = tid; i < cnt; i += T) {
+                    const uint64_t k = keys[i], x = key_hash(k);
+                    if (within(x)) insert(k, x);
+                }
             }
         } else {
             const uint32_t n = uint32_t(A.n), items = n * n;

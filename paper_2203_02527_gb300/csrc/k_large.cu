@@ -12,8 +12,9 @@
 //   k_large_move<0>     the keys by partition; the edges below the threshold
 //                       as a list; a tile of few distances keeps one key of
 //                       each and records how many more it stands for
-//   k_large_tree        the tree by Boruvka's rounds (cooperative): on the
-//                       list while it joins components, then on all keys
+//   k_large_tree        the tree by Boruvka's rounds (cooperative): equal
+//                       points first where there are many, then on the list
+//                       while it joins components, then on all keys
 //   k_large_runs, merge the tree's edges in order
 //   k_reduce            their columns' pivot rows (k_reduce.cu)
 //   k_large_count       every edge up to the last killing edge counted at its
@@ -21,20 +22,25 @@
 //   k_large_sub,        the partitions' keys by bucket of about ten thousand
 //   k_large_move<1>
 //   k_large_repeats     step 3: repeated distances, a bucket at a time in a
-//                       bit table in shared memory
+//                       bit table in shared memory, buckets beyond their room
+//                       in tables of their distinct keys
 //   k_large_emit        running sums, the bars
 // Every step is exact for any input: partitions and buckets are counted before
 // they are filled, a list that overflows is not used, and ties are ordered by
 // (u, v) throughout, so the results equal the sorted path's bit for bit.
 //
 // Measured (device time, 1.25G edges of 50,021 points in the plane; the short
-// sort's path 67.4 ms): k_dist 5.9 ms, k_large_move<0> 7.0, the tree and its
-// pivots 1.2, the count 1.8, k_large_sub 1.4, k_large_move<1> 5.8,
-// k_large_repeats 5.2: 28.5 ms.  32,768 points of four circles in 16
+// sort's path 67.4 ms): k_dist 5.8 ms, k_large_move<0> 6.6, the tree and its
+// pivots 1.3, the count 1.9, k_large_sub 1.4, k_large_move<1> 5.8,
+// k_large_repeats 5.2: 28.1 ms.  32,768 points of four circles in 16
 // dimensions (537M edges): 26.4 ms (packed sort 34.4), of which the distances,
 // bound by the binary64 adder, 15.6.  The count, k_large_sub and the tree's
 // passes run near the copy bandwidth; the moves are bound by shared-memory
-// wavefronts (60 to 66% of the peak) and their barriers.
+// wavefronts (60 to 66% of the peak) and their barriers, with spills to local
+// memory on the same pipe: at the 32 registers that 2,048 threads per SM leave,
+// k_large_move<0> has a frame of 152 bytes and k_large_move<1> of 64, and a
+// warp issues 38 and 27 spill instructions for its 256 keys of a tile;
+// k_large_tree (64 registers) has a frame of 80 bytes.
 #include "ph0_common.cuh"
 
 namespace ph0 {
