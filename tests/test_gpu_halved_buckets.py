@@ -31,7 +31,7 @@ def _cases():
         "uniform_1500": inputs.uniform(1500, 3, seed=82),                          # buckets of 4,096 keys
         "uniform_2896": inputs.uniform(2896, 2, seed=83),                          # of 8,192
         "integers_2500": rng.integers(0, 100, (2500, 2)),                          # buckets beyond their room
-        "lattice_75": inputs.lattice(75, 2),                                       # few distances, large buckets
+        "lattice_60": inputs.lattice(60, 2),                                       # few distances, large buckets
         "bytes_6000": rng.integers(0, 256, (6000, 3)),
         "copies_5000": copies,
     }

@@ -3,6 +3,8 @@ a sort by default, and the distance kernel's settings on every form that takes
 them.  Every field of every bar against the oracle (integers and keys, so
 there is no tolerance), and the form that ran: 0 the short sort, 2 the
 complete sort after a fix-up met a group that it cannot order."""
+import functools
+
 import numpy as np
 import pytest
 
@@ -73,16 +75,25 @@ def test_settings_with_a_sort(split, tile, top):
     run(inputs.exponent_gaps(200, 4, seed=93), t, 2)  # rows whose distances agree in 36 bits
 
 
+@functools.lru_cache(maxsize=None)
+def _far(d):
+    x = inputs.uniform(2950 if d < 4 else 4400, d, seed=96 + d)
+    x[:, 0] += np.float32(1000.0)
+    return x, oracle.barcodes(x)
+
+
 @pytest.mark.parametrize("split,tile", [(0, 128), (5, 64), (16, 32), (11, 128), (8, 32), (16, 64)])
 @pytest.mark.parametrize("d", [2, 5, 33])
 def test_settings_without_a_sort(split, tile, d):
     """Above 2,896 points the form without a sort takes the distance kernel's
     settings; coordinates far from zero need more than 32 bits each, their
     differences fewer."""
-    n = 2950 if d < 4 else 4400
-    x = inputs.uniform(n, d, seed=96 + d)
-    x[:, 0] += np.float32(1000.0)
-    run(x, {"dist_split16": split, "dist_tile": tile}, 3)
+    from paper_2203_02527_gb300 import ph0
+    x, (want, inf_v, nd) = _far(d)
+    got = ph0.barcodes(torch.from_numpy(x).cuda(), tuning={"dist_split16": split, "dist_tile": tile})
+    assert got.stats["sort_form"] == 3
+    assert_bars_equal(got.numpy(), want)
+    assert got.inf[0] == inf_v and got.stats["n_distinct"] == nd
 
 
 def test_served_clouds_that_take_the_short_sort():
